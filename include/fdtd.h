@@ -202,7 +202,9 @@ fdtd_status fdtd_wall_coefficients(const fdtd_grid_desc* d, const fdtd_wall_desc
  * step n: H^{n+1/2} (with CPML psi) -> H soft source at (n+1/2) dt ->
  * fluence += |E^n x (H^{n-1/2}+H^{n+1/2})/2| dt at cell centres ->
  * E^{n+1} (with CPML psi) -> E soft source at (n+1) dt (Eq. 13) -> wall
- * source at (n+1) dt.  One or two kernel launches per step (tile variant).
+ * source at (n+1) dt.  One or two kernel launches per step (tile variant);
+ * an FP32 grid on its default tile takes pairs of steps in one launch (see
+ * fdtd_set_tile).
  * Small grids, whose passes take a few microseconds, are bound by the cost
  * of those launches; a batch of one grid (fdtd_batch_create with n = 1)
  * replays 64 steps from one CUDA graph instead, with the same results
@@ -250,27 +252,31 @@ int64_t fdtd_antenna_points(const fdtd_grid* g, int component);
  *   7  two steps per launch (temporal blocking; FP32 grids, ty 8 or 16,
  *      else EINVAL; lz 2 interleaves the window rows in the CTAs' work so
  *      that x-neighbouring windows march side by side, any other lz takes
- *      the windows row by row): windows of 32 x ty columns march along z,
- *      recomputing two rings of halo columns, so that fields, psi and the
- *      fluence cross HBM once per two steps.  An odd step count ends with
+ *      the windows row by row): windows of 32 x 24 columns (ty 16; 32 x 12
+ *      with ty 8) march along z, recomputing their halo columns, so that
+ *      fields, psi and the fluence cross HBM once per two steps.  An odd step count ends with
  *      one step of variant 5.  The CTAs' shares of the work are balanced on
  *      per-window costs (fdtd_set_balance).
  * The TMA variants (1, 2, 4) have no FP64 32x16 tile (EINVAL).  A z-walled
  * grid or one with a wall source takes variant 5 only (EINVAL otherwise;
  * fdtd_autotune then times the ty of variant 5 only).
- * fdtd_create_grid picks a default (variant 5, ty 4); fdtd_autotune times
+ * fdtd_create_grid picks a default (variant 5, ty 4).  As long as no tile is
+ * chosen, an FP32 grid (z-walled ones from 40 planes per cell of a z face's
+ * CPML on) takes its pairs of steps with the two-step kernel instead, which
+ * then rounds every operation as variant 5 does: the results are variant 5's,
+ * bit for bit.  fdtd_autotune times
  * the candidates on this grid (running `steps` steps for each, then
  * restoring the state) and keeps the fastest.  Results agree to rounding
  * for every configuration. */
 fdtd_status fdtd_set_tile(fdtd_grid* g, int variant, int ty, int lz);
 
 /* Work-split weights of tile variant 7 (the paper has no counterpart): a
- * window's plane is estimated to cost 1, plus w_shell if the window holds
- * CPML shell columns, plus w_antenna if it holds antenna columns, and each
- * CTA takes a contiguous range of (window, plane) work of equal estimated
- * cost; a window also costs three planes at its start (the two-step
- * wavefront refills there).  Weights in [0, 16] (else EINVAL); defaults 0.25
- * and 0.2.  fdtd_autotune times a few pairs, then refines the fastest pair's
+ * window's plane is estimated to cost 1, plus w_shell for a window that
+ * holds x shell or wall columns and for one that holds y ones (2.4 w_shell
+ * for both), plus w_antenna if it holds antenna columns, and each CTA takes a
+ * contiguous range of (window, plane) work of equal estimated cost; a window
+ * also costs some planes at its start (the two-step wavefront refills
+ * there).  Weights in [0, 16] (else EINVAL); defaults 0.4 and 0.15.  fdtd_autotune times a few pairs, then refines the fastest pair's
  * ranges on measured times (fdtd_measure_balance), with the windows row by
  * row and interleaved (lz 1 and 2), and times those; it keeps the fastest.
  * While refined ranges are in use, fdtd_get_balance returns -1 for both
@@ -392,7 +398,9 @@ fdtd_status fdtd_batch_set_engine(fdtd_batch* b, int engine);
 int fdtd_batch_get_engine(const fdtd_batch* b);
 /* Mode of grid q (0-based, creation order) in the graph engine; EINVAL for
  * an unknown mode or the two-step mode on a grid that cannot take it.  The
- * default is FDTD_BATCH_MODE_CELL4.  -1 from the getter for a bad index. */
+ * default is FDTD_BATCH_MODE_CELL4; as long as no mode is chosen (and the batch
+ * is not tuned), grids that would take the two-step kernel on their default
+ * tile (fdtd_set_tile) take it in the graph too, with the same results.  -1 from the getter for a bad index. */
 fdtd_status fdtd_batch_set_grid_mode(fdtd_batch* b, int q, int mode);
 int fdtd_batch_get_grid_mode(const fdtd_batch* b, int q);
 /* CTAs of grid q's two-step launches in the graph engine (-1 for a bad index). */

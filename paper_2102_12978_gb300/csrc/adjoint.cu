@@ -471,7 +471,7 @@ fdtd_status fdtd_adjoint_create(fdtd_grid* g, int component, const int64_t* prob
     if (!g || !arena || component < 0 || component > 2 || n_probes < 0 || (n_probes > 0 && !probe_cells))
         return fail(FDTD_EINVAL, "invalid adjoint arguments");
     if (reinterpret_cast<uintptr_t>(arena) % 256 != 0) return fail(FDTD_EINVAL, "arena not 256-byte aligned");
-    if (needs_cell_passes(g)) return fail(FDTD_EINVAL, "no adjoint for grids with z walls or a wall source");
+    if (has_walls(g)) return fail(FDTD_EINVAL, "no adjoint for grids with z walls or a wall source");
     if (!g->has_source) return fail(FDTD_ESTATE, "set the antenna source before creating its adjoint");
     const fdtd_status dev_st = check_device(g, "fdtd_adjoint_create");
     if (dev_st != FDTD_OK) return dev_st;

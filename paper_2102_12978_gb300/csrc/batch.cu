@@ -40,6 +40,7 @@
 #include "../../include/fdtd.h"
 #include "grid_impl.h"
 #include "yee_cell.cuh"
+#include "yee_tb2.cuh"
 
 namespace fdtd {
 
@@ -270,9 +271,12 @@ struct fdtd_batch {
     int nbranch;
     std::vector<unsigned char> host_times;
     std::vector<int> mode;           // graph engine: each grid's mode (kModeCell4 ... kModeTwoStep)
+    bool automatic;                  // nobody chose modes: grids take the two-step kernel where the default
+                                     // tile would (default_two_step), the results being the same
     std::vector<int> ctas;           // two-step mode: CTAs of the grid's launches
     bool shared_sms;                 // two-step launches on proportional shares of the SMs (else all)
-    int cur;
+    int cur;                         // copy parity of the grids (fdtd_grid::flip applied)
+    std::vector<int> pe, flip;       // the grids' copies that the graphs and launch parameters hold
     int64_t step;
     cudaGraphExec_t exec[2];         // graph engine, by read copy at the replay's start
     bool built[2];
@@ -309,8 +313,8 @@ cudaError_t cell_launch_grid(fdtd_batch* b, int q, int parity, int step, cudaStr
     const dim3 block(32, TY);
     constexpr int kMaxPlanes = 65535;   // gridDim.z limit: taller grids go in chunks of planes
     const int nz = g->desc.nz, nchunk = (nz + kMaxPlanes - 1) / kMaxPlanes;
-    StepArgs<real> a = make_args<real>(g, parity);
-    const bool wall = needs_cell_passes(g);   // z walls or a wall sheet
+    StepArgs<real> a = make_args<real>(g, parity ^ g->flip);
+    const bool wall = has_walls(g);   // z walls or a wall sheet
     for (int c = 0; c < nchunk; ++c) {
         a.kbase = c * kMaxPlanes;
         const dim3 grid((g->desc.nx + 31) / 32, (g->desc.ny + TY - 1) / TY,
@@ -347,11 +351,42 @@ cudaError_t cell_launch_grid_any(fdtd_batch* b, int q, int parity, int step, cud
     return cell_launch_grid<float, 4>(b, q, parity, step, s);
 }
 
-// One step of every grid on one stream (steps outside a graph replay).
-cudaError_t cell_launch_any(fdtd_batch* b, int parity, int step, cudaStream_t s)
+// Grid q's pairs of steps run on the two-step kernel.
+bool takes_two_step(const fdtd_batch* b, int q)
+{
+    if (b->automatic) return b->precision == FDTD_F32 && default_two_step(b->grids[size_t(q)]);
+    return b->mode[size_t(q)] == kModeTwoStep;
+}
+
+// An even number of two-step launches of grid q (the first steps of the time
+// table): copies and E-side psi flip once per launch and end as they were.
+cudaError_t two_step_launches(fdtd_batch* b, int q, int parity, int launches, int ctas, cudaStream_t s)
+{
+    const StepTime<float>* times =
+        reinterpret_cast<const StepTime<float>*>(static_cast<char*>(b->table) + b->times_off);
+    const int n = int(b->grids.size());
+    fdtd_grid* g = b->grids[size_t(q)];
+    const int pe0 = g->pe;
+    cudaError_t e = cudaSuccess;
+    for (int l = 0; l < launches && e == cudaSuccess; ++l) {
+        g->pe = pe0 ^ (l & 1);   // make_args picks the E-side psi copy of this launch
+        e = launch_tb2_table(g, parity ^ g->flip ^ (l & 1), times, 2 * l * n + q, (2 * l + 1) * n + q, ctas,
+                             b->automatic, s);
+    }
+    g->pe = pe0;
+    return e;
+}
+
+// `count` steps of every grid on one stream (steps that do not fill a graph
+// replay): where nobody chose modes, the two-step kernel in pairs of launches
+// on all SMs as far as they go, and the cell passes.
+cudaError_t remainder_steps(fdtd_batch* b, int parity, int count, cudaStream_t s)
 {
     for (int q = 0; q < int(b->grids.size()); ++q) {
-        cudaError_t e = cell_launch_grid_any(b, q, parity, step, s);
+        const int paired = b->automatic && takes_two_step(b, q) ? count / 4 * 4 : 0;
+        cudaError_t e = two_step_launches(b, q, parity, paired / 2, kTb2MaxCtas, s);
+        for (int st = paired; st < count && e == cudaSuccess; ++st)
+            e = cell_launch_grid_any(b, q, parity ^ (st & 1), st, s);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -362,21 +397,7 @@ cudaError_t cell_launch_any(fdtd_batch* b, int parity, int step, cudaStream_t s)
 // they were) or K single steps.
 cudaError_t graph_grid(fdtd_batch* b, int q, int parity, cudaStream_t s)
 {
-    if (b->mode[size_t(q)] == kModeTwoStep) {
-        const StepTime<float>* times =
-            reinterpret_cast<const StepTime<float>*>(static_cast<char*>(b->table) + b->times_off);
-        const int n = int(b->grids.size());
-        fdtd_grid* g = b->grids[size_t(q)];
-        const int pe0 = g->pe;
-        cudaError_t e = cudaSuccess;
-        for (int l = 0; l < kBatchGraphSteps / 2 && e == cudaSuccess; ++l) {
-            g->pe = pe0 ^ (l & 1);   // make_args picks the E-side psi copy of this launch
-            e = launch_tb2_table(g, parity ^ (l & 1), times, 2 * l * n + q, (2 * l + 1) * n + q,
-                                 b->ctas[size_t(q)], s);
-        }
-        g->pe = pe0;
-        return e;
-    }
+    if (takes_two_step(b, q)) return two_step_launches(b, q, parity, kBatchGraphSteps / 2, b->ctas[size_t(q)], s);
     for (int st = 0; st < kBatchGraphSteps; ++st) {
         cudaError_t e = cell_launch_grid_any(b, q, parity ^ (st & 1), st, s);
         if (e != cudaSuccess) return e;
@@ -408,12 +429,12 @@ fdtd_status pcell_fill(fdtd_batch* b)
         int blocks = 0;
         for (int q = 0; q < P.ngrids; ++q) {
             const fdtd_grid* g = b->grids[P.q0 + q];
-            for (int cur = 0; cur < 2; ++cur) P.args[q][cur] = make_args<real>(g, cur);
+            for (int cur = 0; cur < 2; ++cur) P.args[q][cur] = make_args<real>(g, cur ^ g->flip);
             P.ntx[q] = (g->desc.nx + 31) / 32;
             P.nty[q] = (g->desc.ny + kCellTY - 1) / kCellTY;
             P.nz[q] = g->desc.nz;
             P.block0[q] = blocks;
-            P.wall[q] = needs_cell_passes(g) ? 1 : 0;
+            P.wall[q] = has_walls(g) ? 1 : 0;
             blocks += P.ntx[q] * P.nty[q] * g->desc.nz;
         }
         P.block0[P.ngrids] = blocks;
@@ -530,7 +551,7 @@ void two_step_ctas(fdtd_batch* b, bool shared)
 
 bool two_step_eligible(const fdtd_batch* b, int q)
 {
-    return b->precision == FDTD_F32 && !needs_cell_passes(b->grids[size_t(q)]);
+    return b->precision == FDTD_F32 && !has_walls(b->grids[size_t(q)]);
 }
 
 }  // namespace
@@ -554,7 +575,8 @@ fdtd_status fdtd_batch_create(fdtd_grid* const* grids, int n, void* dev_table, s
     for (int q = 0; q < n; ++q) {
         if (!grids[q]) return fail(FDTD_EINVAL, "null grid %d", q);
         if (grids[q]->desc.precision != prec) return fail(FDTD_EINVAL, "mixed precisions in one batch");
-        if (grids[q]->cur != grids[0]->cur) return fail(FDTD_ESTATE, "grids must start from the same copy parity");
+        if ((grids[q]->cur ^ grids[q]->flip) != (grids[0]->cur ^ grids[0]->flip))
+            return fail(FDTD_ESTATE, "grids must start from the same copy parity");
         const fdtd_status dev_st = check_device(grids[q], "fdtd_batch_create");
         if (dev_st != FDTD_OK) return dev_st;
     }
@@ -567,13 +589,14 @@ fdtd_status fdtd_batch_create(fdtd_grid* const* grids, int n, void* dev_table, s
     b->table = dev_table;
     b->table_bytes = table_bytes;
     b->stream = static_cast<cudaStream_t>(stream);
-    b->cur = grids[0]->cur;
+    b->cur = grids[0]->cur ^ grids[0]->flip;
     b->step = 0;
     b->engine = FDTD_BATCH_CELL;
     b->times_off = times_offset();
     b->bar_off = bar_offset();
     b->fault = 0;
     b->mode.assign(size_t(n), kModeCell4);
+    b->automatic = true;
     two_step_ctas(b, true);
     b->built[0] = b->built[1] = false;
     fdtd_status st = cuda_check(cudaStreamCreateWithFlags(&b->capture, cudaStreamNonBlocking), "capture stream");
@@ -584,6 +607,12 @@ fdtd_status fdtd_batch_create(fdtd_grid* const* grids, int n, void* dev_table, s
     st = cuda_check(cudaStreamSynchronize(b->stream), "batch create");
     if (st == FDTD_OK) st = cuda_check(cudaMemcpy(b->table, &h, sizeof(h), cudaMemcpyHostToDevice), "batch table");
     if (st != FDTD_OK) { cudaStreamDestroy(b->capture); delete b; return st; }
+    b->pe.assign(size_t(n), 0);
+    b->flip.assign(size_t(n), 0);
+    for (int q = 0; q < n; ++q) {
+        b->pe[size_t(q)] = grids[q]->pe;
+        b->flip[size_t(q)] = grids[q]->flip;
+    }
     cell_fill(b);
     st = prec == FDTD_F64 ? pcell_fill<double>(b) : pcell_fill<float>(b);
     if (st != FDTD_OK) { cudaStreamDestroy(b->capture); delete b; return st; }
@@ -623,8 +652,9 @@ fdtd_status fdtd_batch_set_grid_mode(fdtd_batch* b, int q, int mode)
         return fail(FDTD_EINVAL, "mode %d is not a batch grid mode", mode);
     if (mode == FDTD_BATCH_MODE_TWO_STEP && !two_step_eligible(b, q))
         return fail(FDTD_EINVAL, "the two-step mode takes FP32 z-periodic grids without a wall source");
-    if (b->mode[size_t(q)] != mode) {
+    if (b->mode[size_t(q)] != mode || b->automatic) {
         b->mode[size_t(q)] = mode;
+        b->automatic = false;
         drop_graphs(b);
     }
     return FDTD_OK;
@@ -669,7 +699,23 @@ static fdtd_status batch_step_ranges(fdtd_batch* b, int nsteps)
     const fdtd_status dev_st = check_device(b->grids[0], "fdtd_batch_step");
     if (dev_st != FDTD_OK) return dev_st;
     for (fdtd_grid* g : b->grids)
-        if (g->cur != b->cur) return fail(FDTD_ESTATE, "a batched grid was stepped outside the batch");
+        if ((g->cur ^ g->flip) != b->cur) return fail(FDTD_ESTATE, "a batched grid was stepped outside the batch");
+    // a state loaded into a batched grid may hold its fields or its E-side psi
+    // in the other copy: the graphs and launch parameters are made again for it
+    bool same = true;
+    for (size_t q = 0; q < b->grids.size(); ++q)
+        same = same && b->pe[q] == b->grids[q]->pe && b->flip[q] == b->grids[q]->flip;
+    if (!same) {
+        for (size_t q = 0; q < b->grids.size(); ++q) {
+            b->pe[q] = b->grids[q]->pe;
+            b->flip[q] = b->grids[q]->flip;
+        }
+        const fdtd_status fill_st = cuda_check(cudaStreamSynchronize(b->stream), "batch parameters");
+        if (fill_st != FDTD_OK) return fill_st;
+        drop_graphs(b);
+        const fdtd_status pst = b->precision == FDTD_F64 ? pcell_fill<double>(b) : pcell_fill<float>(b);
+        if (pst != FDTD_OK) return pst;
+    }
     int done = 0;
     while (done < nsteps) {
         const int count = nsteps - done < kBatchGraphSteps ? nsteps - done : kBatchGraphSteps;
@@ -696,17 +742,15 @@ static fdtd_status batch_step_ranges(fdtd_batch* b, int nsteps)
             st = cuda_check(cudaGraphLaunch(b->exec[b->cur], b->stream), "graph launch");
             if (st != FDTD_OK) return st;
         } else {
-            for (int s = 0; s < count; ++s) {
-                cudaError_t e = cell_launch_any(b, b->cur ^ (s & 1), s, b->stream);
-                if (e != cudaSuccess) return cuda_check(e, "batch launch");
-            }
+            const cudaError_t e = remainder_steps(b, b->cur, count, b->stream);
+            if (e != cudaSuccess) return cuda_check(e, "batch launch");
             b->cur ^= (count & 1);
         }
         done += count;
         b->step += count;
         for (fdtd_grid* g : b->grids) {
             g->step += count;
-            g->cur = b->cur;
+            g->cur = b->cur ^ g->flip;
         }
     }
     return FDTD_OK;
@@ -811,6 +855,7 @@ fdtd_status fdtd_batch_autotune(fdtd_batch* b, int steps, void* scratch, size_t 
         for (int m = kModeCell4; m <= kModeCell16 && err == cudaSuccess; ++m) {
             TileConfig tc = keep;
             tc.variant = 5;
+            tc.automatic = false;
             tc.ty = m == kModeCell8 ? 8 : (m == kModeCell16 ? 16 : 4);
             g->tile = tc;
             if (fdtd_step(g, 2) != FDTD_OK) err = cudaErrorUnknown;   // warm-up
@@ -860,6 +905,7 @@ fdtd_status fdtd_batch_autotune(fdtd_batch* b, int steps, void* scratch, size_t 
         return st == FDTD_OK;
     };
     const int keep_engine = b->engine;
+    b->automatic = false;
     float best_t = 1e30f;
     long long best_thr = -1;
     bool best_shared = true;

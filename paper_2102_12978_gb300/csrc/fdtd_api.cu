@@ -83,7 +83,8 @@ bool compute_layout(const fdtd_grid_desc& d, Layout& L)
     L.psz_elems = w2z * ny * p;
     for (int buf = 0; buf < 2; ++buf)
         for (int c = 0; c < 2; ++c) L.phz[buf][c] = take(L.psz_elems * b);
-    for (int c = 0; c < 2; ++c) L.pez[c] = take(L.psz_elems * b);
+    for (int buf = 0; buf < 2; ++buf)
+        for (int c = 0; c < 2; ++c) L.pez[buf][c] = take(L.psz_elems * b);
     L.fluence = d.fluence ? take(nz * ny * p * 8) : 0;
     L.dynamic_bytes = off;
     L.chx = take(nx * b); L.cex = take(nx * b);
@@ -274,7 +275,8 @@ StepArgs<real> make_args(const fdtd_grid* g, int cur)
     for (int c = 0; c < 2; ++c) {
         a.phz_in[c] = reinterpret_cast<const real*>(A + L.phz[cur][c]);
         a.phz_out[c] = reinterpret_cast<real*>(A + L.phz[nxt][c]);
-        a.pez[c] = reinterpret_cast<real*>(A + L.pez[c]);
+        a.pez[c] = reinterpret_cast<real*>(A + L.pez[g->pe][c]);
+        a.pez_out[c] = reinterpret_cast<real*>(A + L.pez[g->pe ^ 1][c]);
     }
     a.chz = reinterpret_cast<const real*>(A + L.chz);
     a.cez = reinterpret_cast<const real*>(A + L.cez);
@@ -337,7 +339,7 @@ static cudaError_t launch_tma(const fdtd_grid* cg, int cur, long long n, int lz,
 cudaError_t launch_step(const fdtd_grid* g, int cur, long long n, const TileConfig& tc, cudaStream_t s,
                         cudaEvent_t mid)
 {
-    if (tc.variant != 5 && needs_cell_passes(g)) return cudaErrorInvalidValue;   // z walls / wall source
+    if (tc.variant != 5 && has_walls(g)) return cudaErrorInvalidValue;   // z walls / wall source
     if (tc.variant == 7) return cudaErrorInvalidValue;   // two steps per launch: launch_tb2
     if (tc.variant >= 3) return launch_split(g, cur, n, tc, s, mid);   // variants 3-6
     if (tc.variant == 1) {
@@ -391,6 +393,7 @@ TileConfig default_tile(const fdtd_grid_desc& d, int sm_count)
     (void)sm_count;
     TileConfig tc;
     tc.variant = 5; tc.tx = 32; tc.ty = 4; tc.lz = d.nz;
+    tc.automatic = true;
     return tc;
 }
 
@@ -445,6 +448,7 @@ fdtd_status fdtd_create_grid(const fdtd_grid_desc* d, void* arena, size_t arena_
     g->step = 0;
     g->cur = 0;
     g->pe = 0;
+    g->flip = 0;
     g->has_source = false;
     g->src_gen = 0;
     g->tb2_key.ry = 0;
@@ -475,6 +479,8 @@ fdtd_status fdtd_create_grid(const fdtd_grid_desc* d, void* arena, size_t arena_
     g->tile = default_tile(*d, sms);
     for (int a = 0; a < 2; ++a)
         for (int b = 0; b < 3; ++b) g->maps_ok[a][b] = g->hmaps_ok[a][b] = false;
+    for (int a = 0; a < 2; ++a)
+        for (int b = 0; b < 2; ++b) g->tb2maps_ok[a][b] = false;
     st = cuda_check(cudaMemsetAsync(arena, 0, L.total, g->stream), "zero arena");
     if (st == FDTD_OK)
         st = (d->precision == FDTD_F64) ? upload_tables<double>(g) : upload_tables<float>(g);
@@ -719,12 +725,18 @@ fdtd_status fdtd_clear_source(fdtd_grid* g)
 static cudaError_t run_steps(fdtd_grid* g, int nsteps, const TileConfig& tc)
 {
     int s = 0;
-    if (tc.variant == 7)
+    TileConfig two = tc;
+    if (tc.automatic && default_two_step(g)) {   // the default tile
+        two.variant = 7;
+        two.ty = 16;
+    }
+    if (two.variant == 7)
         for (; s + 2 <= nsteps; s += 2) {
-            cudaError_t e = launch_tb2(g, g->cur, g->step, tc, g->stream);
+            cudaError_t e = launch_tb2(g, g->cur, g->step, two, g->stream);
             if (e != cudaSuccess) return e;
             g->cur ^= 1;
             g->pe ^= 1;
+            if (tc.automatic) g->flip ^= 1;
             g->step += 2;
         }
     const TileConfig one = single_step_tile(tc);
@@ -973,7 +985,7 @@ fdtd_status fdtd_save_state(fdtd_grid* g, void* dev_dst)
     if (!g || !dev_dst) return fail(FDTD_EINVAL, "null argument");
     const fdtd_status dev_st = check_device(g, "fdtd_save_state");
     if (dev_st != FDTD_OK) return dev_st;
-    int64_t hdr[4] = {g->step, g->cur, 0x46445444, g->pe};
+    int64_t hdr[5] = {g->step, g->cur, 0x46445444, g->pe, g->flip};
     char* D = static_cast<char*>(dev_dst);
     fdtd_status st = cuda_check(cudaMemcpyAsync(D, g->arena, g->L.dynamic_bytes, cudaMemcpyDeviceToDevice,
                                                 g->stream), "save state");
@@ -989,13 +1001,14 @@ fdtd_status fdtd_load_state(fdtd_grid* g, const void* dev_src)
     if (!g || !dev_src) return fail(FDTD_EINVAL, "null argument");
     const fdtd_status dev_st = check_device(g, "fdtd_load_state");
     if (dev_st != FDTD_OK) return dev_st;
-    int64_t hdr[4];
+    int64_t hdr[5];
     const char* S = static_cast<const char*>(dev_src);
     fdtd_status st = cuda_check(cudaMemcpyAsync(hdr, S + g->L.dynamic_bytes, sizeof(hdr), cudaMemcpyDeviceToHost,
                                                 g->stream), "load state");
     if (st == FDTD_OK) st = fdtd_sync(g);
     if (st != FDTD_OK) return st;
-    if (hdr[2] != 0x46445444 || (hdr[1] != 0 && hdr[1] != 1) || (hdr[3] != 0 && hdr[3] != 1))
+    if (hdr[2] != 0x46445444 || (hdr[1] != 0 && hdr[1] != 1) || (hdr[3] != 0 && hdr[3] != 1) ||
+        (hdr[4] != 0 && hdr[4] != 1))
         return fail(FDTD_EINVAL, "state blob does not come from fdtd_save_state");
     st = cuda_check(cudaMemcpyAsync(g->arena, S, g->L.dynamic_bytes, cudaMemcpyDeviceToDevice, g->stream),
                     "load state");
@@ -1003,6 +1016,7 @@ fdtd_status fdtd_load_state(fdtd_grid* g, const void* dev_src)
     g->step = hdr[0];
     g->cur = int(hdr[1]);
     g->pe = int(hdr[3]);
+    g->flip = int(hdr[4]);
     return fdtd_sync(g);
 }
 
@@ -1033,11 +1047,12 @@ fdtd_status fdtd_set_tile(fdtd_grid* g, int variant, int ty, int lz)
     if (variant == 7 && (ty == 4 || g->desc.precision != FDTD_F32))
         return fail(FDTD_EINVAL, "variant 7 takes FP32 grids and ty 8 or 16");
     if (variant == 6 && g->desc.nz > 65535) return fail(FDTD_EINVAL, "variant 6 takes nz <= 65535");
-    if (variant != 5 && needs_cell_passes(g))
+    if (variant != 5 && has_walls(g))
         return fail(FDTD_EINVAL, "a grid with z walls or a wall source takes tile variant 5");
     if ((variant == 1 || variant == 2 || variant == 4) && ty == 16 && g->desc.precision == FDTD_F64)
         return fail(FDTD_EINVAL, "the TMA variants have no FP64 32x16 tile");
     if (lz < 1) return fail(FDTD_EINVAL, "lz=%d < 1", lz);
+    g->tile.automatic = false;
     g->tile.variant = variant;
     g->tile.tx = 32;
     g->tile.ty = ty;
@@ -1096,7 +1111,7 @@ fdtd_status fdtd_autotune(fdtd_grid* g, int steps, void* scratch_state)
         cands.insert(cands.begin(), {{7, 16, 0.0f, 0.0f}, {7, 16, 0.15f, 0.1f}, {7, 16, 0.3f, 0.2f},
                                      {7, 16, 0.45f, 0.3f}, {7, 16, 0.3f, 0.4f}, {7, 16, 0.6f, 0.4f},
                                      {7, 8, 0.3f, 0.2f}});
-    if (needs_cell_passes(g)) cands = {{5, 4}, {5, 8}, {5, 16}};
+    if (has_walls(g)) cands = {{5, 4}, {5, 8}, {5, 16}};
     const int nz = g->desc.nz;
     std::vector<int> lzs;
     for (int segs : {1, 2, 3, 4, 6, 8, 12, 16}) {

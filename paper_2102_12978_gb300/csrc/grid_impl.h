@@ -21,7 +21,7 @@ struct Layout {
     size_t phx[2][2] = {}, phy[2][2] = {};
     size_t pex[2][2] = {}, pey[2][2] = {};   // [copy][component]: E psi, updated in place except by variant 7
     size_t psz_elems = 0;                 // z shell psi of z-walled grids: [2 npml_z][ny][pitch]
-    size_t phz[2][2] = {}, pez[2] = {};   // Hxz, Hyz (ping-pong); Exz, Eyz (in place)
+    size_t phz[2][2] = {}, pez[2][2] = {};   // Hxz, Hyz; Exz, Eyz: [copy][component], as phx and pex
     size_t fluence = 0;
     size_t dynamic_bytes = 0;
     size_t chx = 0, cex = 0, chy = 0, cey = 0, chz = 0, cez = 0;
@@ -51,10 +51,13 @@ struct TileConfig {
     // variant 7: extra cost per plane of a window holding CPML shell / antenna
     // columns, relative to a plain window (the CTAs' work ranges are balanced
     // on these estimates)
-    float w_shell = 0.25f, w_ant = 0.2f;
+    float w_shell = 0.4f, w_ant = 0.15f;
     // variant 7: run the ranges refined from measured per-CTA times
     // (fdtd_grid::tb2_refined) instead of those of the weights above
     bool measured = false;
+    // the default tile, chosen by nobody: runs of steps take the two-step
+    // kernel where it is the faster one (default_two_step)
+    bool automatic = false;
 };
 
 fdtd_status fail(fdtd_status st, const char* fmt, ...);
@@ -83,6 +86,9 @@ struct fdtd_grid {
     double dt;
     int64_t step;
     int cur;                 // which ping-pong copy holds the current state
+    int flip;                // cur ^ flip is the copy parity that a batch compares its grids by: the one
+                             // single steps would have left (a two-step launch of the default tile
+                             // changes copy once for two steps, and flips this)
     int pe;                  // which copy of the E-side psi is current (flipped by variant 7)
     bool has_source;
     fdtd_annulus_desc src;
@@ -95,6 +101,8 @@ struct fdtd_grid {
     bool maps_ok[2][3];
     fdtd::TmaMaps hmaps[2][3];  // the same for the boxes of yee_hflu_tma
     bool hmaps_ok[2][3];
+    fdtd::TmaMaps tb2maps[2][2];   // [read copy][window height] of the two-step kernel
+    bool tb2maps_ok[2][2];
     int fault;                  // fdtd_debug_inject_fault: applies to the next step only
     int batch_refs;             // batches holding this grid (their kernels hold copies of its arguments)
     bool has_wall;              // fdtd_set_wall_source
@@ -126,9 +134,9 @@ StepArgs<real> make_args(const fdtd_grid* g, int cur);
 // kernels of a two-pass variant (ignored by the one-pass variants).
 cudaError_t launch_step(const fdtd_grid* g, int cur, long long n, const TileConfig& tc, cudaStream_t s,
                         cudaEvent_t mid = nullptr);
-// True if the grid needs the cell passes of tile variant 5 (z walls or a
-// wall source: the other variants implement z-periodic grids only).
-inline bool needs_cell_passes(const fdtd_grid* g)
+// True if the grid has z walls or a wall source (tile variants 0-4 and 6
+// implement z-periodic grids without a sheet only).
+inline bool has_walls(const fdtd_grid* g)
 {
     return g->desc.z_boundary == FDTD_Z_WALLS || g->has_wall;
 }
@@ -136,8 +144,8 @@ inline bool needs_cell_passes(const fdtd_grid* g)
 // once per two steps).
 inline int passes_per_step(const TileConfig& tc) { return tc.variant >= 3 && tc.variant <= 5 ? 2 : 1; }
 // Tile variant 7: two steps n, n+1 from copy `cur` (fields, H psi) and E psi
-// copy g->pe into the other copies.  FP32, z-periodic grids without a wall
-// source only.
+// copy g->pe into the other copies.  FP32 only; with tc.automatic (the default
+// tile) also z walls and wall sheets, and the cell passes' roundings.
 cudaError_t launch_tb2(const fdtd_grid* g, int cur, long long n, const TileConfig& tc, cudaStream_t s);
 // Windows of variant 7 with 32 x ry columns on grid d: t along x, u along y.
 void tb2_windows(const fdtd_grid_desc& d, int ry, int* t, int* u);
@@ -155,9 +163,14 @@ std::vector<long long> tb2_refined_ranges(const std::vector<long long>& s, const
 int tb2_slots(const fdtd_grid* g, int ry);
 // The same two steps with their time factors from a device table of
 // StepTime<float> (entries i0, i1), on at most max_ctas CTAs (a batch runs
-// several grids side by side): the batched graph's launch.
+// several grids side by side): the batched graph's launch.  automatic: with
+// the cell passes' roundings (nobody chose the two-step mode).
 cudaError_t launch_tb2_table(const fdtd_grid* g, int cur, const StepTime<float>* times, int i0, int i1,
-                             int max_ctas, cudaStream_t s);
+                             int max_ctas, bool automatic, cudaStream_t s);
+// True if a run of steps on the grid's default tile takes the two-step kernel
+// for its pairs of steps (the results are those of the cell passes, bit for
+// bit).
+bool default_two_step(const fdtd_grid* g);
 // The tile of the single step that completes an odd step count of variant 7.
 inline TileConfig single_step_tile(const TileConfig& tc)
 {

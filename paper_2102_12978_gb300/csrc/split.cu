@@ -141,7 +141,7 @@ static cudaError_t launch_cell(const fdtd_grid* g, int cur, long long n, cudaStr
     const StepTime<real> t = step_time<real>(g->srct, g->has_wall ? &g->wallt : nullptr, g->dt, n);
     const int nz = g->desc.nz, nchunk = (nz + kMaxPlanes - 1) / kMaxPlanes;
     dim3 block(32, TY);
-    const bool wall = needs_cell_passes(g);   // z walls or a wall sheet: the *_w kernels
+    const bool wall = has_walls(g);   // z walls or a wall sheet: the *_w kernels
     const bool apart = sizeof(real) == 8 && g->has_source && g->ant_apart && !wall;
     const StepArgs<real> full = make_args<real>(g, cur);
     StepArgs<real> a = full;

@@ -5,17 +5,22 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 
 #include "grid_impl.h"
+#include "tma_host.h"
 #include "yee_tb2.cuh"
 
 namespace fdtd {
 
+// Window rows of the kernel that serves tile height ty.
+static int tb2_rows(int ty) { return ty == 8 ? kTb2RowsSmall : kTb2Rows; }
+
 void tb2_windows(const fdtd_grid_desc& d, int ry, int* t, int* u)
 {
-    *t = d.nx <= kTb2Wx ? 1 : (d.nx - kTb2Wx + kTb2Sx - 1) / kTb2Sx + 1;
-    *u = d.ny <= ry ? 1 : (d.ny - ry + (ry - 4) - 1) / (ry - 4) + 1;
+    *t = (d.nx + kTb2Sx - 1) / kTb2Sx;
+    *u = (d.ny + ry - 5) / (ry - 4);
 }
 
 std::vector<long long> tb2_refined_ranges(const std::vector<long long>& s, const unsigned long long* cycles,
@@ -49,8 +54,9 @@ std::vector<long long> tb2_refined_ranges(const std::vector<long long>& s, const
     return ns;
 }
 
-void tb2_refine(fdtd_grid* g, int ry, int slots, const unsigned long long* cycles, double step)
+void tb2_refine(fdtd_grid* g, int ty, int slots, const unsigned long long* cycles, double step)
 {
+    const int ry = tb2_rows(ty);
     // the ranges the measured launches ran: the cached plan of this shape
     if (g->tb2_key.ry != ry || g->tb2_key.slots != slots || g->tb2_start.size() != size_t(slots) + 1) return;
     g->tb2_refined = tb2_refined_ranges(g->tb2_start, cycles, step);
@@ -91,18 +97,33 @@ static int tb2_window_host(int T, int U, int D, int pos)
 // CTA work ranges of variant 7 on grid g: windows of 32 x RY columns, `slots`
 // resident CTAs.  Each CTA gets a contiguous range of (window, plane) items.
 // The ranges either have equal estimated cost -- a window-plane costs 1,
-// plus w_shell if the window holds CPML shell columns, plus w_ant if it holds
-// antenna columns, and a window costs kRestart more planes at its start (the
-// wavefront refills) -- or (tc.measured) are the ones tb2_refine moved until
+// plus w_shell for each of the x and y shell or wall codes the window runs and
+// kCorner w_shell more for both, plus w_ant if it holds antenna columns,
+// kZPlane times that in the z shells, and a window costs kRestart more planes
+// at its start (the wavefront refills: four planes and the first loads'
+// latency) -- or (tc.measured) are the ones tb2_refine moved until
 // the CTAs' measured times were equal.  Cached on the grid until the antenna,
 // the weights or the launch shape change.
-constexpr double kRestart = 3.0;
+// Measured on GB300 (cycles per plane, 256 x 256 x 128 cells): inner windows
+// 2400, with antenna columns 2750, x shell 3340, y shell 3380, both 4720; the
+// default weights 0.4 and 0.15 follow.
+constexpr double kRestart = 5.3;
+constexpr double kCorner = 0.4;
+constexpr double kZPlane = 1.6;
+// A z-walled grid takes the two-step kernel from this many planes per CPML
+// cell of a z face on: a z-shell plane costs it about four inner ones, so
+// that short boxes run faster on the cell passes (411 x 411 cells, 16-cell z
+// CPML, us per step on both: 200 planes 743 / 712, 400 planes 1283 / 1376, 738
+// planes 2184 / 2486; without a z CPML, 200 planes, 480 / 686).
+constexpr int kShellPlanes = 40;
 static void tb2_plan(fdtd_grid* g, int RY, int slots, const TileConfig& tc, Tb2Plan& P)
 {
     const fdtd_grid_desc& d = g->desc;
     tb2_windows(d, RY, &P.T, &P.U);
     P.prof = nullptr;
-    const int order = tc.lz == 2 ? 2 : 1;
+    P.dt16 = float(g->dt * 0.0625);
+    P.err = reinterpret_cast<int*>(static_cast<char*>(g->arena) + g->L.err);
+    const int order = tc.lz == 2 && !tc.automatic ? 2 : 1;
     P.D = tb2_order_d(P.T, P.U, d.nz, slots, order);
     const bool meas = tc.measured && g->tb2_ref_ry == RY && g->tb2_ref_slots == slots &&
                       g->tb2_ref_src == g->src_gen && g->tb2_refined.size() == size_t(slots) + 1 &&
@@ -119,22 +140,31 @@ static void tb2_plan(fdtd_grid* g, int RY, int slots, const TileConfig& tc, Tb2P
             std::vector<double> cost(size_t(nw), 1.0);
             for (int wy = 0; wy < P.U; ++wy)
                 for (int wx = 0; wx < P.T; ++wx) {
-                    const int i0 = kTb2Sx * wx, i1 = std::min(i0 + kTb2Wx, nx);
-                    const int j0 = (RY - 4) * wy, j1 = std::min(j0 + RY, ny);
-                    const bool shell = npml > 0 && (i0 < npml || i1 > nx - npml || j0 < npml || j1 > ny - npml);
+                    const int L0 = kTb2Sx * wx - kTb2Ox, M0 = (RY - 4) * wy - kTb2Oy;
+                    const int i0 = std::max(L0, 0), i1 = std::min(L0 + kTb2Wx, nx);
+                    const int j0 = std::max(M0, 0), j1 = std::min(M0 + RY, ny);
+                    // windows that run the x (y) shell and wall code
+                    const int sx = wx == 0 || wx == P.T - 1 || (npml > 0 && (L0 < npml || L0 + kTb2Wx > nx - npml));
+                    const int sy = wy == 0 || wy == P.U - 1 || (npml > 0 && (M0 < npml || M0 + RY > ny - npml));
                     bool ant = false;
                     if (!g->hmask.empty())
                         for (int j = j0; j < j1 && !ant; ++j)
                             for (int i = i0; i < i1 && !ant; ++i) ant = g->hmask[size_t(j) * nx + i] != 0;
-                    cost[size_t(wy) * P.T + wx] = 1.0 + (shell ? tc.w_shell : 0.0) + (ant ? tc.w_ant : 0.0);
+                    cost[size_t(wy) * P.T + wx] = 1.0 + (sx + sy + kCorner * sx * sy) * tc.w_shell + (ant ? tc.w_ant : 0.0);
                 }
+            // planes of the z shells cost kZPlane times a plain one
+            std::vector<double> zc(size_t(nz) + 1, 0.0);   // cost of the planes [0, k)
+            const bool zw = d.z_boundary == FDTD_Z_WALLS;
+            const int pz = zw ? d.npml_z : 0;
+            for (int k = 0; k < nz; ++k) zc[size_t(k) + 1] = zc[size_t(k)] + (k < pz || k >= nz - pz ? kZPlane : 1.0);
+            const double zsum = zc[size_t(nz)];
             if (P.D > 1) {   // costs by position
                 std::vector<double> byp(cost.size());
                 for (int m = 0; m < nw; ++m) byp[size_t(m)] = cost[size_t(tb2_window_host(P.T, P.U, P.D, m))];
                 cost.swap(byp);
             }
             double total = 0.0;
-            for (double c : cost) total += c * (nz + kRestart);
+            for (double c : cost) total += c * (zsum + kRestart);
             const double share = total / slots;
             std::vector<long long> start(size_t(slots) + 1, (long long)nw * nz);
             start[0] = 0;
@@ -142,9 +172,10 @@ static void tb2_plan(fdtd_grid* g, int RY, int slots, const TileConfig& tc, Tb2P
             double cum = 0.0;
             for (int w = 0; w < nw && c < slots; ++w) {
                 const double cw = cost[size_t(w)];
-                const double span = cw * (nz + kRestart), base = cum + cw * kRestart;
+                const double span = cw * (zsum + kRestart), base = cum + cw * kRestart;
                 while (c < slots && c * share < cum + span) {
-                    long long k = (long long)std::ceil((c * share - base) / cw);
+                    // the first plane whose cost from the window's start reaches the share
+                    long long k = std::lower_bound(zc.begin(), zc.end(), (c * share - base) / cw) - zc.begin();
                     k = std::max(0LL, std::min((long long)nz, k));
                     start[size_t(c)] = std::max(start[size_t(c) - 1], (long long)w * nz + k);
                     ++c;
@@ -167,30 +198,71 @@ static cudaError_t tb2_blocks_per_sm(int* out)
 {
     using S = Tb2Smem<RY>;
     static_assert(S::bytes() <= 232448, "the window's shared memory exceeds the 227 KB a CTA can hold");
-    static int blocks_per_sm = 0;
-    if (blocks_per_sm == 0) {
-        cudaError_t e = cudaFuncSetAttribute(yee_tb2<RY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             int(S::bytes()));
-
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(yee_tb2_t<RY>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(S::bytes()));
+    static std::atomic<int> blocks_per_sm{0};
+    if (blocks_per_sm.load() == 0) {
+        const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+        const int bytes = int(S::bytes());
+        cudaError_t e = cudaFuncSetAttribute(yee_tb2<RY, false, false>, at, bytes);
+        if constexpr (RY == kTb2Rows) {
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(yee_tb2<RY, false, true>, at, bytes);
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(yee_tb2<RY, true, true>, at, bytes);
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(yee_tb2_t<RY, false, false>, at, bytes);
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(yee_tb2_t<RY, false, true>, at, bytes);
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(yee_tb2_t<RY, true, true>, at, bytes);
+        }
         if (e != cudaSuccess) return e;
         int n = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, yee_tb2<RY>, 32 * RY, S::bytes());
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, yee_tb2<RY, false, false>, S::NT, S::bytes());
         if (e != cudaSuccess) return e;
         if (n < 1) return cudaErrorInvalidConfiguration;
-        blocks_per_sm = n;
+        blocks_per_sm.store(n);
     }
-    *out = blocks_per_sm;
+    *out = blocks_per_sm.load();
     return cudaSuccess;
 }
 
-int tb2_slots(const fdtd_grid* g, int ry)
+// Every FP32 box but short z-walled ones: the two-step kernel is the faster
+// one, or as fast, at every size measured (us per step, two-step / cell passes:
+// 16 x 16 x 8 7.2 / 8.2; 48 x 40 x 16 8.2 / 9.1; 64 x 64 x 32 10.3 / 10.3;
+// 96 x 96 x 64 15 / 18; 160 x 160 x 64 27 / 41; 332 x 332 x 46 66 / 111;
+// 640 x 640 x 64 352 / 514; 560 x 560 x 5 36 / 36).
+bool default_two_step(const fdtd_grid* g)
+{
+    const fdtd_grid_desc& d = g->desc;
+    if (d.precision != FDTD_F32) return false;
+    return d.z_boundary != FDTD_Z_WALLS || d.nz >= kShellPlanes * d.npml_z;
+}
+
+int tb2_slots(const fdtd_grid* g, int ty)
 {
     int per_sm = 0;
-    const cudaError_t e = ry == 8 ? tb2_blocks_per_sm<8>(&per_sm) : tb2_blocks_per_sm<16>(&per_sm);
+    const cudaError_t e = ty == 8 ? tb2_blocks_per_sm<kTb2RowsSmall>(&per_sm) : tb2_blocks_per_sm<kTb2Rows>(&per_sm);
     if (e != cudaSuccess) return -1;
     return std::min(kTb2MaxCtas, (g->sm_count > 0 ? g->sm_count : 152) * per_sm);
+}
+
+// Tensor maps of the fields of copy `cur` and of the fluence accumulator, in
+// boxes of one window (32 x RY columns of one plane).
+template <int RY>
+static bool tb2_maps(fdtd_grid* g, int cur, TmaMaps** out)
+{
+    const int sl = RY == kTb2RowsSmall ? 0 : 1;
+    TmaMaps& m = g->tb2maps[cur][sl];
+    if (!g->tb2maps_ok[cur][sl]) {
+        char* A = static_cast<char*>(g->arena);
+        bool ok = true;
+        for (int c = 0; c < 3; ++c) {
+            ok = ok && encode_map(&m.e[c], A + g->L.field[cur][c], 4, g->desc, g->L.pitch, kTb2Wx, RY, CU_TENSOR_MAP_L2_PROMOTION_L2_64B);
+            ok = ok && encode_map(&m.h[c], A + g->L.field[cur][3 + c], 4, g->desc, g->L.pitch, kTb2Wx, RY, CU_TENSOR_MAP_L2_PROMOTION_L2_64B);
+        }
+        void* f = g->desc.fluence ? A + g->L.fluence : A + g->L.field[cur][0];   // unused without a fluence
+        if (g->desc.fluence) ok = ok && encode_map(&m.f, f, 8, g->desc, g->L.pitch, kTb2Wx, RY, CU_TENSOR_MAP_L2_PROMOTION_L2_64B);
+        else m.f = m.e[0];
+        if (!ok) return false;
+        g->tb2maps_ok[cur][sl] = true;
+    }
+    *out = &m;
+    return true;
 }
 
 template <int RY>
@@ -206,27 +278,40 @@ static cudaError_t launch_tb2_t(const fdtd_grid* cg, int cur, long long n, const
     tb2_plan(g, RY, slots, tc, plan);
     if (g->tb2_profile)
         plan.prof = reinterpret_cast<unsigned long long*>(static_cast<char*>(g->arena) + g->L.tb2prof);
-    const StepTime<float> t0 = step_time<float>(g->srct, nullptr, g->dt, n);
-    const StepTime<float> t1 = step_time<float>(g->srct, nullptr, g->dt, n + 1);
+    const SrcTime* wall = g->has_wall ? &g->wallt : nullptr;
+    const StepTime<float> t0 = step_time<float>(g->srct, wall, g->dt, n);
+    const StepTime<float> t1 = step_time<float>(g->srct, wall, g->dt, n + 1);
     Tb2Times tt;
-    tt.th0 = t0.th; tt.te0 = t0.te; tt.th1 = t1.th; tt.te1 = t1.te;
-    yee_tb2<RY><<<unsigned(slots), dim3(32, RY), S::bytes(), s>>>(make_args<float>(g, cur), tt, plan);
+    tt.th0 = t0.th; tt.te0 = t0.te; tt.tw0 = t0.tw;
+    tt.th1 = t1.th; tt.te1 = t1.te; tt.tw1 = t1.tw;
+    TmaMaps* m = nullptr;
+    if (!tb2_maps<RY>(g, cur, &m)) return cudaErrorInvalidValue;
+    const StepArgs<float> a = make_args<float>(g, cur);
+    const unsigned ctas = unsigned(slots);
+    if constexpr (RY == kTb2Rows) {
+        if (tc.automatic) {   // runs on the default tile: the cell passes' roundings
+            if (has_walls(g)) yee_tb2<RY, true, true><<<ctas, S::NT, S::bytes(), s>>>(a, tt, *m, plan);
+            else yee_tb2<RY, false, true><<<ctas, S::NT, S::bytes(), s>>>(a, tt, *m, plan);
+            return cudaGetLastError();
+        }
+    }
+    yee_tb2<RY, false, false><<<ctas, S::NT, S::bytes(), s>>>(a, tt, *m, plan);
     return cudaGetLastError();
 }
 
 cudaError_t launch_tb2(const fdtd_grid* g, int cur, long long n, const TileConfig& tc, cudaStream_t s)
 {
-    if (g->desc.precision != FDTD_F32 || needs_cell_passes(g)) return cudaErrorInvalidValue;
-    if (tc.ty == 8) return launch_tb2_t<8>(g, cur, n, tc, s);
-    return launch_tb2_t<16>(g, cur, n, tc, s);
+    if (g->desc.precision != FDTD_F32 || (has_walls(g) && !tc.automatic)) return cudaErrorInvalidValue;
+    if (tc.ty == 8) return launch_tb2_t<kTb2RowsSmall>(g, cur, n, tc, s);
+    return launch_tb2_t<kTb2Rows>(g, cur, n, tc, s);
 }
 
 cudaError_t launch_tb2_table(const fdtd_grid* cg, int cur, const StepTime<float>* times, int i0, int i1,
-                             int max_ctas, cudaStream_t s)
+                             int max_ctas, bool automatic, cudaStream_t s)
 {
     fdtd_grid* g = const_cast<fdtd_grid*>(cg);
-    if (g->desc.precision != FDTD_F32 || needs_cell_passes(g)) return cudaErrorInvalidValue;
-    constexpr int RY = 16;
+    if (g->desc.precision != FDTD_F32 || (has_walls(g) && !automatic)) return cudaErrorInvalidValue;
+    constexpr int RY = kTb2Rows;
     using S = Tb2Smem<RY>;
     int per_sm = 0;
     cudaError_t e = tb2_blocks_per_sm<RY>(&per_sm);
@@ -236,7 +321,13 @@ cudaError_t launch_tb2_table(const fdtd_grid* cg, int cur, const StepTime<float>
     TileConfig tc = g->tile;
     Tb2Plan plan;
     tb2_plan(g, RY, slots, tc, plan);
-    yee_tb2_t<RY><<<unsigned(slots), dim3(32, RY), S::bytes(), s>>>(make_args<float>(g, cur), times, i0, i1, plan);
+    TmaMaps* m = nullptr;
+    if (!tb2_maps<RY>(g, cur, &m)) return cudaErrorInvalidValue;
+    const StepArgs<float> a = make_args<float>(g, cur);
+    const unsigned ctas = unsigned(slots);
+    if (!automatic) yee_tb2_t<RY, false, false><<<ctas, S::NT, S::bytes(), s>>>(a, times, i0, i1, *m, plan);
+    else if (has_walls(g)) yee_tb2_t<RY, true, true><<<ctas, S::NT, S::bytes(), s>>>(a, times, i0, i1, *m, plan);
+    else yee_tb2_t<RY, false, true><<<ctas, S::NT, S::bytes(), s>>>(a, times, i0, i1, *m, plan);
     return cudaGetLastError();
 }
 

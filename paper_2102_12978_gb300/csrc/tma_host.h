@@ -25,7 +25,7 @@ inline PFN_cuTensorMapEncodeTiled_v12000 encode_fn()
 // 3-D tiled tensor map over one pitched [nz][ny][pitch] array; elements past
 // nx / ny (and before 0) read as zero.
 inline bool encode_map(CUtensorMap* m, void* base, size_t elem, const fdtd_grid_desc& d, int pitch, int bx,
-                       int by)
+                       int by, CUtensorMapL2promotion promotion = CU_TENSOR_MAP_L2_PROMOTION_L2_128B)
 {
     auto fn = encode_fn();
     if (!fn) return false;
@@ -35,7 +35,7 @@ inline bool encode_map(CUtensorMap* m, void* base, size_t elem, const fdtd_grid_
     cuuint32_t estr[3] = {1, 1, 1};
     CUresult r = fn(m, elem == 8 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT64 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, base, dims,
                     strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                    CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                    promotion, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS;
 }
 

@@ -89,13 +89,18 @@ __device__ __forceinline__ bool cell_gen_z(const StepArgs<real>& a, int k)
     return a.zw && (k == 0 || k + 1 == a.nz || k < a.npz || k >= a.nz - a.npz);
 }
 
-// Rounding of the source terms pinned by explicit operations (no contraction
-// left to the compiler), so that the term added inside a pass and the one
-// added by antenna_add round alike.
+// Rounding pinned by explicit operations (no contraction left to the
+// compiler): the source term added inside a pass and the one added by
+// antenna_add round alike, and the cell passes agree bit for bit with the
+// two-step kernel, whichever of them a run of steps takes.
 __device__ __forceinline__ float mul_rn(float x, float y) { return __fmul_rn(x, y); }
 __device__ __forceinline__ double mul_rn(double x, double y) { return __dmul_rn(x, y); }
 __device__ __forceinline__ float fma_rn(float x, float y, float z) { return __fmaf_rn(x, y, z); }
 __device__ __forceinline__ double fma_rn(double x, double y, double z) { return __fma_rn(x, y, z); }
+
+// CPML psi update b psi + aa d.
+template <typename real>
+__device__ __forceinline__ real psi_next(real b, real psi, real aa, real d) { return fma_rn(aa, d, mul_rn(b, psi)); }
 
 template <typename real>
 __device__ __forceinline__ Cpx<real> plane_factor(const StepArgs<real>& a, int k, Cpx<real> t)
@@ -207,17 +212,17 @@ __device__ __forceinline__ void h_cell(const StepArgs<real>& a, Cpx<real> th, in
     const real cz = (WALL && GEN && a.zw) ? fld<NC>(a.chz + k) : a.cz;
     const real dEz_y = ezj - ez, dEy_z = ey1 - ey, dEx_z = ex1 - ex;
     const real dEz_x = ezi - ez, dEy_x = eyi - ey, dEx_y = exj - ex;
-    hx = hx - chy * dEz_y + cz * dEy_z;
-    hy = hy - cz * dEx_z + chx * dEz_x;
-    hz = hz - chx * dEy_x + chy * dEx_y;
+    hx = fma_rn(cz, dEy_z, fma_rn(-chy, dEz_y, hx));
+    hy = fma_rn(chx, dEz_x, fma_rn(-cz, dEx_z, hy));
+    hz = fma_rn(chy, dEx_y, fma_rn(-chx, dEy_x, hz));
     if (GEN && a.npml > 0) {
         const int npml = a.npml, w2 = 2 * npml;
         if (i < npml || i >= nx - npml) {
             const int ii = i < npml ? i : i - nx + w2;
             const int q = (k * ny + j) * w2 + ii;
             const real b = a.bhx[ii], aa = a.ahx[ii];
-            const real p0 = b * a.phx_in[0][q] + aa * dEz_x;   // Hyx
-            const real p1 = b * a.phx_in[1][q] + aa * dEy_x;   // Hzx
+            const real p0 = psi_next(b, a.phx_in[0][q], aa, dEz_x);   // Hyx
+            const real p1 = psi_next(b, a.phx_in[1][q], aa, dEy_x);   // Hzx
             hy += p0;
             hz -= p1;
             a.phx_out[0][q] = p0; a.phx_out[1][q] = p1;
@@ -226,8 +231,8 @@ __device__ __forceinline__ void h_cell(const StepArgs<real>& a, Cpx<real> th, in
             const int jj = j < npml ? j : j - ny + w2;
             const int q = (k * w2 + jj) * pitch + i;
             const real b = a.bhy[jj], aa = a.ahy[jj];
-            const real p0 = b * a.phy_in[0][q] + aa * dEz_y;   // Hxy
-            const real p1 = b * a.phy_in[1][q] + aa * dEx_y;   // Hzy
+            const real p0 = psi_next(b, a.phy_in[0][q], aa, dEz_y);   // Hxy
+            const real p1 = psi_next(b, a.phy_in[1][q], aa, dEx_y);   // Hzy
             hx -= p0;
             hz += p1;
             a.phy_out[0][q] = p0; a.phy_out[1][q] = p1;
@@ -237,8 +242,8 @@ __device__ __forceinline__ void h_cell(const StepArgs<real>& a, Cpx<real> th, in
         const int w2 = 2 * a.npz, kk = k < a.npz ? k : k - nz + w2;
         const int q = (kk * ny + j) * pitch + i;
         const real b = a.bhz[kk], aa = a.ahz[kk];
-        const real p0 = b * a.phz_in[0][q] + aa * dEy_z;   // Hxz
-        const real p1 = b * a.phz_in[1][q] + aa * dEx_z;   // Hyz
+        const real p0 = psi_next(b, a.phz_in[0][q], aa, dEy_z);   // Hxz
+        const real p1 = psi_next(b, a.phz_in[1][q], aa, dEx_z);   // Hyz
         hx += p0;
         hy -= p1;
         a.phz_out[0][q] = p0; a.phz_out[1][q] = p1;
@@ -294,17 +299,17 @@ __device__ __forceinline__ void e_cell(const StepArgs<real>& a, Cpx<real> te, Cp
     const real cz = (WALL && GEN && a.zw) ? fld<NC>(a.cez + k) : a.cz;
     const real dHz_y = hz - hzj, dHy_z = hy - hym, dHx_z = hx - hxm;
     const real dHz_x = hz - hzi, dHy_x = hy - hyi, dHx_y = hx - hxj;
-    real nex = ex + cey * dHz_y - cz * dHy_z;
-    real ney = ey + cz * dHx_z - cex * dHz_x;
-    real nez = ez + cex * dHy_x - cey * dHx_y;
+    real nex = fma_rn(-cz, dHy_z, fma_rn(cey, dHz_y, ex));
+    real ney = fma_rn(-cex, dHz_x, fma_rn(cz, dHx_z, ey));
+    real nez = fma_rn(-cey, dHx_y, fma_rn(cex, dHy_x, ez));
     if (GEN && a.npml > 0) {
         const int npml = a.npml, w2 = 2 * npml;
         if (i < npml || i >= nx - npml) {
             const int ii = i < npml ? i : i - nx + w2;
             const int q = (k * ny + j) * w2 + ii;
             const real b = a.bex[ii], aa = a.aex[ii];
-            const real p0 = b * a.pex[0][q] + aa * dHz_x;   // Eyx
-            const real p1 = b * a.pex[1][q] + aa * dHy_x;   // Ezx
+            const real p0 = psi_next(b, a.pex[0][q], aa, dHz_x);   // Eyx
+            const real p1 = psi_next(b, a.pex[1][q], aa, dHy_x);   // Ezx
             if (live) { a.pex[0][q] = p0; a.pex[1][q] = p1; }
             ney -= p0;
             nez += p1;
@@ -313,8 +318,8 @@ __device__ __forceinline__ void e_cell(const StepArgs<real>& a, Cpx<real> te, Cp
             const int jj = j < npml ? j : j - ny + w2;
             const int q = (k * w2 + jj) * pitch + i;
             const real b = a.bey[jj], aa = a.aey[jj];
-            const real p0 = b * a.pey[0][q] + aa * dHz_y;   // Exy
-            const real p1 = b * a.pey[1][q] + aa * dHx_y;   // Ezy
+            const real p0 = psi_next(b, a.pey[0][q], aa, dHz_y);   // Exy
+            const real p1 = psi_next(b, a.pey[1][q], aa, dHx_y);   // Ezy
             if (live) { a.pey[0][q] = p0; a.pey[1][q] = p1; }
             nex += p0;
             nez -= p1;
@@ -324,8 +329,8 @@ __device__ __forceinline__ void e_cell(const StepArgs<real>& a, Cpx<real> te, Cp
         const int w2 = 2 * a.npz, kk = k < a.npz ? k : k - nz + w2;
         const int q = (kk * ny + j) * pitch + i;
         const real b = a.bez[kk], aa = a.aez[kk];
-        const real p0 = b * a.pez[0][q] + aa * dHy_z;   // Exz
-        const real p1 = b * a.pez[1][q] + aa * dHx_z;   // Eyz
+        const real p0 = psi_next(b, a.pez[0][q], aa, dHy_z);   // Exz
+        const real p1 = psi_next(b, a.pez[1][q], aa, dHx_z);   // Eyz
         if (live) { a.pez[0][q] = p0; a.pez[1][q] = p1; }
         nex -= p0;
         ney += p1;
@@ -342,7 +347,7 @@ __device__ __forceinline__ void e_cell(const StepArgs<real>& a, Cpx<real> te, Cp
     }
     if (WALL && a.wcoefr && k == a.wplane) {   // wall source (Section 2), after the antenna
         const Cpx<real> w = static_cast<const Cpx<real>*>(a.wcoefr)[j * nx + i];
-        nex += w.x * tw.x - w.y * tw.y;
+        nex += fma_rn(w.x, tw.x, -mul_rn(w.y, tw.y));
     }
     if (GEN) {
         if (j == 0) { nex = real(0); nez = real(0); }   // PEC: tangential E
@@ -433,12 +438,13 @@ __device__ __forceinline__ void e_cell(const StepArgs<real>& a, Cpx<real> te, Cp
             hby = (oy + hy) + (oyj + hyj);
             hbz = (oz + hz) + (oz1 + hz1);
         }
-        const real sx = cy * hbz - cc * hby;
-        const real sy = cc * hbx - cx * hbz;
-        const real sz = cx * hby - cy * hbx;
+        const real sx = fma_rn(cy, hbz, -mul_rn(cc, hby));
+        const real sy = fma_rn(cc, hbx, -mul_rn(cx, hbz));
+        const real sz = fma_rn(cx, hby, -mul_rn(cy, hbx));
+        const real s2 = fma_rn(sz, sz, fma_rn(sy, sy, mul_rn(sx, sx)));
         acc_t* F = static_cast<acc_t*>(a.fluence);
         const real dt16 = real(a.dt16);
-        if (live) F[g] = Acc::add(F[g], vec_norm(sx * sx + sy * sy + sz * sz) * dt16);
+        if (live) F[g] = Acc::add_fma(F[g], vec_norm(s2), dt16);
     }
 }
 

@@ -73,12 +73,13 @@ struct StepArgs {
     const void* zphr;        // the same in the field precision (float2 / double2)
     SrcTime st;
     int fault;               // test hook (fdtd_debug_inject_fault): 1 = CTA (0,0,0) withholds one plane's copies
-    // z walls (Section 2's Bessel-Gauss box; the cell passes only): PEC at
-    // z = 0 and z = nz dz, npz CPML cells inside each
+    // z walls (Section 2's Bessel-Gauss box; the cell passes and the two-step
+    // kernel): PEC at z = 0 and z = nz dz, npz CPML cells inside each
     int zw, npz;
     const real* phz_in[2];   // z shell H psi: Hxz, Hyz   [2 npz][ny][pitch]
     real* phz_out[2];
     real* pez[2];            // z shell E psi: Exz, Eyz (in place)
+    real* pez_out[2];        // the other copy, as pex_out
     const real* chz;         // dt / (kappa dz) at H z-positions (k+1/2), length nz
     const real* cez;         // dt / (kappa dz) at E z-positions k
     const real* bhz;         // CPML b and a' = dt a / dz on the z shell, length 2 npz
@@ -125,12 +126,20 @@ template <typename real> struct FluAcc;
 template <> struct FluAcc<double> {
     using T = double;
     __device__ __forceinline__ static T add(T old, double v_dt) { return old + v_dt; }
+    __device__ __forceinline__ static T add_fma(T old, double v, double dt) { return __fma_rn(v, dt, old); }
 };
 template <> struct FluAcc<float> {
     using T = float2;
     __device__ __forceinline__ static T add(T old, float v_dt)
     {
         const float y = v_dt - old.y;
+        const float t = old.x + y;
+        return make_float2(t, (t - old.x) - y);
+    }
+    // the same with the product v dt inside the first fused multiply-add
+    __device__ __forceinline__ static T add_fma(T old, float v, float dt)
+    {
+        const float y = __fmaf_rn(v, dt, -old.y);
         const float t = old.x + y;
         return make_float2(t, (t - old.x) - y);
     }

@@ -5,35 +5,45 @@
 // fluence accumulator and the CPML psi cross HBM once per two steps: half the
 // bytes per cell-update of any one-step pass.  Every arithmetic step is the
 // one of the cell passes (Section 4 Yee update with the Roden-Gedney CPML,
-// the soft source of Eq. 13, the fluence of Section 2), in the same order.
+// the soft source of Eq. 13, the fluence of Section 2), in the same order; with
+// CR (see tb2_flux) the two agree bit for bit.
 //
 // Work decomposition.
-//   * A CTA of 32 x RY threads owns a window of 32 x RY (i, j) columns; each
-//     thread owns one column and marches along z.  Windows overlap by two
-//     columns / rows on each side: a window updates E^{n+2} only on its inner
-//     28 x (RY - 4) columns (windows on the box faces also on the face side,
-//     where the PEC wall supplies the neighbours), and recomputes the two
-//     outer rings itself (H^{n+1/2} on the window less its last column,
-//     E^{n+1} one column in, H^{n+3/2} another).  Columns past the box hold
-//     exact zeros at every stage (zero-filled loads, zero coefficients): the
-//     wall values the stencil reads there.
+//   * A CTA owns a window of 32 x RY (i, j) columns and marches along z; each
+//     thread owns two x-adjacent columns (16 RY threads, a half warp per
+//     row).  A window writes E^{n+2} and H^{n+3/2} only on its own 24 x
+//     (RY - 4) columns, which start 4 columns and 2 rows in, and recomputes
+//     what they need around them itself (E^{n+2} can be had from 2 columns and
+//     rows in).  Columns past the box hold exact zeros at every stage
+//     (zero-filled loads, zero coefficients): the wall values the stencil
+//     reads there.
+//   * Own columns start at multiples of 8, so that every store fills whole
+//     32-byte sectors.  Stores of partial sectors were what held the kernel:
+//     with own columns 28 wide (of the same 32), whose rows begin and end
+//     inside a sector, a plane of an inner window took 3900 cycles, against
+//     2380 with full sectors and 2050 without any loads and stores
+//     (256 x 256 x 128 cells, one GB300); the 24-wide windows are a fifth more
+//     and still faster by a third.
+//   * Two columns per thread, because the kernel is bound by instruction
+//     issue and latency before HBM and the FP32 pipe: the FP32 arithmetic of
+//     the two columns is one packed instruction (fma.rn.f32x2 and its kin run
+//     at half the rate of the scalar ones, so the pipe is as busy and the
+//     issue slots are halved), shared-memory accesses and stores move both
+//     columns at once, the x neighbours of the pair take one shuffle, and a
+//     window of 32 x 24 columns fits the register file with 12 warps.  430
+//     instructions per warp and plane of 64 columns, against 385 per 32
+//     columns with one column per thread.
 //   * z-march with a wavefront of four stages per plane p: A, H^{n+1/2} of
 //     plane p-1; B, E^{n+1} of plane p-1; C, H^{n+3/2} of plane p-2; D,
-//     E^{n+2} of plane p-2.  The +x / -x neighbours come from the adjacent
-//     lane by warp shuffle, the +y / -y neighbours from per-plane shared
-//     exchange buffers (two CTA barriers per plane), the +z / -z neighbours
-//     from registers carried from plane to plane.
-//   * Each thread streams its own column: the E^n and H^{n-1/2} values and
-//     the fluence accumulator of plane p + 3 and the CPML psi of plane p + 2
-//     (shell columns) are copied by cp.async (zero-filled past the box) into
-//     a per-thread ring of four plane slots in shared memory (see
-//     tb2_issue); a thread waits only for its
-//     own copies, so the ring needs no barrier.  The psi of a plane are
-//     updated in place in its slot (n-1/2 -> n+1/2, n -> n+1) and read back
-//     by the second step's stages.  The plane loop is unrolled by two, so
-//     the exchange buffers' parities are constants; the ring slot is an index
-//     (a four-fold unroll that made it a constant too ran 1 % slower: its
-//     loop body is twice as large).
+//     E^{n+2} of plane p-2.  The y neighbours come from per-plane shared
+//     exchange buffers (E^n straight from the ring of loaded planes), the
+//     z neighbours from registers carried from plane to plane; two CTA
+//     barriers per plane.
+//   * Planes are loaded by TMA, one box per array (32 x RY columns of E^n and
+//     H^{n-1/2} of plane p + 3 and of the fluence of plane p), zero-filled
+//     past the box, into a ring of four slots; a slot completes on its own
+//     mbarrier.  A thread copies the CPML psi of its own shell columns by
+//     cp.async into two slots of its own.
 //   * The antenna coefficients of a window's columns are staged in shared
 //     memory when the window starts; the per-plane phase e^{i beta z_k} is
 //     loaded one plane ahead.
@@ -47,12 +57,13 @@
 //     recompute race-free.
 //   * Every row of a window runs every stage, whether or not a column the
 //     window writes depends on it, so that the stage code has no branches
-//     on the row; a row with antenna points adds the source terms on all its
+//     on the row; a warp with antenna points adds the source terms on all its
 //     lanes (zero terms where a column has none), and the x-shell windows
 //     update the x psi on all lanes (zero coefficients off the shell).
-//     Windows off the box faces and the CPML shells run code without the
-//     checks of the walls, psi and columns past the box (template flags GX,
-//     GY).
+//     Windows off the x (y) faces and shells run code without the checks of
+//     the x (y) walls, psi and columns past the box (template flags GX, GY).
+//     A plane of an inner window takes 2400 cycles, of an x- or y-shell window
+//     3400, of a corner 4700.
 //   * A CTA takes a contiguous range of the flattened (window, plane) work:
 //     ranges of equal estimated cost (windows with CPML shell or antenna
 //     columns weigh more, with weights the autotuner picks by timing), or
@@ -60,12 +71,16 @@
 //     (the kernel records each CTA's SM cycles when asked).  The window rows
 //     may be interleaved in the flattened order, so that x-neighbouring
 //     windows march side by side (tb2_window_at).  Where a range starts or
-//     crosses into the next window the wavefront restarts, which costs three
-//     planes of recompute.
+//     crosses into the next window the wavefront restarts, which costs four
+//     planes of recompute and the latency of the first loads.
 //   * Outputs are stored with the L2 evict-last policy; every sum of two
 //     products is rounded explicitly (see below).
-// z-periodic grids only (the antenna boxes of Section 4); FP32 fields with the
-// Kahan FP32 fluence.
+//   * Grids with z walls or a wall sheet run an instantiation of their own
+//     (W), whose planes off the z shells run the loop above with the walls'
+//     few extra tests; z-shell planes run apart.
+// FP32 fields with the Kahan FP32 fluence.  256 x 256 x 128 cells with a
+// 16-cell CPML, antenna and fluence: 101-105 us per step (one column per
+// thread, windows of 32 x 16 with 28 x 12 own columns: 122-130 us).
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -75,9 +90,9 @@
 namespace fdtd {
 
 // Source time factors f e^{-i Phi} of the two steps: H at (n+1/2) dt and
-// (n+3/2) dt, E at (n+1) dt and (n+2) dt.
+// (n+3/2) dt, E (and the wall sheet) at (n+1) dt and (n+2) dt.
 struct Tb2Times {
-    Cpx<float> th0, te0, th1, te1;
+    Cpx<float> th0, te0, th1, te1, tw0, tw1;
 };
 
 // Flattened work: windows T (along x) by U (along y), nz planes each, items
@@ -99,6 +114,8 @@ constexpr int kTb2MaxCtas = 512;
 struct Tb2Plan {
     int T, U, D;
     unsigned long long* prof;
+    int* err;                    // the grid's error word (an expired wait raises it)
+    float dt16;                  // dt / 16
     long long start[kTb2MaxCtas + 1];
 };
 
@@ -114,29 +131,44 @@ __device__ __forceinline__ int tb2_window_at(const Tb2Plan& tw, int pos)
 
 // Columns per window along x, and the stride between windows.
 constexpr int kTb2Wx = 32;
-constexpr int kTb2Sx = 28;
-
+constexpr int kTb2Sx = 24;
+constexpr int kTb2Ox = 4;   // first own column of a window
+constexpr int kTb2Oy = 2;   // first own row
+// Window rows: tile heights (ty) 16 and 8.
+constexpr int kTb2Rows = 24;
+constexpr int kTb2RowsSmall = 12;
 
 template <int RY>
 struct Tb2Smem {
-    static constexpr int NT = 32 * RY;   // threads (columns) per window
-    static constexpr int R = 4;          // ring slots per thread (see tb2_issue)
-    static constexpr int NF = 14;        // ring floats per slot: E^n 3, H^{n-1/2} 3, psi 8
-    // exchange arrays: a row of zeros before and after the window's RY rows
-    // (the values of the rows beyond it), so that a y neighbour is one plain
-    // shared load; thread tid's value at XO + tid.  Consecutive arrays share
-    // a zero row (the row after array a is the row before array a + 1), and
-    // one more zero row follows the last array.
-    static constexpr int XS = NT + 32, XO = 32;
-    static constexpr int NX = 14;         // 2x2 E^n, 3 H^{n+1/2}, 2x2 E^{n+1}, 3 H^{n+3/2}
+    static constexpr int NT = 16 * RY;   // threads: two columns each
+    static constexpr int NC = 32 * RY;   // columns per window
+    static constexpr int R = 4;          // ring slots (see tb2_issue)
+    static constexpr int SLOT = 8 * NC;  // floats per slot: E^n 3, H^{n-1/2} 3, fluence (float2)
+    static constexpr int NP = 8;         // psi values per column and slot (two slots)
+    // exchange arrays, and a row's room before the first and after the last
+    // (a y neighbour past the window's rows reads there, for halo rows only)
+    static constexpr int XS = NC, XO = 32;
+    static constexpr int NX = 10;        // 3 H^{n+1/2}, 2x2 E^{n+1}, 3 H^{n+3/2}
     static constexpr size_t bytes()
     {
-        return size_t(R) * NT * 8                 // fluence accumulator (float2) per slot
-               + size_t(R) * NF * NT * 4          // fields and psi per slot
-               + (size_t(NX) * XS + 32) * 4       // exchange arrays and their zero rows
-               + size_t(12) * NT * 4;             // antenna coefficients of the column (6 complex)
+        return size_t(R) * SLOT * 4 + size_t(2) * NP * NC * 4    // planes, psi
+               + (size_t(NX) * XS + 64) * 4                      // exchange arrays
+               + size_t(12) * NC * 4                             // antenna coefficients of the columns (6 complex)
+               + R * 8 + 128;                                    // mbarriers, alignment
     }
 };
+
+// ---- pairs of columns: packed FP32, rounded as the scalar operations.  The
+// compiler may contract a packed multiply whose result feeds a packed add or
+// subtract (it does so across one side of an unrolled loop and not the
+// other, which would make results depend on the work split): no mul2 below
+// feeds an add2 or sub2, only the addend of an fma2.
+__device__ __forceinline__ float2 dup2(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 neg2(float2 v) { return make_float2(-v.x, -v.y); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __fadd2_rn(a, neg2(b)); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 
 __device__ __forceinline__ void cpa4(float* dst, const float* src, bool valid)
 {
@@ -144,31 +176,32 @@ __device__ __forceinline__ void cpa4(float* dst, const float* src, bool valid)
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(valid ? 4 : 0)
                  : "memory");
 }
-__device__ __forceinline__ void cpa8(float2* dst, const float2* src, bool valid)
+// bytes: 8, or 4 (the second element zero-filled), or 0
+__device__ __forceinline__ void cpa8(float* dst, const float* src, int bytes)
 {
     const unsigned d = static_cast<unsigned>(__cvta_generic_to_shared(dst));
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(src), "r"(valid ? 8 : 0)
-                 : "memory");
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(src), "r"(bytes) : "memory");
 }
 __device__ __forceinline__ void cpa_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cpa_wait2() { asm volatile("cp.async.wait_group 2;" ::: "memory"); }
+__device__ __forceinline__ void cpa_wait1() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }
 __device__ __forceinline__ void cpa_wait0() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
-// Every sum of two products below is written with explicit roundings
-// (mul_rn / fma_rn): the plane loop runs two instantiations of tb2_plane
-// (the exchange parities), and which one computes a plane depends on where
-// the CTA's range of planes starts; left to the compiler, the two could
-// contract such a sum into a fused multiply-add in different ways, and the
-// results would depend on the CTAs' work split.
-
-// |E x Hbar| dt of a cell from its centre sums (the 1/16 of the four-edge E
-// means and the two-face, two-time H means is folded into dt16).
-__device__ __forceinline__ float tb2_flux(float cx, float cy, float cc, float hbx, float hby, float hbz, float dt16)
+// |E x Hbar| of a cell from its centre sums, times dt16 unless CR (the 1/16 of
+// the four-edge E means and the two-face, two-time H means is folded into
+// dt16).  CR: the roundings of the cell passes, which fuse the product with
+// dt16 into the accumulator's add and take the CPML products in the other order
+// (runs on the default tile, which mix both kernels); otherwise those of tile
+// variant 7.
+template <bool CR>
+__device__ __forceinline__ float2 tb2_flux(float2 cx, float2 cy, float2 cc, float2 hbx, float2 hby, float2 hbz,
+                                           float dt16)
 {
-    const float sx = fma_rn(cy, hbz, -mul_rn(cc, hby));
-    const float sy = fma_rn(cc, hbx, -mul_rn(cx, hbz));
-    const float sz = fma_rn(cx, hby, -mul_rn(cy, hbx));
-    return mul_rn(vec_norm(fma_rn(sz, sz, fma_rn(sy, sy, mul_rn(sx, sx)))), dt16);
+    const float2 sx = fma2(cy, hbz, neg2(mul2(cc, hby)));
+    const float2 sy = fma2(cc, hbx, neg2(mul2(cx, hbz)));
+    const float2 sz = fma2(cx, hby, neg2(mul2(cy, hbx)));
+    const float2 s = fma2(sz, sz, fma2(sy, sy, mul2(sx, sx)));
+    if (CR) return make_float2(vec_norm(s.x), vec_norm(s.y));
+    return make_float2(mul_rn(vec_norm(s.x), dt16), mul_rn(vec_norm(s.y), dt16));
 }
 
 __device__ __forceinline__ Cpx<float> cmul(Cpx<float> z, Cpx<float> t)
@@ -177,10 +210,8 @@ __device__ __forceinline__ Cpx<float> cmul(Cpx<float> z, Cpx<float> t)
 }
 
 // Stores of the window's outputs with the L2 evict-last priority: a window
-// writes its own 28 columns of a row, so the first and last 32-byte sectors
-// of the row are shared with the neighbouring windows, which write their
-// part at another time; kept in L2 until the neighbour's part arrives, such
-// a sector reaches DRAM whole.
+// writes 96 bytes of a row, so its first or last 128-byte line is shared with a
+// neighbouring window, which writes its part at another time.
 __device__ __forceinline__ uint64_t tb2_store_policy()
 {
     uint64_t p;
@@ -196,88 +227,129 @@ __device__ __forceinline__ void st_keep(float2* q, float2 v, uint64_t pol)
     asm volatile("st.global.L2::cache_hint.v2.f32 [%0], {%1, %2}, %3;" ::"l"(q), "f"(v.x), "f"(v.y), "l"(pol)
                  : "memory");
 }
+__device__ __forceinline__ void st_keep(float4* q, float4 v, uint64_t pol)
+{
+    asm volatile("st.global.L2::cache_hint.v4.f32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(q), "f"(v.x), "f"(v.y),
+                 "f"(v.z), "f"(v.w), "l"(pol)
+                 : "memory");
+}
 
-// CPML psi update b psi + a d.
-__device__ __forceinline__ float psi_rn(float b, float psi, float aa, float d) { return fma_rn(b, psi, mul_rn(aa, d)); }
+// CPML psi update b psi + a d (CR: rounded as the cell passes' psi_next).
+template <bool CR>
+__device__ __forceinline__ float2 psi2(float2 b, float2 psi, float2 aa, float2 d)
+{
+    return CR ? fma2(aa, d, mul2(b, psi)) : fma2(b, psi, mul2(aa, d));
+}
 
-// Per-window constants of a thread's column.
+// Per-window constants of a thread's two columns (i, j), (i + 1, j).
 struct Tb2Col {
-    int i, j, lane, row, tid;
-    bool indom, own, fown, sx, sy, ant;   // ant: the window holds antenna columns
-    bool anth, ante;                      // warp-uniform: the row holds antenna H / E points
-    uint8_t mk;
+    int i, j, l, row, at;                 // l: half-warp lane; at: the pair's offset in a window array
+    bool own0, own1, f0, f1;              // columns whose fields / fluence the window writes
+    bool sx0, sx1, sy;                    // columns in an x shell, row in a y shell
+    bool in0, in1;                        // columns inside the box
+    bool xpair;                           // nx and npml even: an x shell holds whole pairs at even offsets
+    bool ant, anth, ante;                 // the window holds antenna columns; the warp holds H / E points
     int col, colx, coly;
-    float chx, chy, cex, cey, bhx, ahx, bex, aex, bhy, ahy, bey, aey;
+    float2 chx, chy, cex, cey, bhx, ahx, bex, aex, bhy, ahy, bey, aey;
 };
 
 // Values carried from plane to plane (planes relative to the current p).
 struct Tb2Carry {
-    float e0[3];                  // E^n(p-1)
-    float h1p[3];                 // H^{n+1/2}(p-2)
-    float e1p[3];                 // E^{n+1}(p-2)
-    float h2px, h2py;             // H^{n+3/2}(p-3), x and y
+    float2 e0[3];                  // E^n(p-1)
+    float2 h1p[3];                 // H^{n+1/2}(p-2)
+    float2 e1p[3];                 // E^{n+1}(p-2)
+    float2 h2px, h2py;             // H^{n+3/2}(p-3), x and y
     // fluence centre sums: step n of plane p-2 (f), step n+1 of plane p-3 (g)
-    float fPEx, fPEy, fcz, fhbx, fhby, fHsz;
-    float gPEx, gPEy, gcz, ghbx, ghby, gHsz;
-    float tn;                     // fluence term of step n, plane p-3
-    int kp, kq, kr, k3, ki;       // planes of p, p-1, p-2, p-3 and p+2 (modulo nz)
-    Cpx<float> zq, zr;            // e^{i beta z} of planes p-1 and p-2
+    float2 fPEx, fPEy, fcz, fhbx, fhby, fHsz;
+    float2 gPEx, gPEy, gcz, ghbx, ghby, gHsz;
+    float2 tn;                     // fluence term of step n, plane p-3
+    float2 px[4], py[4];           // psi of plane p-2 after step n: Hyx Hzx Eyx Ezx, Hxy Hzy Exy Ezy
+    int kp, kq, kr, k3, ki;        // planes of p, p-1, p-2, p-3 and p+3 (modulo nz; as they are on z-walled grids)
+    Cpx<float> zq, zr;             // e^{i beta z} of planes p-1 and p-2
 };
 
 template <int RY>
 struct Tb2Bufs {
-    float2* fring;   // [R][NT]
-    float* ring;     // [R][NF][NT]
-    float* EB;       // [2][Ez, Ex][XS]: E^n of a plane
+    float* ring;     // [R][SLOT]: E^n, H^{n-1/2} [6][RY][32], fluence [RY][32] (float2)
+    float* psi;      // [2][NP][NC]: Hyx Hzx Hxy Hzy Eyx Ezx Exy Ezy
     float* HB;       // [Hx, Hz, Hy^{n-1/2} + Hy^{n+1/2}][XS]
     float* E1B;      // [2][Ez, Ex][XS]: E^{n+1}
     float* H1B;      // [Hx, Hz, Hy^{n+1/2} + Hy^{n+3/2}][XS]
-    float2* SC;      // [6][NT]: antenna coefficients (zero where a column has no point of the component)
+    float* SC;       // [6][re, im][NC]: antenna coefficients (zero where a column has no point of the component)
+    uint64_t* bars;  // [R]
+    int* err;        // the grid's error word
+    uint64_t pol;    // L2 evict-last policy of the stores
 };
 
 __device__ __forceinline__ int next_plane(int k, int nz) { return k + 1 == nz ? 0 : k + 1; }
+// The plane after k; W: planes past the walls of a z-walled grid are real
+// indices (their boxes read as zeros, the wall's values).
+template <bool W>
+__device__ __forceinline__ int tb2_next(const StepArgs<float>& a, int k)
+{
+    return W && a.zw ? k + 1 : next_plane(k, a.nz);
+}
 
-// Copies of this thread's column, one cp.async group: E^n and H^{n-1/2} of
-// plane k and the fluence accumulator of plane kf into slot s, the psi of
-// plane kp into slot sp.  A plane's fields are first read at its own stage A
-// (E^n) and its psi one plane later (stage A of the next plane), so that at
-// the end of plane p the fields of p + 3 (fluence p) go into the slot the
-// fields of p - 1 have left and the psi of p + 2 into the slot the psi of
-// p - 2 have left: with four slots the fields are copied three planes ahead
-// of their first use, the psi two and a half.
-template <int RY, int G>
-__device__ __forceinline__ void tb2_issue(const StepArgs<float>& a, const Tb2Col& c, const Tb2Bufs<RY>& b, int s,
-                                          int k, int kf, int sp, int kp)
+__device__ __forceinline__ float2 ld2(const float* q) { return *reinterpret_cast<const float2*>(q); }
+__device__ __forceinline__ void st2(float* q, float2 v) { *reinterpret_cast<float2*>(q) = v; }
+
+// Box loads of one iteration into ring slot s: E^n and H^{n-1/2} of plane k,
+// the fluence of plane kf, at window corner (x, y).  Called by every thread;
+// lane 0 of each of the first seven warps issues one box (warps loop where
+// there are fewer), lane 0 of warp 0 arms the slot's mbarrier (bytes landing
+// before it does keep the phase open: its arrival is the one the phase waits
+// for).
+template <int RY>
+__device__ __forceinline__ void tb2_issue(const StepArgs<float>& a, const TmaMaps& m, const Tb2Bufs<RY>& b, int s,
+                                          int k, int kf, int x, int y)
 {
     using S = Tb2Smem<RY>;
-    constexpr int NT = S::NT, NF = S::NF;
-    float* r = b.ring + s * NF * NT + c.tid;
-    float* rs = b.ring + sp * NF * NT + c.tid;
+    if ((threadIdx.x & 31) != 0) return;
+    float* dst = b.ring + s * S::SLOT;
+    uint64_t* bar = b.bars + s;
+    const int nbox = a.fluence ? 7 : 6;
+    #pragma unroll 1
+    for (int q = threadIdx.x >> 5; q < nbox; q += S::NT / 32) {
+        if (q == 0) mbar_expect_tx(bar, uint32_t((a.fluence ? 8 : 6) * S::NC * 4));
+        tma_load_3d(dst + q * S::NC, &m.e[0] + q, bar, x, y, q < 6 ? k : kf);
+    }
+}
+
+// The CPML psi of this thread's shell columns in plane k into psi slot s, one
+// cp.async group.
+template <int RY, int G, bool W>
+__device__ __forceinline__ void tb2_issue_psi(const StepArgs<float>& a, const Tb2Col& c, const Tb2Bufs<RY>& b, int s,
+                                              int k)
+{
+    using S = Tb2Smem<RY>;
+    constexpr int NC = S::NC;
     constexpr bool GX = G & 1, GY = G & 2;
-    const int g = k * (a.pitch * a.ny) + c.col;
-    cpa4(r + 0 * NT, a.ein[0] + g, (!GX && !GY) || c.indom);
-    cpa4(r + 1 * NT, a.ein[1] + g, (!GX && !GY) || c.indom);
-    cpa4(r + 2 * NT, a.ein[2] + g, (!GX && !GY) || c.indom);
-    cpa4(r + 3 * NT, a.hin[0] + g, (!GX && !GY) || c.indom);
-    cpa4(r + 4 * NT, a.hin[1] + g, (!GX && !GY) || c.indom);
-    cpa4(r + 5 * NT, a.hin[2] + g, (!GX && !GY) || c.indom);
+    if (!GX && !GY) return;
+    const bool in = !(W && a.zw) || (k >= 0 && k < a.nz);   // zeros past a z wall
+    if (W && !in) k = 0;
+    float* r = b.psi + s * S::NP * NC + c.at;
     if (GX) {   // every lane: zeros where the column is not in an x shell
-        const int q = kp * a.ny * (2 * a.npml) + c.colx;
-        cpa4(rs + 6 * NT, a.phx_in[0] + q, c.sx);    // Hyx
-        cpa4(rs + 7 * NT, a.phx_in[1] + q, c.sx);    // Hzx
-        cpa4(rs + 10 * NT, a.pex[0] + q, c.sx);      // Eyx
-        cpa4(rs + 11 * NT, a.pex[1] + q, c.sx);      // Ezx
+        const int q = k * a.ny * (2 * a.npml) + c.colx;
+        const float* src[4] = {a.phx_in[0], a.phx_in[1], a.pex[0], a.pex[1]};
+        constexpr int slot[4] = {0, 1, 4, 5};
+        if (c.xpair) {
+            #pragma unroll
+            for (int v = 0; v < 4; ++v) cpa8(r + slot[v] * NC, src[v] + q, in && c.sx0 ? 8 : 0);
+        } else
+        #pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            cpa4(r + slot[v] * NC, src[v] + q, in && c.sx0);
+            cpa4(r + slot[v] * NC + 1, src[v] + q + (c.sx1 ? 1 : 0), in && c.sx1);
+        }
     }
-    if (GY && c.sy) {
-        const int q = kp * (2 * a.npml) * a.pitch + c.coly;
-        cpa4(rs + 8 * NT, a.phy_in[0] + q, true);    // Hxy
-        cpa4(rs + 9 * NT, a.phy_in[1] + q, true);    // Hzy
-        cpa4(rs + 12 * NT, a.pey[0] + q, true);      // Exy
-        cpa4(rs + 13 * NT, a.pey[1] + q, true);      // Ezy
+    if (GY) {
+        const int q = k * (2 * a.npml) * a.pitch + c.coly;
+        const int bytes = in && c.sy ? (c.in1 ? 8 : (c.in0 ? 4 : 0)) : 0;
+        cpa8(r + 2 * NC, a.phy_in[0] + q, bytes);
+        cpa8(r + 3 * NC, a.phy_in[1] + q, bytes);
+        cpa8(r + 6 * NC, a.pey[0] + q, bytes);
+        cpa8(r + 7 * NC, a.pey[1] + q, bytes);
     }
-    const float2* F = static_cast<const float2*>(a.fluence);
-    cpa8(b.fring + s * NT + c.tid, c.fown ? F + kf * (a.pitch * a.ny) + c.col : reinterpret_cast<const float2*>(a.ein[0]),
-         c.fown);
     cpa_commit();
 }
 
@@ -285,196 +357,292 @@ __device__ __forceinline__ void tb2_issue(const StepArgs<float>& a, const Tb2Col
 // SC; zero, and the increment a signed zero, where the column has no point of
 // the component).
 template <int RY>
-__device__ __forceinline__ float tb2_src(const Tb2Bufs<RY>& b, const Tb2Col& c, int comp, Cpx<float> u)
+__device__ __forceinline__ float2 tb2_src(const Tb2Bufs<RY>& b, const Tb2Col& c, int comp, Cpx<float> u)
 {
-    constexpr int NT = Tb2Smem<RY>::NT;
-    const float2 v = b.SC[comp * NT + c.tid];
-    return fma_rn(v.x, u.x, -mul_rn(v.y, u.y));
+    constexpr int NC = Tb2Smem<RY>::NC;
+    const float2 re = ld2(b.SC + (2 * comp) * NC + c.at), im = ld2(b.SC + (2 * comp + 1) * NC + c.at);
+    return fma2(re, dup2(u.x), neg2(mul2(im, dup2(u.y))));
 }
 
-// One plane p of the wavefront: u = (p - P0) mod 4 is its ring slot, and
-// U = (p - P0) mod 2 gives the exchange-buffer parities at compile time.
-// Every row runs every stage: a row whose results no written column needs
-// computes values that reach no output (rows beyond the window read the zero
-// rows of the exchange arrays), and the stage code stays free of branches.
-template <int RY, int U, int G>
-__device__ __forceinline__ void tb2_plane(const StepArgs<float>& a, const Tb2Times& tt, const Tb2Col& c,
-                                          const Tb2Bufs<RY>& b, Tb2Carry& s, bool valid, bool issue_next,
-                                          float dt16, int u)
+// x-shell psi of the pair stored from values v (offset q of the first column;
+// xpair: the pair lies in the shell as a whole, at an even offset).
+__device__ __forceinline__ void st_psix(float* p, int q, float2 v, bool w0, bool w1, bool xpair, uint64_t pol)
+{
+    if (xpair) {
+        if (w0) st_keep(reinterpret_cast<float2*>(p + q), v, pol);
+        return;
+    }
+    if (w0) st_keep(p + q, v.x, pol);
+    if (w1) st_keep(p + q + 1, v.y, pol);
+}
+
+// A pair of row-contiguous values at element q of p (q even).
+__device__ __forceinline__ void st_pair(float* p, int q, float2 v, bool w0, bool w1, uint64_t pol)
+{
+    if (w1) st_keep(reinterpret_cast<float2*>(p + q), v, pol);
+    else if (w0) st_keep(p + q, v.x, pol);
+}
+
+// z-shell index of plane k, or -1.
+__device__ __forceinline__ int tb2_zshell(const StepArgs<float>& a, int k)
+{
+    if (k < 0 || k >= a.nz) return -1;
+    return k < a.npz ? k : (k >= a.nz - a.npz ? k - a.nz + 2 * a.npz : -1);
+}
+
+// z-shell psi update of a pair of columns: the value read from array t.
+__device__ __forceinline__ float2 tb2_ldz(const float* t, const StepArgs<float>& a, const Tb2Col& c, int kk)
+{
+    const float* q = t + (long long)kk * (a.pitch * a.ny) + c.col;
+    return make_float2(c.in0 ? q[0] : 0.0f, c.in1 ? q[1] : 0.0f);
+}
+
+// The wall sheet's E_x increment at the pair's columns.
+__device__ __forceinline__ float2 tb2_sheet(const StepArgs<float>& a, const Tb2Col& c, Cpx<float> tw)
+{
+    const Cpx<float>* t = static_cast<const Cpx<float>*>(a.wcoefr) + c.j * a.nx + c.i;
+    const Cpx<float> zero{0.0f, 0.0f}, w0 = c.in0 ? t[0] : zero, w1 = c.in1 ? t[1] : zero;
+    return make_float2(fma_rn(w0.x, tw.x, -mul_rn(w0.y, tw.y)), fma_rn(w1.x, tw.x, -mul_rn(w1.y, tw.y)));
+}
+
+// One plane p of the wavefront: u = ring slot of plane p, U = (p - P0) mod 2
+// gives the exchange-buffer parities at compile time.  Every row runs every
+// stage: a row whose results no written column needs computes values that
+// reach no output (rows beyond the window read the zero rows of the exchange
+// arrays), and the stage code stays free of branches.
+// W: 1, the z walls and the wall sheet compiled in; 2, the z CPML too (planes
+// of the z shells).  valid: plane p-2's fields are the range's to store; okF:
+// plane p-3's fluence.
+//
+// The walls: E_x and E_y are zero on the planes 0 and nz (plane nz reads as
+// zeros; its E^{n+1} is set to zero here), and with that no value of a plane
+// below 0 or above nz reaches a stored one.
+template <int RY, int U, int G, int W, bool CR>
+__device__ __forceinline__ void tb2_plane(const StepArgs<float>& a, const TmaMaps& m, const Tb2Times& tt,
+                                          const Tb2Col& c, const Tb2Bufs<RY>& b, Tb2Carry& s, bool valid, bool okF,
+                                          bool issue_next, bool issue_psi, float dt16, uint32_t gq, int wx0, int wy0, bool& dead)
 {
     using S = Tb2Smem<RY>;
-    constexpr int NT = S::NT, NF = S::NF, XS = S::XS;
+    constexpr int NC = S::NC, XS = S::XS;
     constexpr bool GX = G & 1, GY = G & 2;
-    const int SP = u, SQ = (u + 3) & 3, SR = (u + 2) & 3;   // slots of planes p, p-1, p-2
-    constexpr int PP = U & 1, PQ = PP ^ 1;                        // exchange parities of planes p, p-1
-    const int lane = c.lane, tid = c.tid;
-    // (a window off the x faces, !GX, takes the edge lane's own value past
-    // the window: lanes 0 and 31 are halo there, and what they compute
-    // reaches no column the window writes)
-    auto xp = [&](float v) {   // value of the +x neighbour (0 past the window)
-        const float u = __shfl_down_sync(0xffffffffu, v, 1);
-        return GX && lane == 31 ? 0.0f : u;
+    const uint32_t SP = gq & 3, SQ = (gq + 3) & 3;                 // ring slots of planes p, p-1
+    constexpr int PP = U & 1, PQ = PP ^ 1;                         // exchange parities of planes p, p-1
+    // (past the window's edge: the edge column's own value; a column so
+    // computed is halo and reaches no column the window writes)
+    auto xp = [&](float2 v) {   // value of the +x neighbours
+        float w = __shfl_down_sync(0xffffffffu, v.x, 1, 16);
+        return make_float2(v.y, w);
     };
-    auto xm = [&](float v) {   // value of the -x neighbour
-        const float u = __shfl_up_sync(0xffffffffu, v, 1);
-        return GX && lane == 0 ? 0.0f : u;
+    auto xm = [&](float2 v) {   // value of the -x neighbours
+        float w = __shfl_up_sync(0xffffffffu, v.y, 1, 16);
+        return make_float2(w, v.x);
     };
-    // y neighbours from the padded exchange arrays (zero beyond the window)
-    auto yp = [&](const float* q) { return q[S::XO + tid + 32]; };
-    auto ym = [&](const float* q) { return q[S::XO + tid - 32]; };
-    auto put = [&](float* q, float v) { q[S::XO + tid] = v; };
-    const float cz = a.cz;
+    // y neighbours from the exchange arrays (past the window's rows: another
+    // array's row, for halo rows only)
+    auto yp = [&](const float* q) { return ld2(q + S::XO + c.at + 32); };
+    auto ym = [&](const float* q) { return ld2(q + S::XO + c.at - 32); };
+    auto put = [&](float* q, float2 v) { st2(q + S::XO + c.at, v); };
+    // +y neighbour of E^n from the ring
+    auto ype = [&](const float* q) { return ld2(q + c.at + 32); };
+    const float2 cz = dup2(a.cz);
+    // dt / (kappa dz) at the H and E positions of planes p-1 and p-2
+    auto czat = [&](const float* t, int k) { return W == 2 ? dup2(t[min(max(k, 0), a.nz - 1)]) : cz; };
+    const float2 czh = czat(a.chz, s.kq), cze = czat(a.cez, s.kq), czh1 = czat(a.chz, s.kr), cze1 = czat(a.cez, s.kr);
+    const float2 zero2 = make_float2(0.0f, 0.0f);
+    const int zsq = W == 2 ? tb2_zshell(a, s.kq) : -1, zsr = W == 2 ? tb2_zshell(a, s.kr) : -1;
+    // the z-shell psi: of plane p-1 read ahead of the wait below, updated by
+    // step n into this thread's place in shared memory (the antenna's, which
+    // z-walled grids do not have), from there by step n+1 one plane later
+    float2 ipz[4] = {zero2, zero2, zero2, zero2};
+    if (W == 2 && zsq >= 0) {
+        ipz[0] = tb2_ldz(a.phz_in[0], a, c, zsq); ipz[1] = tb2_ldz(a.phz_in[1], a, c, zsq);
+        ipz[2] = tb2_ldz(a.pez[0], a, c, zsq); ipz[3] = tb2_ldz(a.pez[1], a, c, zsq);
+    }
+    float* zw = b.SC + PP * 4 * NC + c.at;         // psi of plane p-1 after step n: Hxz Hyz Exz Eyz
+    const float* zr = b.SC + PQ * 4 * NC + c.at;   // of plane p-2
 
-    cpa_wait2();   // this plane's fields and the last plane's psi (planes p + 1, p + 2 may still run)
-    float* rp = b.ring + SP * NF * NT + tid;
-    float* rq = b.ring + SQ * NF * NT + tid;
-    float* rr = b.ring + SR * NF * NT + tid;
+    if (!dead && !mbar_wait_bounded(b.bars + SP, (gq >> 2) & 1)) {
+        dead = true;
+        atomicOr(b.err, 1);
+    }
+    if (GX || GY) cpa_wait1();                                       // and the last plane's psi
+    const float* rp = b.ring + SP * S::SLOT + c.at;
+    const float* rq = b.ring + SQ * S::SLOT;
+    float* ps = b.psi + PQ * S::NP * NC + c.at;                      // psi of plane p-1
     // e^{i beta z} of plane p, used from the next plane on
     Cpx<float> zn{0.0f, 0.0f};
     if (c.ant) zn = static_cast<const Cpx<float>*>(a.zphr)[s.kp];
 
     // ---- stage A: H^{n+1/2} of plane q = p-1
-    const float en0 = rp[0], en1 = rp[NT], en2 = rp[2 * NT];         // E^n(p)
-    const float ex = s.e0[0], ey = s.e0[1], ez = s.e0[2];
-    float hx = 0.0f, hy = 0.0f, hz = 0.0f, hsy = 0.0f;
-    float nPEx = 0.0f, nPEy = 0.0f, ncz = 0.0f, nHsz = 0.0f, nhbx = 0.0f;
+    const float2 en0 = ld2(rp), en1 = ld2(rp + NC), en2 = ld2(rp + 2 * NC);   // E^n(p)
+    const float2 ex = s.e0[0], ey = s.e0[1], ez = s.e0[2];
+    float2 hx, hy, hz, hsy, npx[4], npy[4];
+    float2 nPEx, nPEy, ncz, nHsz, nhbx;
     {
-        const float ox = rq[3 * NT], oy = rq[4 * NT], oz = rq[5 * NT];   // H^{n-1/2}(q)
-        const float* EBq = b.EB + PQ * 2 * XS;
-        const float ezj = yp(EBq), exj = yp(EBq + XS);
-        const float ezi = xp(ez), eyi = xp(ey);
-        const float dEz_y = ezj - ez, dEy_z = en1 - ey, dEx_z = en0 - ex;
-        const float dEz_x = ezi - ez, dEy_x = eyi - ey, dEx_y = exj - ex;
-        hx = ox - c.chy * dEz_y + cz * dEy_z;
-        hy = oy - cz * dEx_z + c.chx * dEz_x;
-        hz = oz - c.chx * dEy_x + c.chy * dEx_y;
+        const float2 ox = ld2(rq + 3 * NC + c.at), oy = ld2(rq + 4 * NC + c.at), oz = ld2(rq + 5 * NC + c.at);
+        const float2 ezj = ype(rq + 2 * NC), exj = ype(rq);
+        const float2 ezi = xp(ez), eyi = xp(ey);
+        const float2 dEz_y = sub2(ezj, ez), dEy_z = sub2(en1, ey), dEx_z = sub2(en0, ex);
+        const float2 dEz_x = sub2(ezi, ez), dEy_x = sub2(eyi, ey), dEx_y = sub2(exj, ex);
+        hx = fma2(czh, dEy_z, fma2(neg2(c.chy), dEz_y, ox));
+        hy = fma2(c.chx, dEz_x, fma2(neg2(czh), dEx_z, oy));
+        hz = fma2(c.chy, dEx_y, fma2(neg2(c.chx), dEy_x, oz));
         if (GX) {   // every lane (zero coefficients and psi off the x shells)
-            const float p0 = psi_rn(c.bhx, rq[6 * NT], c.ahx, dEz_x);   // Hyx
-            const float p1 = psi_rn(c.bhx, rq[7 * NT], c.ahx, dEy_x);   // Hzx
-            hy += p0;
-            hz -= p1;
-            rq[6 * NT] = p0; rq[7 * NT] = p1;
+            npx[0] = psi2<CR>(c.bhx, ld2(ps + 0 * NC), c.ahx, dEz_x);   // Hyx
+            npx[1] = psi2<CR>(c.bhx, ld2(ps + 1 * NC), c.ahx, dEy_x);   // Hzx
+            hy = add2(hy, npx[0]);
+            hz = sub2(hz, npx[1]);
         }
-        if (GY && c.sy) {
-            const float p0 = psi_rn(c.bhy, rq[8 * NT], c.ahy, dEz_y);   // Hxy
-            const float p1 = psi_rn(c.bhy, rq[9 * NT], c.ahy, dEx_y);   // Hzy
-            hx -= p0;
-            hz += p1;
-            rq[8 * NT] = p0; rq[9 * NT] = p1;
+        if (GY) {
+            npy[0] = psi2<CR>(c.bhy, ld2(ps + 2 * NC), c.ahy, dEz_y);   // Hxy
+            npy[1] = psi2<CR>(c.bhy, ld2(ps + 3 * NC), c.ahy, dEx_y);   // Hzy
+            hx = sub2(hx, npy[0]);
+            hz = add2(hz, npy[1]);
         }
-        if (c.anth) {   // the whole row: zero terms where a column has no point
+        if (W == 2 && zsq >= 0) {
+            const float2 bz = dup2(a.bhz[zsq]), az = dup2(a.ahz[zsq]);
+            const float2 p0 = psi2<CR>(bz, ipz[0], az, dEy_z);   // Hxz
+            const float2 p1 = psi2<CR>(bz, ipz[1], az, dEx_z);   // Hyz
+            hx = add2(hx, p0);
+            hy = sub2(hy, p1);
+            st2(zw, p0);
+            st2(zw + NC, p1);
+        }
+        if (c.anth) {   // the whole warp: zero terms where a column has no point
             const Cpx<float> u = cmul(s.zq, tt.th0);
-            hx += tb2_src(b, c, 3, u);
-            hy += tb2_src(b, c, 4, u);
-            hz += tb2_src(b, c, 5, u);
+            hx = add2(hx, tb2_src(b, c, 3, u));
+            hy = add2(hy, tb2_src(b, c, 4, u));
+            hz = add2(hz, tb2_src(b, c, 5, u));
         }
         // centre sums of step n for plane q
-        nPEx = ex + exj;
-        nPEy = ey + eyi;
-        ncz = (ez + ezi) + (ezj + xp(ezj));
-        const float hsx = ox + hx;
-        hsy = oy + hy;
-        nHsz = oz + hz;
-        nhbx = hsx + xp(hsx);
+        nPEx = add2(ex, exj);
+        nPEy = add2(ey, eyi);
+        ncz = add2(add2(ez, ezi), add2(ezj, xp(ezj)));
+        const float2 hsx = add2(ox, hx);
+        hsy = add2(oy, hy);
+        nHsz = add2(oz, hz);
+        nhbx = add2(hsx, xp(hsx));
     }
-    {
-        float* EBp = b.EB + PP * 2 * XS;
-        put(EBp, en2);
-        put(EBp + XS, en0);
-        put(b.HB, hx);
-        put(b.HB + XS, hz);
-        put(b.HB + 2 * XS, hsy);
-    }
-    __syncthreads();
+    put(b.HB, hx);
+    put(b.HB + XS, hz);
+    put(b.HB + 2 * XS, hsy);
+    __syncthreads();   // H^{n+1/2} of plane q is there, and every read of ring slot SQ is done
+    // refill: the boxes of the iteration of plane p + 3 into the slot of p - 1
+    if (issue_next) tb2_issue<RY>(a, m, b, SQ, s.ki, s.kp, wx0, wy0);
 
     // ---- stage B: E^{n+1} of plane q
-    float nex = 0.0f, ney = 0.0f, nez = 0.0f;
+    float2 nex, ney, nez;
     {
-        const float hyi = xm(hy), hzi = xm(hz);
-        const float hxj = ym(b.HB), hzj = ym(b.HB + XS);
-        const float dHz_y = hz - hzj, dHy_z = hy - s.h1p[1], dHx_z = hx - s.h1p[0];
-        const float dHz_x = hz - hzi, dHy_x = hy - hyi, dHx_y = hx - hxj;
-        nex = ex + c.cey * dHz_y - cz * dHy_z;
-        ney = ey + cz * dHx_z - c.cex * dHz_x;
-        nez = ez + c.cex * dHy_x - c.cey * dHx_y;
+        const float2 hyi = xm(hy), hzi = xm(hz);
+        const float2 hxj = ym(b.HB), hzj = ym(b.HB + XS);
+        const float2 dHz_y = sub2(hz, hzj), dHy_z = sub2(hy, s.h1p[1]), dHx_z = sub2(hx, s.h1p[0]);
+        const float2 dHz_x = sub2(hz, hzi), dHy_x = sub2(hy, hyi), dHx_y = sub2(hx, hxj);
+        nex = fma2(neg2(cze), dHy_z, fma2(c.cey, dHz_y, ex));
+        ney = fma2(neg2(c.cex), dHz_x, fma2(cze, dHx_z, ey));
+        nez = fma2(neg2(c.cey), dHx_y, fma2(c.cex, dHy_x, ez));
         if (GX) {   // every lane (zero coefficients and psi off the x shells)
-            const float p0 = psi_rn(c.bex, rq[10 * NT], c.aex, dHz_x);   // Eyx
-            const float p1 = psi_rn(c.bex, rq[11 * NT], c.aex, dHy_x);   // Ezx
-            rq[10 * NT] = p0; rq[11 * NT] = p1;
-            ney -= p0;
-            nez += p1;
+            npx[2] = psi2<CR>(c.bex, ld2(ps + 4 * NC), c.aex, dHz_x);   // Eyx
+            npx[3] = psi2<CR>(c.bex, ld2(ps + 5 * NC), c.aex, dHy_x);   // Ezx
+            ney = sub2(ney, npx[2]);
+            nez = add2(nez, npx[3]);
         }
-        if (GY && c.sy) {
-            const float p0 = psi_rn(c.bey, rq[12 * NT], c.aey, dHz_y);   // Exy
-            const float p1 = psi_rn(c.bey, rq[13 * NT], c.aey, dHx_y);   // Ezy
-            rq[12 * NT] = p0; rq[13 * NT] = p1;
-            nex += p0;
-            nez -= p1;
+        if (GY) {
+            npy[2] = psi2<CR>(c.bey, ld2(ps + 6 * NC), c.aey, dHz_y);   // Exy
+            npy[3] = psi2<CR>(c.bey, ld2(ps + 7 * NC), c.aey, dHx_y);   // Ezy
+            nex = add2(nex, npy[2]);
+            nez = sub2(nez, npy[3]);
         }
-        if (c.ante) {   // the whole row: zero terms where a column has no point
+        if (W == 2 && zsq >= 0) {
+            const float2 bz = dup2(a.bez[zsq]), az = dup2(a.aez[zsq]);
+            const float2 p0 = psi2<CR>(bz, ipz[2], az, dHy_z);   // Exz
+            const float2 p1 = psi2<CR>(bz, ipz[3], az, dHx_z);   // Eyz
+            nex = sub2(nex, p0);
+            ney = add2(ney, p1);
+            st2(zw + 2 * NC, p0);
+            st2(zw + 3 * NC, p1);
+        }
+        if (c.ante) {   // the whole warp: zero terms where a column has no point
             const Cpx<float> u = cmul(s.zq, tt.te0);
-            nex += tb2_src(b, c, 0, u);
-            ney += tb2_src(b, c, 1, u);
-            nez += tb2_src(b, c, 2, u);
+            nex = add2(nex, tb2_src(b, c, 0, u));
+            ney = add2(ney, tb2_src(b, c, 1, u));
+            nez = add2(nez, tb2_src(b, c, 2, u));
         }
-        if (GY && c.j == 0) { nex = 0.0f; nez = 0.0f; }   // PEC: tangential E
-        if (GX && c.i == 0) { ney = 0.0f; nez = 0.0f; }
+        if (W && a.wcoefr && s.kq == a.wplane) nex = add2(nex, tb2_sheet(a, c, tt.tw0));
+        if (GY && c.j == 0) { nex = zero2; nez = zero2; }   // PEC: tangential E
+        if (GX && c.i == 0) { ney.x = 0.0f; nez.x = 0.0f; }
+        if (W && a.zw && (s.kq == 0 || s.kq == a.nz)) nex = ney = zero2;
     }
-    // fluence term of step n for plane r (sums of planes r and q)
-    float nhby = 0.0f, tn_new = 0.0f;
-    {
-        nhby = hsy + yp(b.HB + 2 * XS);
-        tn_new = tb2_flux(s.fPEx + nPEx, s.fPEy + nPEy, s.fcz, s.fhbx, s.fhby, s.fHsz + nHsz, dt16);
+    // the psi of plane p + 1 into the slot of p - 1 (read above)
+    if (GX || GY) {
+        if (issue_psi) tb2_issue_psi<RY, G, W != 0>(a, c, b, PQ, tb2_next<W != 0>(a, s.kp));
+        else cpa_commit();
     }
+    // fluence term of step n for plane r = p-2 (sums of planes r and q)
+    const float2 nhby = add2(hsy, yp(b.HB + 2 * XS));
+    const float2 tn_new = tb2_flux<CR>(add2(s.fPEx, nPEx), add2(s.fPEy, nPEy), s.fcz, s.fhbx, s.fhby, add2(s.fHsz, nHsz),
+                                   dt16);
 
-    // ---- stage C: H^{n+3/2} of plane r = p-2
-    float h2x = 0.0f, h2y = 0.0f, h2z = 0.0f, gsy = 0.0f;
-    float mPEx = 0.0f, mPEy = 0.0f, mcz = 0.0f, mHsz = 0.0f, mhbx = 0.0f;
+    // ---- stage C: H^{n+3/2} of plane r
+    float2 h2x, h2y, h2z, gsy;
+    float2 mPEx, mPEy, mcz, mHsz, mhbx;
     {
         const float* E1Br = b.E1B + PP * 2 * XS;   // written one plane ago (parity of r = parity of p)
-        const float fezj = yp(E1Br), fexj = yp(E1Br + XS);
-        const float fezi = xp(s.e1p[2]), feyi = xp(s.e1p[1]);
-        const float dEz_y = fezj - s.e1p[2], dEy_z = ney - s.e1p[1], dEx_z = nex - s.e1p[0];
-        const float dEz_x = fezi - s.e1p[2], dEy_x = feyi - s.e1p[1], dEx_y = fexj - s.e1p[0];
-        h2x = s.h1p[0] - c.chy * dEz_y + cz * dEy_z;
-        h2y = s.h1p[1] - cz * dEx_z + c.chx * dEz_x;
-        h2z = s.h1p[2] - c.chx * dEy_x + c.chy * dEx_y;
+        const float2 fezj = yp(E1Br), fexj = yp(E1Br + XS);
+        const float2 fezi = xp(s.e1p[2]), feyi = xp(s.e1p[1]);
+        const float2 dEz_y = sub2(fezj, s.e1p[2]), dEy_z = sub2(ney, s.e1p[1]), dEx_z = sub2(nex, s.e1p[0]);
+        const float2 dEz_x = sub2(fezi, s.e1p[2]), dEy_x = sub2(feyi, s.e1p[1]), dEx_y = sub2(fexj, s.e1p[0]);
+        h2x = fma2(czh1, dEy_z, fma2(neg2(c.chy), dEz_y, s.h1p[0]));
+        h2y = fma2(c.chx, dEz_x, fma2(neg2(czh1), dEx_z, s.h1p[1]));
+        h2z = fma2(c.chy, dEx_y, fma2(neg2(c.chx), dEy_x, s.h1p[2]));
         if (GX) {   // every lane (zero coefficients and psi off the x shells)
-            const float p0 = psi_rn(c.bhx, rr[6 * NT], c.ahx, dEz_x);
-            const float p1 = psi_rn(c.bhx, rr[7 * NT], c.ahx, dEy_x);
-            h2y += p0;
-            h2z -= p1;
-            if (valid && c.own && c.sx) {
+            const float2 p0 = psi2<CR>(c.bhx, s.px[0], c.ahx, dEz_x);
+            const float2 p1 = psi2<CR>(c.bhx, s.px[1], c.ahx, dEy_x);
+            h2y = add2(h2y, p0);
+            h2z = sub2(h2z, p1);
+            if (valid && (c.sx0 || c.sx1)) {
                 const int qo = s.kr * a.ny * (2 * a.npml) + c.colx;
-                const uint64_t pol = tb2_store_policy();
-                st_keep(a.phx_out[0] + qo, p0, pol); st_keep(a.phx_out[1] + qo, p1, pol);
+                const uint64_t pol = b.pol;
+                st_psix(a.phx_out[0], qo, p0, c.own0 && c.sx0, c.own1 && c.sx1, c.xpair, pol);
+                st_psix(a.phx_out[1], qo, p1, c.own0 && c.sx0, c.own1 && c.sx1, c.xpair, pol);
             }
         }
-        if (GY && c.sy) {
-            const float p0 = psi_rn(c.bhy, rr[8 * NT], c.ahy, dEz_y);
-            const float p1 = psi_rn(c.bhy, rr[9 * NT], c.ahy, dEx_y);
-            h2x -= p0;
-            h2z += p1;
-            if (valid && c.own) {
+        if (GY) {
+            const float2 p0 = psi2<CR>(c.bhy, s.py[0], c.ahy, dEz_y);
+            const float2 p1 = psi2<CR>(c.bhy, s.py[1], c.ahy, dEx_y);
+            h2x = sub2(h2x, p0);
+            h2z = add2(h2z, p1);
+            if (valid && c.sy) {
                 const int qo = s.kr * (2 * a.npml) * a.pitch + c.coly;
-                const uint64_t pol = tb2_store_policy();
-                st_keep(a.phy_out[0] + qo, p0, pol); st_keep(a.phy_out[1] + qo, p1, pol);
+                const uint64_t pol = b.pol;
+                st_pair(a.phy_out[0], qo, p0, c.own0, c.own1, pol);
+                st_pair(a.phy_out[1], qo, p1, c.own0, c.own1, pol);
             }
         }
-        if (c.anth) {   // the whole row: zero terms where a column has no point
+        if (W == 2 && zsr >= 0) {
+            const float2 bz = dup2(a.bhz[zsr]), az = dup2(a.ahz[zsr]);
+            const float2 p0 = psi2<CR>(bz, ld2(zr), az, dEy_z), p1 = psi2<CR>(bz, ld2(zr + NC), az, dEx_z);
+            h2x = add2(h2x, p0);
+            h2y = sub2(h2y, p1);
+            if (valid) {
+                const int qo = zsr * (a.pitch * a.ny) + c.col;
+                st_pair(a.phz_out[0], qo, p0, c.own0, c.own1, b.pol);
+                st_pair(a.phz_out[1], qo, p1, c.own0, c.own1, b.pol);
+            }
+        }
+        if (c.anth) {   // the whole warp: zero terms where a column has no point
             const Cpx<float> u = cmul(s.zr, tt.th1);
-            h2x += tb2_src(b, c, 3, u);
-            h2y += tb2_src(b, c, 4, u);
-            h2z += tb2_src(b, c, 5, u);
+            h2x = add2(h2x, tb2_src(b, c, 3, u));
+            h2y = add2(h2y, tb2_src(b, c, 4, u));
+            h2z = add2(h2z, tb2_src(b, c, 5, u));
         }
         // centre sums of step n+1 for plane r
-        mPEx = s.e1p[0] + fexj;
-        mPEy = s.e1p[1] + feyi;
-        mcz = (s.e1p[2] + fezi) + (fezj + xp(fezj));
-        const float gsx = s.h1p[0] + h2x;
-        gsy = s.h1p[1] + h2y;
-        mHsz = s.h1p[2] + h2z;
-        mhbx = gsx + xp(gsx);
+        mPEx = add2(s.e1p[0], fexj);
+        mPEy = add2(s.e1p[1], feyi);
+        mcz = add2(add2(s.e1p[2], fezi), add2(fezj, xp(fezj)));
+        const float2 gsx = add2(s.h1p[0], h2x);
+        gsy = add2(s.h1p[1], h2y);
+        mHsz = add2(s.h1p[2], h2z);
+        mhbx = add2(gsx, xp(gsx));
     }
     {
         float* E1Bq = b.E1B + PQ * 2 * XS;
@@ -488,60 +656,93 @@ __device__ __forceinline__ void tb2_plane(const StepArgs<float>& a, const Tb2Tim
 
     // ---- stage D: E^{n+2} of plane r
     {
-        const float hyi = xm(h2y), hzi = xm(h2z);
-        const float hxj = ym(b.H1B), hzj = ym(b.H1B + XS);
-        const float dHz_y = h2z - hzj, dHy_z = h2y - s.h2py, dHx_z = h2x - s.h2px;
-        const float dHz_x = h2z - hzi, dHy_x = h2y - hyi, dHx_y = h2x - hxj;
-        float fx = s.e1p[0] + c.cey * dHz_y - cz * dHy_z;
-        float fy = s.e1p[1] + cz * dHx_z - c.cex * dHz_x;
-        float fz = s.e1p[2] + c.cex * dHy_x - c.cey * dHx_y;
+        const float2 hyi = xm(h2y), hzi = xm(h2z);
+        const float2 hxj = ym(b.H1B), hzj = ym(b.H1B + XS);
+        const float2 dHz_y = sub2(h2z, hzj), dHy_z = sub2(h2y, s.h2py), dHx_z = sub2(h2x, s.h2px);
+        const float2 dHz_x = sub2(h2z, hzi), dHy_x = sub2(h2y, hyi), dHx_y = sub2(h2x, hxj);
+        float2 fx = fma2(neg2(cze1), dHy_z, fma2(c.cey, dHz_y, s.e1p[0]));
+        float2 fy = fma2(neg2(c.cex), dHz_x, fma2(cze1, dHx_z, s.e1p[1]));
+        float2 fz = fma2(neg2(c.cey), dHx_y, fma2(c.cex, dHy_x, s.e1p[2]));
         if (GX) {   // every lane (zero coefficients and psi off the x shells)
-            const float p0 = psi_rn(c.bex, rr[10 * NT], c.aex, dHz_x);
-            const float p1 = psi_rn(c.bex, rr[11 * NT], c.aex, dHy_x);
-            fy -= p0;
-            fz += p1;
-            if (valid && c.own && c.sx) {
+            const float2 p0 = psi2<CR>(c.bex, s.px[2], c.aex, dHz_x);
+            const float2 p1 = psi2<CR>(c.bex, s.px[3], c.aex, dHy_x);
+            fy = sub2(fy, p0);
+            fz = add2(fz, p1);
+            if (valid && (c.sx0 || c.sx1)) {
                 const int qo = s.kr * a.ny * (2 * a.npml) + c.colx;
-                const uint64_t pol = tb2_store_policy();
-                st_keep(a.pex_out[0] + qo, p0, pol); st_keep(a.pex_out[1] + qo, p1, pol);
+                const uint64_t pol = b.pol;
+                st_psix(a.pex_out[0], qo, p0, c.own0 && c.sx0, c.own1 && c.sx1, c.xpair, pol);
+                st_psix(a.pex_out[1], qo, p1, c.own0 && c.sx0, c.own1 && c.sx1, c.xpair, pol);
             }
         }
-        if (GY && c.sy) {
-            const float p0 = psi_rn(c.bey, rr[12 * NT], c.aey, dHz_y);
-            const float p1 = psi_rn(c.bey, rr[13 * NT], c.aey, dHx_y);
-            fx += p0;
-            fz -= p1;
-            if (valid && c.own) {
+        if (GY) {
+            const float2 p0 = psi2<CR>(c.bey, s.py[2], c.aey, dHz_y);
+            const float2 p1 = psi2<CR>(c.bey, s.py[3], c.aey, dHx_y);
+            fx = add2(fx, p0);
+            fz = sub2(fz, p1);
+            if (valid && c.sy) {
                 const int qo = s.kr * (2 * a.npml) * a.pitch + c.coly;
-                const uint64_t pol = tb2_store_policy();
-                st_keep(a.pey_out[0] + qo, p0, pol); st_keep(a.pey_out[1] + qo, p1, pol);
+                const uint64_t pol = b.pol;
+                st_pair(a.pey_out[0], qo, p0, c.own0, c.own1, pol);
+                st_pair(a.pey_out[1], qo, p1, c.own0, c.own1, pol);
             }
         }
-        if (c.ante) {   // the whole row: zero terms where a column has no point
-            const Cpx<float> u = cmul(s.zr, tt.te1);
-            fx += tb2_src(b, c, 0, u);
-            fy += tb2_src(b, c, 1, u);
-            fz += tb2_src(b, c, 2, u);
+        if (W == 2 && zsr >= 0) {
+            const float2 bz = dup2(a.bez[zsr]), az = dup2(a.aez[zsr]);
+            const float2 p0 = psi2<CR>(bz, ld2(zr + 2 * NC), az, dHy_z), p1 = psi2<CR>(bz, ld2(zr + 3 * NC), az, dHx_z);
+            fx = sub2(fx, p0);
+            fy = add2(fy, p1);
+            if (valid) {
+                const int qo = zsr * (a.pitch * a.ny) + c.col;
+                st_pair(a.pez_out[0], qo, p0, c.own0, c.own1, b.pol);
+                st_pair(a.pez_out[1], qo, p1, c.own0, c.own1, b.pol);
+            }
         }
-        if (GY && c.j == 0) { fx = 0.0f; fz = 0.0f; }
-        if (GX && c.i == 0) { fy = 0.0f; fz = 0.0f; }
-        if (valid && c.own) {
+        if (c.ante) {   // the whole warp: zero terms where a column has no point
+            const Cpx<float> u = cmul(s.zr, tt.te1);
+            fx = add2(fx, tb2_src(b, c, 0, u));
+            fy = add2(fy, tb2_src(b, c, 1, u));
+            fz = add2(fz, tb2_src(b, c, 2, u));
+        }
+        if (W && a.wcoefr && s.kr == a.wplane) fx = add2(fx, tb2_sheet(a, c, tt.tw1));
+        if (GY && c.j == 0) { fx = zero2; fz = zero2; }
+        if (GX && c.i == 0) { fy.x = 0.0f; fz.x = 0.0f; }
+        if (W && a.zw && s.kr == 0) fx = fy = zero2;
+        if (valid && c.own0) {
             const int g = s.kr * (a.pitch * a.ny) + c.col;
-            const uint64_t pol = tb2_store_policy();
-            st_keep(a.eout[0] + g, fx, pol); st_keep(a.eout[1] + g, fy, pol); st_keep(a.eout[2] + g, fz, pol);
-            st_keep(a.hout[0] + g, h2x, pol); st_keep(a.hout[1] + g, h2y, pol); st_keep(a.hout[2] + g, h2z, pol);
+            const uint64_t pol = b.pol;
+            const bool w1 = !GX || c.own1;   // off the x faces the window writes whole pairs
+            st_pair(a.eout[0], g, fx, true, w1, pol);
+            st_pair(a.eout[1], g, fy, true, w1, pol);
+            st_pair(a.eout[2], g, fz, true, w1, pol);
+            st_pair(a.hout[0], g, h2x, true, w1, pol);
+            st_pair(a.hout[1], g, h2y, true, w1, pol);
+            st_pair(a.hout[2], g, h2z, true, w1, pol);
         }
     }
     // fluence of plane p-3: the step-n term from the last plane, then step n+1
-    float mhby = 0.0f;
+    const float2 mhby = add2(gsy, yp(b.H1B + 2 * XS));
     {   // every lane computes it (no divergent branch); the fluence cells store it
-        mhby = gsy + yp(b.H1B + 2 * XS);
-        const float t1 = tb2_flux(s.gPEx + mPEx, s.gPEy + mPEy, s.gcz, s.ghbx, s.ghby, s.gHsz + mHsz, dt16);
-        float2 acc = b.fring[SP * NT + tid];   // zero-filled off the fluence cells
-        acc = FluAcc<float>::add(acc, s.tn);
-        acc = FluAcc<float>::add(acc, t1);
-        if (valid && c.fown)
-            st_keep(static_cast<float2*>(a.fluence) + s.k3 * (a.pitch * a.ny) + c.col, acc, tb2_store_policy());
+        const float2 t1 = tb2_flux<CR>(add2(s.gPEx, mPEx), add2(s.gPEy, mPEy), s.gcz, s.ghbx, s.ghby, add2(s.gHsz, mHsz),
+                                   dt16);
+        const float4 f = *reinterpret_cast<const float4*>(b.ring + SP * S::SLOT + 6 * NC + 2 * c.at);
+        // FluAcc<float>::add (CR: add_fma), twice
+        float2 sum = make_float2(f.x, f.z), comp = make_float2(f.y, f.w);
+        #pragma unroll
+        for (int n = 0; n < 2; ++n) {
+            const float2 v = n == 0 ? s.tn : t1;
+            const float2 y = CR ? fma2(v, dup2(dt16), neg2(comp)) : sub2(v, comp);
+            const float2 t = add2(sum, y);
+            comp = sub2(sub2(t, sum), y);
+            sum = t;
+        }
+        if (okF) {
+            float2* F = static_cast<float2*>(a.fluence) + (s.k3 * (a.pitch * a.ny) + c.col);
+            const uint64_t pol = b.pol;
+            if (GX ? c.f1 : c.f0)
+                st_keep(reinterpret_cast<float4*>(F), make_float4(sum.x, comp.x, sum.y, comp.y), pol);
+            else if (GX && c.f0) st_keep(F, make_float2(sum.x, comp.x), pol);
+        }
     }
 
     // ---- carry to the next plane
@@ -552,119 +753,201 @@ __device__ __forceinline__ void tb2_plane(const StepArgs<float>& a, const Tb2Tim
     s.fPEx = nPEx; s.fPEy = nPEy; s.fcz = ncz; s.fhbx = nhbx; s.fhby = nhby; s.fHsz = nHsz;
     s.gPEx = mPEx; s.gPEy = mPEy; s.gcz = mcz; s.ghbx = mhbx; s.ghby = mhby; s.gHsz = mHsz;
     s.tn = tn_new;
+    #pragma unroll
+    for (int v = 0; v < 4; ++v) {
+        if (GX) s.px[v] = npx[v];
+        if (GY) s.py[v] = npy[v];
+    }
     s.zr = s.zq; s.zq = zn;
-    // refill: the fields of plane p + 3 (fluence plane p) into the slot of
-    // plane p - 1, whose fields were last read at this plane's stage A, and
-    // the psi of plane p + 2 into the slot of plane p - 2, whose psi were last
-    // read at this plane's stage D
-    if (issue_next) tb2_issue<RY, G>(a, c, b, SQ, s.ki, s.kp, SR, next_plane(next_plane(s.kp, a.nz), a.nz));
-    else cpa_commit();
     s.k3 = s.kr; s.kr = s.kq; s.kq = s.kp;
-    s.kp = next_plane(s.kp, a.nz);
-    s.ki = next_plane(s.ki, a.nz);
+    s.kp = tb2_next<W != 0>(a, s.kp);
+    s.ki = tb2_next<W != 0>(a, s.ki);
+}
+
+// A plane p whose planes p-1 and p-2 lie off the z shells.
+__device__ __forceinline__ bool tb2_plain(const StepArgs<float>& a, const Tb2Carry& s)
+{
+    return a.npz == 0 || (s.kr >= a.npz && s.kq < a.nz - a.npz);
 }
 
 // One window, planes [kb, ke) of its E^{n+2} / H^{n+3/2} output (fluence
-// planes [kb-1, ke-1), modulo nz).
-template <int RY, int G>
-__device__ __forceinline__ void tb2_window(const StepArgs<float>& a, const Tb2Times& tt, const Tb2Plan& tw,
-                                           int window, int kb, int ke, const Tb2Bufs<RY>& b)
+// planes [kb-1, ke-1), modulo nz).  gq counts the CTA's iterations: ring slot
+// gq mod 4, mbarrier parity (gq / 4) mod 2.
+template <int RY, int G, bool W, bool CR>
+__device__ __forceinline__ void tb2_window(const StepArgs<float>& a, const TmaMaps& m, const Tb2Times& tt,
+                                           const Tb2Plan& tw, int window, int kb, int ke, const Tb2Bufs<RY>& b,
+                                           uint32_t& gq, bool& dead)
 {
-    constexpr int NT = Tb2Smem<RY>::NT;
+    using S = Tb2Smem<RY>;
+    constexpr int NC = S::NC;
+    constexpr bool GX = G & 1, GY = G & 2;
     Tb2Col c;
-    c.lane = threadIdx.x; c.row = threadIdx.y; c.tid = c.row * 32 + c.lane;
+    c.l = threadIdx.x & 15; c.row = threadIdx.x >> 4; c.at = c.row * 32 + 2 * c.l;
     const int nx = a.nx, ny = a.ny, nz = a.nz, npml = a.npml, w2 = 2 * npml;
     const int wx = window % tw.T, wy = window / tw.T;
-    const int L0 = kTb2Sx * wx, M0 = (RY - 4) * wy;
-    c.i = L0 + c.lane; c.j = M0 + c.row;
-    c.indom = c.i < nx && c.j < ny;
-    // E^{n+2} / H^{n+3/2} columns this window writes, and its fluence columns
-    const int xa = wx == 0 ? 0 : L0 + 2, xb = wx == tw.T - 1 ? nx : L0 + kTb2Wx - 2;
-    const int ya = wy == 0 ? 0 : M0 + 2, yb = wy == tw.U - 1 ? ny : M0 + RY - 2;
-    c.own = c.i >= xa && c.i < xb && c.j >= ya && c.j < yb;
-    const int fxa = wx == 0 ? 0 : xa - 1, fxb = wx == tw.T - 1 ? nx : xb - 1;
+    const int L0 = kTb2Sx * wx - kTb2Ox, M0 = (RY - 4) * wy - kTb2Oy;
+    c.i = L0 + 2 * c.l; c.j = M0 + c.row;
+    const bool inj = c.j >= 0 && c.j < ny;
+    c.in0 = inj && c.i >= 0 && c.i < nx;
+    c.in1 = inj && c.i >= 0 && c.i + 1 < nx;
+    // E^{n+2} / H^{n+3/2} columns this window writes, and its fluence cells
+    // (the same columns, the rows shifted by -1)
+    const int xa = kTb2Sx * wx, xb = xa + kTb2Sx < nx ? xa + kTb2Sx : nx;
+    const int ya = (RY - 4) * wy, yb = wy == tw.U - 1 ? ny : ya + RY - 4;
     const int fya = wy == 0 ? 0 : ya - 1, fyb = wy == tw.U - 1 ? ny : yb - 1;
-    c.fown = a.fluence != nullptr && c.i >= fxa && c.i < fxb && c.j >= fya && c.j < fyb;
-    c.sx = c.indom && npml > 0 && (c.i < npml || c.i >= nx - npml);
-    c.sy = c.indom && npml > 0 && (c.j < npml || c.j >= ny - npml);
-    const int ii = c.sx ? (c.i < npml ? c.i : c.i - nx + w2) : 0;
+    const bool x0 = c.i >= xa && c.i < xb, x1 = c.i >= xa && c.i + 1 < xb;   // xa is even: x1 implies x0
+    const bool oy = c.j >= ya && c.j < yb;
+    c.own0 = oy && x0;
+    c.own1 = oy && x1;
+    const bool fy = a.fluence != nullptr && c.j >= fya && c.j < fyb;
+    c.f0 = fy && x0;
+    c.f1 = fy && x1;
+    auto shell = [&](int i) { return npml > 0 && (i < npml || i >= nx - npml); };
+    c.xpair = ((nx | npml) & 1) == 0;
+    c.sx0 = c.in0 && shell(c.i);
+    c.sx1 = c.in1 && shell(c.i + 1);
+    c.sy = c.in0 && npml > 0 && (c.j < npml || c.j >= ny - npml);
+    auto shx = [&](int i) { return i < npml ? i : i - nx + w2; };
+    const int i0 = c.sx0 ? shx(c.i) : 0, i1 = c.sx1 ? shx(c.i + 1) : 0;
     const int jj = c.sy ? (c.j < npml ? c.j : c.j - ny + w2) : 0;
-    c.col = c.indom ? c.j * a.pitch + c.i : 0;
-    c.colx = c.sx ? c.j * w2 + ii : 0;
+    c.col = c.in0 ? c.j * a.pitch + c.i : 0;
+    // x-shell offset of the first column of the pair, such that the second is
+    // one on wherever it is in a shell
+    c.colx = c.sx0 ? c.j * w2 + i0 : (c.sx1 ? c.j * w2 + i1 - 1 : 0);
     c.coly = c.sy ? jj * a.pitch + c.i : 0;
     // coefficients of a column past the box are zero: its values stay zero
-    c.chx = c.indom ? a.chx[c.i] : 0.0f; c.chy = c.indom ? a.chy[c.j] : 0.0f;
-    c.cex = c.indom ? a.cex[c.i] : 0.0f; c.cey = c.indom ? a.cey[c.j] : 0.0f;
-    c.bhx = c.sx ? a.bhx[ii] : 0.0f; c.ahx = c.sx ? a.ahx[ii] : 0.0f;
-    c.bex = c.sx ? a.bex[ii] : 0.0f; c.aex = c.sx ? a.aex[ii] : 0.0f;
-    c.bhy = c.sy ? a.bhy[jj] : 0.0f; c.ahy = c.sy ? a.ahy[jj] : 0.0f;
-    c.bey = c.sy ? a.bey[jj] : 0.0f; c.aey = c.sy ? a.aey[jj] : 0.0f;
-    c.mk = (c.indom && a.smask) ? (a.smask[c.j * nx + c.i] & 0x3f) : uint8_t(0);
-    c.ant = __syncthreads_or(c.mk != 0) != 0;
-    c.anth = __any_sync(0xffffffffu, (c.mk & 0x38) != 0);
-    c.ante = __any_sync(0xffffffffu, (c.mk & 0x07) != 0);
+    auto pair = [&](const float* t, bool v0, int q0, bool v1, int q1) {
+        return make_float2(v0 ? t[q0] : 0.0f, v1 ? t[q1] : 0.0f);
+    };
+    c.chx = pair(a.chx, c.in0, c.i, c.in1, c.i + 1);
+    c.cex = pair(a.cex, c.in0, c.i, c.in1, c.i + 1);
+    c.chy = dup2(c.in0 ? a.chy[c.j] : 0.0f);
+    c.cey = dup2(c.in0 ? a.cey[c.j] : 0.0f);
+    if (GX) {
+        c.bhx = pair(a.bhx, c.sx0, i0, c.sx1, i1); c.ahx = pair(a.ahx, c.sx0, i0, c.sx1, i1);
+        c.bex = pair(a.bex, c.sx0, i0, c.sx1, i1); c.aex = pair(a.aex, c.sx0, i0, c.sx1, i1);
+    }
+    if (GY) {
+        c.bhy = dup2(c.sy ? a.bhy[jj] : 0.0f); c.ahy = dup2(c.sy ? a.ahy[jj] : 0.0f);
+        c.bey = dup2(c.sy ? a.bey[jj] : 0.0f); c.aey = dup2(c.sy ? a.aey[jj] : 0.0f);
+    }
+    const uint8_t m0 = (c.in0 && a.smask) ? (a.smask[c.j * nx + c.i] & 0x3f) : uint8_t(0);
+    const uint8_t m1 = (c.in1 && a.smask) ? (a.smask[c.j * nx + c.i + 1] & 0x3f) : uint8_t(0);
+    c.ant = __syncthreads_or((m0 | m1) != 0) != 0;
+    c.anth = __any_sync(0xffffffffu, ((m0 | m1) & 0x38) != 0);
+    c.ante = __any_sync(0xffffffffu, ((m0 | m1) & 0x07) != 0);
     if (c.ant) {   // every column of the window, zeros where it has no point of a component
         const Cpx<float>* coef = static_cast<const Cpx<float>*>(a.scoefr);
+        const Cpx<float> zero{0.0f, 0.0f};
         for (int q = 0; q < 6; ++q) {
-            const Cpx<float> v = (c.mk >> q) & 1 ? coef[q * nx * ny + c.j * nx + c.i] : Cpx<float>{0.0f, 0.0f};
-            b.SC[q * NT + c.tid] = make_float2(v.x, v.y);
+            const Cpx<float>* t = coef + q * nx * ny + c.j * nx + c.i;
+            const Cpx<float> v0 = (m0 >> q) & 1 ? t[0] : zero, v1 = (m1 >> q) & 1 ? t[1] : zero;
+            st2(b.SC + (2 * q) * NC + c.at, make_float2(v0.x, v1.x));
+            st2(b.SC + (2 * q + 1) * NC + c.at, make_float2(v0.y, v1.y));
         }
     }
 
-    const float dt16 = float(a.dt16);
-    const int P0 = kb - 2, P1 = ke + 1;   // planes streamed: kb-2 .. ke+1
+    const float dt16 = tw.dt16;
+    // planes streamed: kb-2 .. ke+1, and one more before the upper z wall,
+    // where the range holds the fluence of the last plane too
+    const int P0 = kb - 2, P1 = ke + 1 + (W && a.zw && ke == nz ? 1 : 0);
     Tb2Carry s;
-    for (int q = 0; q < 3; ++q) { s.e0[q] = 0.0f; s.h1p[q] = 0.0f; s.e1p[q] = 0.0f; }
-    s.h2px = s.h2py = 0.0f;
-    s.fPEx = s.fPEy = s.fcz = s.fhbx = s.fhby = s.fHsz = 0.0f;
-    s.gPEx = s.gPEy = s.gcz = s.ghbx = s.ghby = s.gHsz = 0.0f;
-    s.tn = 0.0f;
+    const float2 z2 = dup2(0.0f);
+    for (int q = 0; q < 3; ++q) { s.e0[q] = z2; s.h1p[q] = z2; s.e1p[q] = z2; }
+    s.h2px = s.h2py = z2;
+    s.fPEx = s.fPEy = s.fcz = s.fhbx = s.fhby = s.fHsz = z2;
+    s.gPEx = s.gPEy = s.gcz = s.ghbx = s.ghby = s.gHsz = z2;
+    s.tn = z2;
+    for (int q = 0; q < 4; ++q) { s.px[q] = z2; s.py[q] = z2; }
     s.zq = s.zr = Cpx<float>{0.0f, 0.0f};
-    s.kp = (P0 % nz + nz) % nz;
-    s.kq = s.kp == 0 ? nz - 1 : s.kp - 1;
-    s.kr = s.kq == 0 ? nz - 1 : s.kq - 1;
-    s.k3 = s.kr == 0 ? nz - 1 : s.kr - 1;
-    // prologue: the fields of planes P0, P0 + 1, P0 + 2 into slots 0, 1, 2
-    // (their fluence planes P0 - 3, P0 - 2, P0 - 1), the psi of planes P0 - 1,
-    // P0, P0 + 1 into slots 3, 0, 1
-    const int k1 = next_plane(s.kp, nz), k2 = next_plane(k1, nz);
-    tb2_issue<RY, G>(a, c, b, 0, s.kp, s.k3, 3, s.kq);
-    tb2_issue<RY, G>(a, c, b, 1, k1, s.kr, 0, s.kp);
-    tb2_issue<RY, G>(a, c, b, 2, k2, s.kq, 1, k1);
-    s.ki = next_plane(k2, nz);
-    // the ring's four slots: plane p uses slot u = (p - P0) mod 4
+    const bool raw = W && a.zw;   // z walls: planes as they are
+    s.kp = raw ? P0 : (P0 % nz + nz) % nz;
+    s.kq = raw ? P0 - 1 : (s.kp == 0 ? nz - 1 : s.kp - 1);
+    s.kr = raw ? P0 - 2 : (s.kq == 0 ? nz - 1 : s.kq - 1);
+    s.k3 = raw ? P0 - 3 : (s.kr == 0 ? nz - 1 : s.kr - 1);
+    // prologue: the boxes of the iterations of planes P0, P0 + 1, P0 + 2 (their
+    // fluence planes P0 - 3, P0 - 2, P0 - 1), the psi of planes P0 - 1 and P0.
+    // The first iteration reads E^n and H^{n-1/2} of plane P0 - 1 from the slot
+    // before the first: stale values, that (like the zero carry) only reach
+    // the recomputed planes below kb.
+    const int k1 = tb2_next<W>(a, s.kp), k2 = tb2_next<W>(a, k1);
+    tb2_issue<RY>(a, m, b, gq & 3, s.kp, s.k3, L0, M0);
+    tb2_issue<RY>(a, m, b, (gq + 1) & 3, k1, s.kr, L0, M0);
+    tb2_issue<RY>(a, m, b, (gq + 2) & 3, k2, s.kq, L0, M0);
+    if (GX || GY) {
+        tb2_issue_psi<RY, G, W>(a, c, b, 1, s.kq);
+        tb2_issue_psi<RY, G, W>(a, c, b, 0, s.kp);
+    }
+    s.ki = tb2_next<W>(a, k2);
+    // stores: fields of plane p-2 in [kb, ke), fluence of plane p-3 in
+    // [kb-1, ke-1) (modulo nz; on z-walled grids [max(kb-1, 0), ke-1), to nz
+    // where ke = nz)
     int p = P0;
-    int u = 0;
-    for (;;) {
-        tb2_plane<RY, 0, G>(a, tt, c, b, s, p >= kb + 2, p + 3 <= P1, dt16, u);
-        u = (u + 1) & 3;
-        if (++p > P1) break;
-        tb2_plane<RY, 1, G>(a, tt, c, b, s, p >= kb + 2, p + 3 <= P1, dt16, u);
-        u = (u + 1) & 3;
-        if (++p > P1) break;
+    auto valid = [&]() { return p >= kb + 2 && (!W || p < ke + 2); };
+    auto okF = [&]() { return p >= kb + 2 && (!raw || p >= 3); };
+    // W: planes of the z shells run their code one by one, the others in a loop
+    // as lean as the z-periodic kernel's (with a choice per plane inside the
+    // loop the body left the instruction cache)
+    int u = 0;   // (p - P0) mod 2
+    bool more = true;
+    while (more) {
+        if constexpr (W) {
+            if (u == 1 || !tb2_plain(a, s)) {
+                if (u == 0)
+                    tb2_plane<RY, 0, G, 2, CR>(a, m, tt, c, b, s, valid(), okF(), p + 3 <= P1, p + 2 <= P1, dt16, gq,
+                                                  L0, M0, dead);
+                else
+                    tb2_plane<RY, 1, G, 2, CR>(a, m, tt, c, b, s, valid(), okF(), p + 3 <= P1, p + 2 <= P1, dt16, gq,
+                                                  L0, M0, dead);
+                u ^= 1;
+                ++gq;
+                more = ++p <= P1;
+                continue;
+            }
+        }
+        #pragma unroll 1
+        for (;;) {
+            tb2_plane<RY, 0, G, W ? 1 : 0, CR>(a, m, tt, c, b, s, valid(), okF(), p + 3 <= P1, p + 2 <= P1, dt16, gq, L0,
+                                           M0, dead);
+            ++gq;
+            u = 1;
+            if (!(more = ++p <= P1)) break;
+            if (W && !tb2_plain(a, s)) break;
+            tb2_plane<RY, 1, G, W ? 1 : 0, CR>(a, m, tt, c, b, s, valid(), okF(), p + 3 <= P1, p + 2 <= P1, dt16, gq, L0,
+                                           M0, dead);
+            ++gq;
+            u = 0;
+            if (!(more = ++p <= P1)) break;
+            if (W && !tb2_plain(a, s)) break;
+        }
     }
     cpa_wait0();
 }
 
-template <int RY>
-__device__ __forceinline__ void tb2_run(const StepArgs<float>& a, const Tb2Times& tt, const Tb2Plan& tw)
+template <int RY, bool W, bool CR>
+__device__ __forceinline__ void tb2_run(const StepArgs<float>& a, const TmaMaps& m, const Tb2Times& tt,
+                                        const Tb2Plan& tw)
 {
     using S = Tb2Smem<RY>;
-    constexpr int NT = S::NT, R = S::R, NF = S::NF;
-    extern __shared__ __align__(16) unsigned char tb2_smem[];
+    constexpr int NT = S::NT, NC = S::NC, R = S::R, XS = S::XS;
+    extern __shared__ unsigned char tb2_smem_raw[];
     Tb2Bufs<RY> b;
-    b.fring = reinterpret_cast<float2*>(tb2_smem);
-    b.ring = reinterpret_cast<float*>(b.fring + R * NT);
-    constexpr int XS = S::XS;
-    b.EB = b.ring + R * NF * NT;
-    b.HB = b.EB + 4 * XS;
+    b.ring = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(tb2_smem_raw) + 127) & ~uintptr_t(127));
+    b.psi = b.ring + R * S::SLOT;
+    b.HB = b.psi + 2 * S::NP * NC;
     b.E1B = b.HB + 3 * XS;
     b.H1B = b.E1B + 4 * XS;
-    b.SC = reinterpret_cast<float2*>(b.H1B + 3 * XS + 32);
-    // the NX + 1 zero rows of the exchange arrays (never written again; the
-    // first window's barrier orders these stores before any read)
-    for (int q = threadIdx.y * 32 + threadIdx.x; q < (S::NX + 1) * 32; q += NT)
-        b.EB[(q / 32) * XS + q % 32] = 0.0f;
+    b.SC = b.H1B + 3 * XS + 64;
+    b.bars = reinterpret_cast<uint64_t*>(b.SC + 12 * NC);
+    b.err = tw.err;
+    b.pol = tb2_store_policy();
+    if (threadIdx.x == 0) {
+        for (int q = 0; q < R; ++q) mbar_init(b.bars + q, 1);
+        mbar_fence_init();
+    }
+    __syncthreads();
+    uint32_t gq = 0;
+    bool dead = false;   // a wait expired: run on without waiting, the error word is raised
     const long long t0 = tw.prof ? clock64() : 0;
     long long w = tw.start[blockIdx.x];
     const long long wend = tw.start[blockIdx.x + 1];
@@ -672,44 +955,51 @@ __device__ __forceinline__ void tb2_run(const StepArgs<float>& a, const Tb2Times
         const int window = tb2_window_at(tw, int(w / a.nz)), kb = int(w % a.nz);
         const long long left = wend - w;
         const int ke = left < (long long)(a.nz - kb) ? kb + int(left) : a.nz;
-        // a window off the box faces and the CPML shells runs without the
-        // checks of walls, psi and columns past the box (G = 0; the x and y
-        // checks are separate flags, but instantiating them apart measured no
-        // faster)
+        // a window off the x (y) faces and shells runs without the checks of
+        // the x (y) walls, psi and columns past the box
         const int wx = window % tw.T, wy = window / tw.T;
-        const int L0 = kTb2Sx * wx, M0 = (RY - 4) * wy;
-        const bool gen = wx == 0 || wx == tw.T - 1 || wy == 0 || wy == tw.U - 1 ||
-                         (a.npml > 0 && (L0 < a.npml || L0 + kTb2Wx > a.nx - a.npml || M0 < a.npml ||
-                                         M0 + RY > a.ny - a.npml));
-        if (gen) tb2_window<RY, 3>(a, tt, tw, window, kb, ke, b);
-        else tb2_window<RY, 0>(a, tt, tw, window, kb, ke, b);
+        const int L0 = kTb2Sx * wx - kTb2Ox, M0 = (RY - 4) * wy - kTb2Oy;
+        const bool gx = wx == 0 || wx == tw.T - 1 || (a.npml > 0 && (L0 < a.npml || L0 + kTb2Wx > a.nx - a.npml));
+        const bool gy = wy == 0 || wy == tw.U - 1 || (a.npml > 0 && (M0 < a.npml || M0 + RY > a.ny - a.npml));
+        if (!gx && !gy) tb2_window<RY, 0, W, CR>(a, m, tt, tw, window, kb, ke, b, gq, dead);
+        else if (!gy) tb2_window<RY, 1, W, CR>(a, m, tt, tw, window, kb, ke, b, gq, dead);
+        else if (!gx) tb2_window<RY, 2, W, CR>(a, m, tt, tw, window, kb, ke, b, gq, dead);
+        else tb2_window<RY, 3, W, CR>(a, m, tt, tw, window, kb, ke, b, gq, dead);
         w += ke - kb;
-        __syncthreads();   // the exchange buffers are reused by the next window
+        __syncthreads();   // the ring and the exchange buffers are reused by the next window
     }
-    if (tw.prof && threadIdx.x == 0 && threadIdx.y == 0)
-        tw.prof[blockIdx.x] += static_cast<unsigned long long>(clock64() - t0);
+    if (dead) {   // copies may still be in flight: give each slot's last phase one more bounded wait
+        for (int q = 0; q < R && q < int(gq); ++q) {
+            const uint32_t last = gq - 1 - ((gq - 1 - q) & 3);   // last iteration that used slot q
+            mbar_wait_bounded(b.bars + q, (last >> 2) & 1);
+        }
+    }
+    if (tw.prof && threadIdx.x == 0) tw.prof[blockIdx.x] += static_cast<unsigned long long>(clock64() - t0);
 }
 
-// Steps n and n+1 with their source time factors as a parameter.
-template <int RY>
-__global__ void __launch_bounds__(32 * RY, 1)
-yee_tb2(const StepArgs<float> a, const Tb2Times tt, const __grid_constant__ Tb2Plan tw)
+// Steps n and n+1 with their source time factors as a parameter.  W: grids
+// with z walls or a wall sheet (kept apart, so that the z-periodic kernel
+// carries none of it).  CR: see tb2_flux.
+template <int RY, bool W, bool CR>
+__global__ void __launch_bounds__(16 * RY, 1)
+yee_tb2(const StepArgs<float> a, const Tb2Times tt, const __grid_constant__ TmaMaps m,
+        const __grid_constant__ Tb2Plan tw)
 {
-    tb2_run<RY>(a, tt, tw);
+    tb2_run<RY, W, CR>(a, m, tt, tw);
 }
 
 // The same with the time factors of the two steps read from a device table
 // (times[i0] for step n, times[i1] for step n+1): the batched graph replays
 // these launches with the table refreshed before each replay.
-template <int RY>
-__global__ void __launch_bounds__(32 * RY, 1)
+template <int RY, bool W, bool CR>
+__global__ void __launch_bounds__(16 * RY, 1)
 yee_tb2_t(const StepArgs<float> a, const StepTime<float>* __restrict__ times, int i0, int i1,
-          const __grid_constant__ Tb2Plan tw)
+          const __grid_constant__ TmaMaps m, const __grid_constant__ Tb2Plan tw)
 {
     Tb2Times tt;
-    tt.th0 = times[i0].th; tt.te0 = times[i0].te;
-    tt.th1 = times[i1].th; tt.te1 = times[i1].te;
-    tb2_run<RY>(a, tt, tw);
+    tt.th0 = times[i0].th; tt.te0 = times[i0].te; tt.tw0 = times[i0].tw;
+    tt.th1 = times[i1].th; tt.te1 = times[i1].te; tt.tw1 = times[i1].tw;
+    tb2_run<RY, W, CR>(a, m, tt, tw);
 }
 
 }  // namespace fdtd
