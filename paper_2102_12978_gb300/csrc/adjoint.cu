@@ -604,13 +604,8 @@ fdtd_status fdtd_adjoint_get(fdtd_adjoint* a, int component, void* dst)
     if (!a || !dst || component < 0 || component > 5) return fail(FDTD_EINVAL, "invalid argument");
     const fdtd_status dev_st = check_device(a->g, "fdtd_adjoint_get");
     if (dev_st != FDTD_OK) return dev_st;
-    const fdtd_grid_desc& d = a->g->desc;
-    const size_t b = a->g->L.elem;
     const size_t off = component < 3 ? a->e[a->cur][component] : a->h[a->cur][component - 3];
-    fdtd_status st = cuda_check(cudaMemcpy2DAsync(dst, size_t(d.nx) * b, static_cast<char*>(a->arena) + off,
-                                                  size_t(a->g->L.pitch) * b, size_t(d.nx) * b, size_t(d.ny) * d.nz,
-                                                  cudaMemcpyDeviceToDevice, a->g->stream),
-                                "copy adjoint field");
+    const fdtd_status st = copy_field_out(a->g, static_cast<char*>(a->arena) + off, dst, true);
     if (st != FDTD_OK) return st;
     return fdtd_sync(a->g);
 }

@@ -74,14 +74,13 @@ fdtd_status fdtd_fluence_noalloc(fdtd_grid* g, void* dst, int on_device, int res
                           : nullptr;
     if (!scratch) return fail(FDTD_ESTATE, "no staging array on device %d", g->device);
     char* A = static_cast<char*>(g->arena);
-    const int blocks = 4 * (g->sm_count > 0 ? g->sm_count : 152);
-    if (d.precision == FDTD_F64)
-        fluence_export<double><<<blocks, 256, 0, g->stream>>>(reinterpret_cast<const double*>(A + g->L.fluence),
-                                                              scratch, d.nx, d.ny, d.nz, g->L.pitch, 1.0);
-    else
-        fluence_export<float2><<<blocks, 256, 0, g->stream>>>(reinterpret_cast<const float2*>(A + g->L.fluence),
-                                                               scratch, d.nx, d.ny, d.nz, g->L.pitch, 1.0);
-    fdtd_status st = cuda_check(cudaGetLastError(), "fluence_export launch");
+    const long long rows = (long long)d.ny * d.nz;
+    const void* F = A + g->L.fluence;
+    fdtd_status st = cuda_check(
+        d.precision == FDTD_F64
+            ? launch_fluence_export(static_cast<const double*>(F), scratch, d.nx, rows, g->L.pitch, g->sm_count, g->stream)
+            : launch_fluence_export(static_cast<const float2*>(F), scratch, d.nx, rows, g->L.pitch, g->sm_count, g->stream),
+        "fluence_export launch");
     if (st == FDTD_OK)
         st = cuda_check(cudaMemcpyAsync(dst, scratch, cells * 8,
                                         on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, g->stream),
