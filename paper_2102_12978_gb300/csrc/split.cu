@@ -111,7 +111,12 @@ static cudaError_t launch_step_cell(const fdtd_grid* g, int cur, long long n, cu
 }
 
 // FP64 grids with an antenna (z-periodic, no wall sheet) add its source in
-// antenna_add after each pass instead of inside it.
+// antenna_add after each pass instead of inside it, from kApartCells cells on.
+// Below, two launches more per step (6 us each with the gap) cost more than the
+// FP64 pipe saves (us per step, apart / inside: 48 x 40 x 16 28 / 16.5, 64 x 64 x
+// 32 37 / 29, 96 x 96 x 64 94.6 / 93.2, 128 x 128 x 64 147.5 / 150.1, 256 x 256
+// x 128 927 / 980).
+constexpr double kApartCells = 8e5;
 template <typename real>
 static cudaError_t antenna_pass(const fdtd_grid* g, const StepArgs<real>& a, int side, Cpx<real> t, cudaStream_t s)
 {
@@ -142,7 +147,8 @@ static cudaError_t launch_cell(const fdtd_grid* g, int cur, long long n, cudaStr
     const int nz = g->desc.nz, nchunk = (nz + kMaxPlanes - 1) / kMaxPlanes;
     dim3 block(32, TY);
     const bool wall = has_walls(g);   // z walls or a wall sheet: the *_w kernels
-    const bool apart = sizeof(real) == 8 && g->has_source && g->ant_apart && !wall;
+    const bool apart = sizeof(real) == 8 && g->has_source && g->ant_apart && !wall &&
+                       double(g->desc.nx) * g->desc.ny * nz >= kApartCells;
     const StepArgs<real> full = make_args<real>(g, cur);
     StepArgs<real> a = full;
     if (apart) a.smask = nullptr;   // the passes run without the antenna
