@@ -562,8 +562,13 @@ fdtd_status fdtd_set_annulus_source(fdtd_grid* g, const fdtd_annulus_desc* s)
     std::vector<double> wamp(ncol, 1.0), wph(ncol, 0.0);
     if (s->w_amp) std::memcpy(wamp.data(), s->w_amp, ncol * 8);
     if (s->w_phase) std::memcpy(wph.data(), s->w_phase, ncol * 8);
-    coef.resize(coef_unw.size());
-    for (size_t q = 0; q < coef_unw.size(); ++q) coef[q] = std::polar(wamp[q % ncol], wph[q % ncol]) * coef_unw[q];
+    // the weights act on the antenna's columns only (one factor per column)
+    coef.assign(coef_unw.size(), std::complex<double>(0.0, 0.0));
+    for (size_t col = 0; col < ncol; ++col) {
+        if (!mask[col]) continue;
+        const std::complex<double> w = std::polar(wamp[col], wph[col]);
+        for (size_t q = col; q < coef.size(); q += ncol) coef[q] = w * coef_unw[q];
+    }
     // e^{i beta k dz}: the coefficients already carry each component's own
     // half-cell z offset, so one table serves every component
     const double beta = 2.0 * M_PI * std::cos(s->theta);
