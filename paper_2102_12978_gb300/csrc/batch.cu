@@ -716,6 +716,7 @@ static fdtd_status batch_step_ranges(fdtd_batch* b, int nsteps)
         const fdtd_status pst = b->precision == FDTD_F64 ? pcell_fill<double>(b) : pcell_fill<float>(b);
         if (pst != FDTD_OK) return pst;
     }
+    for (fdtd_grid* g : b->grids) g->err_dirty = true;   // replays of two-step launches
     int done = 0;
     while (done < nsteps) {
         const int count = nsteps - done < kBatchGraphSteps ? nsteps - done : kBatchGraphSteps;

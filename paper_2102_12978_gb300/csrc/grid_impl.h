@@ -99,6 +99,7 @@ struct fdtd_grid {
     fdtd_annulus_desc src;
     fdtd::SrcTime srct;
     int64_t counts[6];
+    bool err_dirty;          // kernels that may raise the error word were queued since it was last read as zero
     int sm_count;
     int device;                 // CUDA device current at fdtd_create_grid
     fdtd::TileConfig tile;
