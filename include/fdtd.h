@@ -276,7 +276,7 @@ fdtd_status fdtd_set_tile(fdtd_grid* g, int variant, int ty, int lz);
  * for both), plus w_antenna if it holds antenna columns, and each CTA takes a
  * contiguous range of (window, plane) work of equal estimated cost; a window
  * also costs some planes at its start (the two-step wavefront refills
- * there).  Weights in [0, 16] (else EINVAL); defaults 0.4 and 0.15.  fdtd_autotune times a few pairs, then refines the fastest pair's
+ * there).  Weights in [0, 16] (else EINVAL); defaults 0.4 and 0.2.  fdtd_autotune times a few pairs, then refines the fastest pair's
  * ranges on measured times (fdtd_measure_balance), with the windows row by
  * row and interleaved (lz 1 and 2), and times those; it keeps the fastest.
  * While refined ranges are in use, fdtd_get_balance returns -1 for both

@@ -51,7 +51,7 @@ struct TileConfig {
     // variant 7: extra cost per plane of a window holding CPML shell / antenna
     // columns, relative to a plain window (the CTAs' work ranges are balanced
     // on these estimates)
-    float w_shell = 0.4f, w_ant = 0.15f;
+    float w_shell = 0.4f, w_ant = 0.2f;
     // variant 7: run the ranges refined from measured per-CTA times
     // (fdtd_grid::tb2_refined) instead of those of the weights above
     bool measured = false;

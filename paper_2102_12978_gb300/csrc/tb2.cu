@@ -106,7 +106,7 @@ static int tb2_window_host(int T, int U, int D, int pos)
 // the weights or the launch shape change.
 // Measured on GB300 (cycles per plane, 256 x 256 x 128 cells): inner windows
 // 2400, with antenna columns 2750, x shell 3340, y shell 3380, both 4720; the
-// default weights 0.4 and 0.15 follow.
+// default weights 0.4 and 0.2 follow (0.15 is slower by up to 2 %).
 constexpr double kRestart = 5.3;
 constexpr double kCorner = 0.4;
 constexpr double kZPlane = 1.6;
@@ -202,17 +202,19 @@ static cudaError_t tb2_blocks_per_sm(int* out)
     if (blocks_per_sm.load() == 0) {
         const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
         const int bytes = int(S::bytes());
-        cudaError_t e = cudaFuncSetAttribute(yee_tb2<RY, false, false>, at, bytes);
+        cudaError_t e = cudaFuncSetAttribute(yee_tb2<RY, false, false, true>, at, bytes);
         if constexpr (RY == kTb2Rows) {
-            if (e == cudaSuccess) e = cudaFuncSetAttribute(yee_tb2<RY, false, true>, at, bytes);
-            if (e == cudaSuccess) e = cudaFuncSetAttribute(yee_tb2<RY, true, true>, at, bytes);
-            if (e == cudaSuccess) e = cudaFuncSetAttribute(yee_tb2_t<RY, false, false>, at, bytes);
-            if (e == cudaSuccess) e = cudaFuncSetAttribute(yee_tb2_t<RY, false, true>, at, bytes);
-            if (e == cudaSuccess) e = cudaFuncSetAttribute(yee_tb2_t<RY, true, true>, at, bytes);
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(yee_tb2<RY, false, false, false>, at, bytes);
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(yee_tb2<RY, false, true, true>, at, bytes);
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(yee_tb2<RY, false, true, false>, at, bytes);
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(yee_tb2<RY, true, true, true>, at, bytes);
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(yee_tb2_t<RY, false, false, true>, at, bytes);
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(yee_tb2_t<RY, false, true, true>, at, bytes);
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(yee_tb2_t<RY, true, true, true>, at, bytes);
         }
         if (e != cudaSuccess) return e;
         int n = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, yee_tb2<RY, false, false>, S::NT, S::bytes());
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, yee_tb2<RY, false, false, true>, S::NT, S::bytes());
         if (e != cudaSuccess) return e;
         if (n < 1) return cudaErrorInvalidConfiguration;
         blocks_per_sm.store(n);
@@ -290,13 +292,19 @@ static cudaError_t launch_tb2_t(const fdtd_grid* cg, int cur, long long n, const
     const StepArgs<float> a = make_args<float>(g, cur);
     const unsigned ctas = unsigned(slots);
     if constexpr (RY == kTb2Rows) {
+        const bool flu = g->desc.fluence != 0;
         if (tc.automatic) {   // runs on the default tile: the cell passes' roundings
-            if (has_walls(g)) yee_tb2<RY, true, true><<<ctas, S::NT, S::bytes(), s>>>(a, tt, *m, plan);
-            else yee_tb2<RY, false, true><<<ctas, S::NT, S::bytes(), s>>>(a, tt, *m, plan);
+            if (has_walls(g)) yee_tb2<RY, true, true, true><<<ctas, S::NT, S::bytes(), s>>>(a, tt, *m, plan);
+            else if (flu) yee_tb2<RY, false, true, true><<<ctas, S::NT, S::bytes(), s>>>(a, tt, *m, plan);
+            else yee_tb2<RY, false, true, false><<<ctas, S::NT, S::bytes(), s>>>(a, tt, *m, plan);
+            return cudaGetLastError();
+        }
+        if (!flu) {
+            yee_tb2<RY, false, false, false><<<ctas, S::NT, S::bytes(), s>>>(a, tt, *m, plan);
             return cudaGetLastError();
         }
     }
-    yee_tb2<RY, false, false><<<ctas, S::NT, S::bytes(), s>>>(a, tt, *m, plan);
+    yee_tb2<RY, false, false, true><<<ctas, S::NT, S::bytes(), s>>>(a, tt, *m, plan);
     return cudaGetLastError();
 }
 
@@ -327,9 +335,9 @@ cudaError_t launch_tb2_table(const fdtd_grid* cg, int cur, const StepTime<float>
     g->err_dirty = true;
     const StepArgs<float> a = make_args<float>(g, cur);
     const unsigned ctas = unsigned(slots);
-    if (!automatic) yee_tb2_t<RY, false, false><<<ctas, S::NT, S::bytes(), s>>>(a, times, i0, i1, *m, plan);
-    else if (has_walls(g)) yee_tb2_t<RY, true, true><<<ctas, S::NT, S::bytes(), s>>>(a, times, i0, i1, *m, plan);
-    else yee_tb2_t<RY, false, true><<<ctas, S::NT, S::bytes(), s>>>(a, times, i0, i1, *m, plan);
+    if (!automatic) yee_tb2_t<RY, false, false, true><<<ctas, S::NT, S::bytes(), s>>>(a, times, i0, i1, *m, plan);
+    else if (has_walls(g)) yee_tb2_t<RY, true, true, true><<<ctas, S::NT, S::bytes(), s>>>(a, times, i0, i1, *m, plan);
+    else yee_tb2_t<RY, false, true, true><<<ctas, S::NT, S::bytes(), s>>>(a, times, i0, i1, *m, plan);
     return cudaGetLastError();
 }
 

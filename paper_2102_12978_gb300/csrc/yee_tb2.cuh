@@ -417,7 +417,7 @@ __device__ __forceinline__ float2 tb2_sheet(const StepArgs<float>& a, const Tb2C
 // The walls: E_x and E_y are zero on the planes 0 and nz (plane nz reads as
 // zeros; its E^{n+1} is set to zero here), and with that no value of a plane
 // below 0 or above nz reaches a stored one.
-template <int RY, int U, int G, int W, bool CR>
+template <int RY, int U, int G, int W, bool CR, bool FL>
 __device__ __forceinline__ void tb2_plane(const StepArgs<float>& a, const TmaMaps& m, const Tb2Times& tt,
                                           const Tb2Col& c, const Tb2Bufs<RY>& b, Tb2Carry& s, bool valid, bool okF,
                                           bool issue_next, bool issue_psi, float dt16, uint32_t gq, int wx0, int wy0, bool& dead)
@@ -514,18 +514,19 @@ __device__ __forceinline__ void tb2_plane(const StepArgs<float>& a, const TmaMap
             hy = add2(hy, tb2_src(b, c, 4, u));
             hz = add2(hz, tb2_src(b, c, 5, u));
         }
-        // centre sums of step n for plane q
-        nPEx = add2(ex, exj);
-        nPEy = add2(ey, eyi);
-        ncz = add2(add2(ez, ezi), add2(ezj, xp(ezj)));
-        const float2 hsx = add2(ox, hx);
-        hsy = add2(oy, hy);
-        nHsz = add2(oz, hz);
-        nhbx = add2(hsx, xp(hsx));
+        if constexpr (FL) {   // centre sums of step n for plane q
+            nPEx = add2(ex, exj);
+            nPEy = add2(ey, eyi);
+            ncz = add2(add2(ez, ezi), add2(ezj, xp(ezj)));
+            const float2 hsx = add2(ox, hx);
+            hsy = add2(oy, hy);
+            nHsz = add2(oz, hz);
+            nhbx = add2(hsx, xp(hsx));
+        }
     }
     put(b.HB, hx);
     put(b.HB + XS, hz);
-    put(b.HB + 2 * XS, hsy);
+    if constexpr (FL) put(b.HB + 2 * XS, hsy);
     __syncthreads();   // H^{n+1/2} of plane q is there, and every read of ring slot SQ is done
     // refill: the boxes of the iteration of plane p + 3 into the slot of p - 1
     if (issue_next) tb2_issue<RY>(a, m, b, SQ, s.ki, s.kp, wx0, wy0);
@@ -578,9 +579,11 @@ __device__ __forceinline__ void tb2_plane(const StepArgs<float>& a, const TmaMap
         else cpa_commit();
     }
     // fluence term of step n for plane r = p-2 (sums of planes r and q)
-    const float2 nhby = add2(hsy, yp(b.HB + 2 * XS));
-    const float2 tn_new = tb2_flux<CR>(add2(s.fPEx, nPEx), add2(s.fPEy, nPEy), s.fcz, s.fhbx, s.fhby, add2(s.fHsz, nHsz),
-                                   dt16);
+    float2 nhby, tn_new;
+    if constexpr (FL) {
+        nhby = add2(hsy, yp(b.HB + 2 * XS));
+        tn_new = tb2_flux<CR>(add2(s.fPEx, nPEx), add2(s.fPEy, nPEy), s.fcz, s.fhbx, s.fhby, add2(s.fHsz, nHsz), dt16);
+    }
 
     // ---- stage C: H^{n+3/2} of plane r
     float2 h2x, h2y, h2z, gsy;
@@ -635,14 +638,15 @@ __device__ __forceinline__ void tb2_plane(const StepArgs<float>& a, const TmaMap
             h2y = add2(h2y, tb2_src(b, c, 4, u));
             h2z = add2(h2z, tb2_src(b, c, 5, u));
         }
-        // centre sums of step n+1 for plane r
-        mPEx = add2(s.e1p[0], fexj);
-        mPEy = add2(s.e1p[1], feyi);
-        mcz = add2(add2(s.e1p[2], fezi), add2(fezj, xp(fezj)));
-        const float2 gsx = add2(s.h1p[0], h2x);
-        gsy = add2(s.h1p[1], h2y);
-        mHsz = add2(s.h1p[2], h2z);
-        mhbx = add2(gsx, xp(gsx));
+        if constexpr (FL) {   // centre sums of step n+1 for plane r
+            mPEx = add2(s.e1p[0], fexj);
+            mPEy = add2(s.e1p[1], feyi);
+            mcz = add2(add2(s.e1p[2], fezi), add2(fezj, xp(fezj)));
+            const float2 gsx = add2(s.h1p[0], h2x);
+            gsy = add2(s.h1p[1], h2y);
+            mHsz = add2(s.h1p[2], h2z);
+            mhbx = add2(gsx, xp(gsx));
+        }
     }
     {
         float* E1Bq = b.E1B + PQ * 2 * XS;
@@ -650,7 +654,7 @@ __device__ __forceinline__ void tb2_plane(const StepArgs<float>& a, const TmaMap
         put(E1Bq + XS, nex);
         put(b.H1B, h2x);
         put(b.H1B + XS, h2z);
-        put(b.H1B + 2 * XS, gsy);
+        if constexpr (FL) put(b.H1B + 2 * XS, gsy);
     }
     __syncthreads();
 
@@ -721,8 +725,9 @@ __device__ __forceinline__ void tb2_plane(const StepArgs<float>& a, const TmaMap
         }
     }
     // fluence of plane p-3: the step-n term from the last plane, then step n+1
-    const float2 mhby = add2(gsy, yp(b.H1B + 2 * XS));
-    {   // every lane computes it (no divergent branch); the fluence cells store it
+    float2 mhby;
+    if constexpr (FL) {   // every lane computes it (no divergent branch); the fluence cells store it
+        mhby = add2(gsy, yp(b.H1B + 2 * XS));
         const float2 t1 = tb2_flux<CR>(add2(s.gPEx, mPEx), add2(s.gPEy, mPEy), s.gcz, s.ghbx, s.ghby, add2(s.gHsz, mHsz),
                                    dt16);
         const float4 f = *reinterpret_cast<const float4*>(b.ring + SP * S::SLOT + 6 * NC + 2 * c.at);
@@ -750,9 +755,11 @@ __device__ __forceinline__ void tb2_plane(const StepArgs<float>& a, const TmaMap
     s.h1p[0] = hx; s.h1p[1] = hy; s.h1p[2] = hz;
     s.e1p[0] = nex; s.e1p[1] = ney; s.e1p[2] = nez;
     s.h2px = h2x; s.h2py = h2y;
-    s.fPEx = nPEx; s.fPEy = nPEy; s.fcz = ncz; s.fhbx = nhbx; s.fhby = nhby; s.fHsz = nHsz;
-    s.gPEx = mPEx; s.gPEy = mPEy; s.gcz = mcz; s.ghbx = mhbx; s.ghby = mhby; s.gHsz = mHsz;
-    s.tn = tn_new;
+    if constexpr (FL) {
+        s.fPEx = nPEx; s.fPEy = nPEy; s.fcz = ncz; s.fhbx = nhbx; s.fhby = nhby; s.fHsz = nHsz;
+        s.gPEx = mPEx; s.gPEy = mPEy; s.gcz = mcz; s.ghbx = mhbx; s.ghby = mhby; s.gHsz = mHsz;
+        s.tn = tn_new;
+    }
     #pragma unroll
     for (int v = 0; v < 4; ++v) {
         if (GX) s.px[v] = npx[v];
@@ -773,7 +780,7 @@ __device__ __forceinline__ bool tb2_plain(const StepArgs<float>& a, const Tb2Car
 // One window, planes [kb, ke) of its E^{n+2} / H^{n+3/2} output (fluence
 // planes [kb-1, ke-1), modulo nz).  gq counts the CTA's iterations: ring slot
 // gq mod 4, mbarrier parity (gq / 4) mod 2.
-template <int RY, int G, bool W, bool CR>
+template <int RY, int G, bool W, bool CR, bool FL>
 __device__ __forceinline__ void tb2_window(const StepArgs<float>& a, const TmaMaps& m, const Tb2Times& tt,
                                            const Tb2Plan& tw, int window, int kb, int ke, const Tb2Bufs<RY>& b,
                                            uint32_t& gq, bool& dead)
@@ -894,10 +901,10 @@ __device__ __forceinline__ void tb2_window(const StepArgs<float>& a, const TmaMa
         if constexpr (W) {
             if (u == 1 || !tb2_plain(a, s)) {
                 if (u == 0)
-                    tb2_plane<RY, 0, G, 2, CR>(a, m, tt, c, b, s, valid(), okF(), p + 3 <= P1, p + 2 <= P1, dt16, gq,
+                    tb2_plane<RY, 0, G, 2, CR, FL>(a, m, tt, c, b, s, valid(), okF(), p + 3 <= P1, p + 2 <= P1, dt16, gq,
                                                   L0, M0, dead);
                 else
-                    tb2_plane<RY, 1, G, 2, CR>(a, m, tt, c, b, s, valid(), okF(), p + 3 <= P1, p + 2 <= P1, dt16, gq,
+                    tb2_plane<RY, 1, G, 2, CR, FL>(a, m, tt, c, b, s, valid(), okF(), p + 3 <= P1, p + 2 <= P1, dt16, gq,
                                                   L0, M0, dead);
                 u ^= 1;
                 ++gq;
@@ -907,13 +914,13 @@ __device__ __forceinline__ void tb2_window(const StepArgs<float>& a, const TmaMa
         }
         #pragma unroll 1
         for (;;) {
-            tb2_plane<RY, 0, G, W ? 1 : 0, CR>(a, m, tt, c, b, s, valid(), okF(), p + 3 <= P1, p + 2 <= P1, dt16, gq, L0,
+            tb2_plane<RY, 0, G, W ? 1 : 0, CR, FL>(a, m, tt, c, b, s, valid(), okF(), p + 3 <= P1, p + 2 <= P1, dt16, gq, L0,
                                            M0, dead);
             ++gq;
             u = 1;
             if (!(more = ++p <= P1)) break;
             if (W && !tb2_plain(a, s)) break;
-            tb2_plane<RY, 1, G, W ? 1 : 0, CR>(a, m, tt, c, b, s, valid(), okF(), p + 3 <= P1, p + 2 <= P1, dt16, gq, L0,
+            tb2_plane<RY, 1, G, W ? 1 : 0, CR, FL>(a, m, tt, c, b, s, valid(), okF(), p + 3 <= P1, p + 2 <= P1, dt16, gq, L0,
                                            M0, dead);
             ++gq;
             u = 0;
@@ -924,7 +931,7 @@ __device__ __forceinline__ void tb2_window(const StepArgs<float>& a, const TmaMa
     cpa_wait0();
 }
 
-template <int RY, bool W, bool CR>
+template <int RY, bool W, bool CR, bool FL>
 __device__ __forceinline__ void tb2_run(const StepArgs<float>& a, const TmaMaps& m, const Tb2Times& tt,
                                         const Tb2Plan& tw)
 {
@@ -961,10 +968,10 @@ __device__ __forceinline__ void tb2_run(const StepArgs<float>& a, const TmaMaps&
         const int L0 = kTb2Sx * wx - kTb2Ox, M0 = (RY - 4) * wy - kTb2Oy;
         const bool gx = wx == 0 || wx == tw.T - 1 || (a.npml > 0 && (L0 < a.npml || L0 + kTb2Wx > a.nx - a.npml));
         const bool gy = wy == 0 || wy == tw.U - 1 || (a.npml > 0 && (M0 < a.npml || M0 + RY > a.ny - a.npml));
-        if (!gx && !gy) tb2_window<RY, 0, W, CR>(a, m, tt, tw, window, kb, ke, b, gq, dead);
-        else if (!gy) tb2_window<RY, 1, W, CR>(a, m, tt, tw, window, kb, ke, b, gq, dead);
-        else if (!gx) tb2_window<RY, 2, W, CR>(a, m, tt, tw, window, kb, ke, b, gq, dead);
-        else tb2_window<RY, 3, W, CR>(a, m, tt, tw, window, kb, ke, b, gq, dead);
+        if (!gx && !gy) tb2_window<RY, 0, W, CR, FL>(a, m, tt, tw, window, kb, ke, b, gq, dead);
+        else if (!gy) tb2_window<RY, 1, W, CR, FL>(a, m, tt, tw, window, kb, ke, b, gq, dead);
+        else if (!gx) tb2_window<RY, 2, W, CR, FL>(a, m, tt, tw, window, kb, ke, b, gq, dead);
+        else tb2_window<RY, 3, W, CR, FL>(a, m, tt, tw, window, kb, ke, b, gq, dead);
         w += ke - kb;
         __syncthreads();   // the ring and the exchange buffers are reused by the next window
     }
@@ -979,19 +986,21 @@ __device__ __forceinline__ void tb2_run(const StepArgs<float>& a, const TmaMaps&
 
 // Steps n and n+1 with their source time factors as a parameter.  W: grids
 // with z walls or a wall sheet (kept apart, so that the z-periodic kernel
-// carries none of it).  CR: see tb2_flux.
-template <int RY, bool W, bool CR>
+// carries none of it).  CR: see tb2_flux.  FL: the fluence terms compiled in;
+// z-periodic grids without a fluence accumulator take the kernels without (332
+// x 332 x 46 cells 66 us per step with the terms compiled in, 54 without).
+template <int RY, bool W, bool CR, bool FL>
 __global__ void __launch_bounds__(16 * RY, 1)
 yee_tb2(const StepArgs<float> a, const Tb2Times tt, const __grid_constant__ TmaMaps m,
         const __grid_constant__ Tb2Plan tw)
 {
-    tb2_run<RY, W, CR>(a, m, tt, tw);
+    tb2_run<RY, W, CR, FL>(a, m, tt, tw);
 }
 
 // The same with the time factors of the two steps read from a device table
 // (times[i0] for step n, times[i1] for step n+1): the batched graph replays
 // these launches with the table refreshed before each replay.
-template <int RY, bool W, bool CR>
+template <int RY, bool W, bool CR, bool FL>
 __global__ void __launch_bounds__(16 * RY, 1)
 yee_tb2_t(const StepArgs<float> a, const StepTime<float>* __restrict__ times, int i0, int i1,
           const __grid_constant__ TmaMaps m, const __grid_constant__ Tb2Plan tw)
@@ -999,7 +1008,7 @@ yee_tb2_t(const StepArgs<float> a, const StepTime<float>* __restrict__ times, in
     Tb2Times tt;
     tt.th0 = times[i0].th; tt.te0 = times[i0].te; tt.tw0 = times[i0].tw;
     tt.th1 = times[i1].th; tt.te1 = times[i1].te; tt.tw1 = times[i1].tw;
-    tb2_run<RY, W, CR>(a, m, tt, tw);
+    tb2_run<RY, W, CR, FL>(a, m, tt, tw);
 }
 
 }  // namespace fdtd
