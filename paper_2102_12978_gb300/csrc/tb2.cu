@@ -95,7 +95,14 @@ static int tb2_window_host(int T, int U, int D, int pos)
 }
 
 // CTA work ranges of variant 7 on grid g: windows of 32 x RY columns, `slots`
-// resident CTAs.  Each CTA gets a contiguous range of (window, plane) items.
+// resident CTAs.  Each CTA gets a contiguous range of (window, plane) items,
+// on the default tile after as many whole windows as every CTA can have: CTA c
+// takes the windows c, c + slots, ..., so that `slots` consecutive windows
+// march up z together and find each other's halo planes in L2 (a range starts
+// at any plane, and its neighbours' halos come from HBM: 105 bytes read per
+// cell and launch, 32 needed).  us per step, ranges only / whole windows
+// first: 411 x 411 x 738 with z walls 2184 / 1713, 640 x 640 x 64 396 / 282, 384 x
+// 384 x 96 without fluence 159 / 134, 332 x 332 x 46 without 53.7 / 48.2.
 // The ranges either have equal estimated cost -- a window-plane costs 1,
 // plus w_shell for each of the x and y shell or wall codes the window runs and
 // kCorner w_shell more for both, plus w_ant if it holds antenna columns,
@@ -123,8 +130,9 @@ static void tb2_plan(fdtd_grid* g, int RY, int slots, const TileConfig& tc, Tb2P
     P.prof = nullptr;
     P.dt16 = float(g->dt * 0.0625);
     P.err = reinterpret_cast<int*>(static_cast<char*>(g->arena) + g->L.err);
-    const int order = tc.lz == 2 && !tc.automatic ? 2 : 1;
+    const int order = tc.automatic ? 0 : (tc.lz == 2 ? 2 : 1);
     P.D = tb2_order_d(P.T, P.U, d.nz, slots, order);
+    P.whole = order == 0 ? P.T * P.U / slots : 0;
     const bool meas = tc.measured && g->tb2_ref_ry == RY && g->tb2_ref_slots == slots &&
                       g->tb2_ref_src == g->src_gen && g->tb2_refined.size() == size_t(slots) + 1 &&
                       g->tb2_ref_order == order;
@@ -163,19 +171,33 @@ static void tb2_plan(fdtd_grid* g, int RY, int slots, const TileConfig& tc, Tb2P
                 for (int m = 0; m < nw; ++m) byp[size_t(m)] = cost[size_t(tb2_window_host(P.T, P.U, P.D, m))];
                 cost.swap(byp);
             }
-            double total = 0.0;
-            for (double c : cost) total += c * (zsum + kRestart);
-            const double share = total / slots;
-            std::vector<long long> start(size_t(slots) + 1, (long long)nw * nz);
+            // the whole windows, then ranges of the others (from first on) that
+            // bring every CTA to the same cost: CTA c's share of them is what its
+            // whole windows leave below the level
+            const int first = P.whole * slots;
+            std::vector<double> own(size_t(slots), 0.0), reach(size_t(slots) + 1, 0.0);
+            for (int w = 0; w < first; ++w) own[size_t(w % slots)] += cost[size_t(w)] * (zsum + kRestart);
+            double rest = 0.0;
+            for (int w = first; w < nw; ++w) rest += cost[size_t(w)] * (zsum + kRestart);
+            std::vector<double> level(own);
+            std::sort(level.begin(), level.end());
+            double top = 0.0, below = 0.0;
+            for (int n = 1; n <= slots; ++n) {   // the n CTAs with the least share the rest
+                below += level[size_t(n) - 1];
+                top = (rest + below) / n;
+                if (n == slots || top <= level[size_t(n)]) break;
+            }
+            for (int c = 0; c < slots; ++c) reach[size_t(c) + 1] = reach[size_t(c)] + std::max(0.0, top - own[size_t(c)]);
+            std::vector<long long> start(size_t(slots) + 1, (long long)(nw - first) * nz);
             start[0] = 0;
             int c = 1;
             double cum = 0.0;
-            for (int w = 0; w < nw && c < slots; ++w) {
-                const double cw = cost[size_t(w)];
+            for (int w = 0; w < nw - first && c < slots; ++w) {
+                const double cw = cost[size_t(first + w)];
                 const double span = cw * (zsum + kRestart), base = cum + cw * kRestart;
-                while (c < slots && c * share < cum + span) {
+                while (c < slots && reach[size_t(c)] < cum + span) {
                     // the first plane whose cost from the window's start reaches the share
-                    long long k = std::lower_bound(zc.begin(), zc.end(), (c * share - base) / cw) - zc.begin();
+                    long long k = std::lower_bound(zc.begin(), zc.end(), (reach[size_t(c)] - base) / cw) - zc.begin();
                     k = std::max(0LL, std::min((long long)nz, k));
                     start[size_t(c)] = std::max(start[size_t(c) - 1], (long long)w * nz + k);
                     ++c;

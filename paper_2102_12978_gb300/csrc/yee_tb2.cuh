@@ -111,8 +111,10 @@ constexpr int kTb2MaxCtas = 512;
 // positions apart.  The host picks D so that D windows of planes are close to
 // a whole number of CTA shares: x-neighbours then start at nearly the same
 // plane and march side by side.  D = 1: row by row.
+// whole > 0: CTA c first takes the windows c, c + CTAs, ... (whole of them) from
+// plane 0 to nz; the items then are those of the windows after these.
 struct Tb2Plan {
-    int T, U, D;
+    int T, U, D, whole;
     unsigned long long* prof;
     int* err;                    // the grid's error word (an expired wait raises it)
     float dt16;                  // dt / 16
@@ -956,12 +958,20 @@ __device__ __forceinline__ void tb2_run(const StepArgs<float>& a, const TmaMaps&
     uint32_t gq = 0;
     bool dead = false;   // a wait expired: run on without waiting, the error word is raised
     const long long t0 = tw.prof ? clock64() : 0;
-    long long w = tw.start[blockIdx.x];
-    const long long wend = tw.start[blockIdx.x + 1];
-    while (w < wend) {
-        const int window = tb2_window_at(tw, int(w / a.nz)), kb = int(w % a.nz);
-        const long long left = wend - w;
-        const int ke = left < (long long)(a.nz - kb) ? kb + int(left) : a.nz;
+    const long long items = tw.start[blockIdx.x + 1] - tw.start[blockIdx.x];
+    // this CTA's work: its whole windows, then its range of items
+    for (long long w = -(long long)tw.whole * a.nz; w < items;) {
+        int window, kb, ke;
+        if (w < 0) {
+            window = int((w + (long long)tw.whole * a.nz) / a.nz) * int(gridDim.x) + int(blockIdx.x);
+            kb = 0;
+            ke = a.nz;
+        } else {
+            const long long at = tw.start[blockIdx.x] + w, left = items - w;
+            window = tw.whole * int(gridDim.x) + tb2_window_at(tw, int(at / a.nz));
+            kb = int(at % a.nz);
+            ke = left < (long long)(a.nz - kb) ? kb + int(left) : a.nz;
+        }
         // a window off the x (y) faces and shells runs without the checks of
         // the x (y) walls, psi and columns past the box
         const int wx = window % tw.T, wy = window / tw.T;

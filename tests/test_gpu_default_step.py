@@ -53,7 +53,8 @@ def _pair(shape, npml, steps, walls=False, npml_z=0, antenna=None, sheet=None, f
 
 @pytest.mark.parametrize("shape,npml", [((2, 2, 1), 0), ((4, 4, 2), 1), ((23, 19, 3), 3), ((24, 20, 4), 5),
                                         ((25, 25, 5), 6), ((47, 39, 6), 7), ((48, 40, 7), 10), ((49, 41, 33), 8),
-                                        ((97, 61, 9), 6), ((70, 130, 3), 0), ((130, 24, 12), 6), ((31, 200, 2), 4)])
+                                        ((97, 61, 9), 6), ((70, 130, 3), 0), ((130, 24, 12), 6), ((31, 200, 2), 4), ((400, 270, 4), 6),
+                                        ((505, 330, 3), 8)])
 def test_periodic_boxes(shape, npml):
     _pair(shape, npml, (6, 5))
 
