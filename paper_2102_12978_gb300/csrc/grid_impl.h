@@ -125,6 +125,7 @@ struct fdtd_grid {
         float w_shell, w_ant;
         bool measured;
     } tb2_key;                          // what they were computed for (ry 0: nothing cached)
+    int tb2_whole;                      // variant 7: windows of the plan that CTAs take whole
     std::vector<long long> tb2_refined; // variant 7: CTA ranges refined from measured per-CTA times
     int tb2_ref_ry, tb2_ref_slots;      // the window height and CTA count they are for (ry 0: none)
     int tb2_ref_src;                    // the antenna generation they were measured with

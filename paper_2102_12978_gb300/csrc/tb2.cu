@@ -96,13 +96,13 @@ static int tb2_window_host(int T, int U, int D, int pos)
 
 // CTA work ranges of variant 7 on grid g: windows of 32 x RY columns, `slots`
 // resident CTAs.  Each CTA gets a contiguous range of (window, plane) items,
-// on the default tile after as many whole windows as every CTA can have: CTA c
-// takes the windows c, c + slots, ..., so that `slots` consecutive windows
+// on the default tile after as many whole windows as every CTA can have
+// (kWholeMost): CTA c takes the windows c, c + slots, ..., so that `slots` consecutive windows
 // march up z together and find each other's halo planes in L2 (a range starts
 // at any plane, and its neighbours' halos come from HBM: 105 bytes read per
 // cell and launch, 32 needed).  us per step, ranges only / whole windows
-// first: 411 x 411 x 738 with z walls 2184 / 1713, 640 x 640 x 64 396 / 282, 384 x
-// 384 x 96 without fluence 159 / 134, 332 x 332 x 46 without 53.7 / 48.2.
+// first: 512 x 512 x 64 199 / 182, 400 x 330 x 48 88.6 / 78.0, 411 x 411 x 738 with z
+// walls 2184 / 1610; without fluence 384 x 384 x 96 159 / 134, 332 x 332 x 46 52.4 / 47.7.
 // The ranges either have equal estimated cost -- a window-plane costs 1,
 // plus w_shell for each of the x and y shell or wall codes the window runs and
 // kCorner w_shell more for both, plus w_ant if it holds antenna columns,
@@ -123,6 +123,14 @@ constexpr double kZPlane = 1.6;
 // CPML, us per step on both: 200 planes 743 / 712, 400 planes 1283 / 1376, 738
 // planes 2184 / 2486; without a z CPML, 200 planes, 480 / 686).
 constexpr int kShellPlanes = 40;
+// Whole windows first only as far as no CTA's whole windows cost more than this
+// times a CTA's mean share: few windows per CTA and the dear ones on the shell
+// would leave the others waiting (288 x 252 x 128, 156 windows on 152 SMs: 151 us
+// per step with one round of whole windows, 113 with ranges only).  us per
+// step at limits 1.0 / 1.12 / 1.18 / 1.25: 332 x 332 x 46 52.4 / 47.7 / 47.7 / 47.6,
+// 360 x 300 x 64 82.3 / 82.4 / 76.9 / 76.9, 430 x 350 x 64 87.1 / 87.1 / 86.3 / 91.9, 600 x
+// 500 x 24 87.4 / 87.4 / 87.0 / 94.5.
+constexpr double kWholeMost = 1.18;
 static void tb2_plan(fdtd_grid* g, int RY, int slots, const TileConfig& tc, Tb2Plan& P)
 {
     const fdtd_grid_desc& d = g->desc;
@@ -132,7 +140,6 @@ static void tb2_plan(fdtd_grid* g, int RY, int slots, const TileConfig& tc, Tb2P
     P.err = reinterpret_cast<int*>(static_cast<char*>(g->arena) + g->L.err);
     const int order = tc.automatic ? 0 : (tc.lz == 2 ? 2 : 1);
     P.D = tb2_order_d(P.T, P.U, d.nz, slots, order);
-    P.whole = order == 0 ? P.T * P.U / slots : 0;
     const bool meas = tc.measured && g->tb2_ref_ry == RY && g->tb2_ref_slots == slots &&
                       g->tb2_ref_src == g->src_gen && g->tb2_refined.size() == size_t(slots) + 1 &&
                       g->tb2_ref_order == order;
@@ -142,6 +149,7 @@ static void tb2_plan(fdtd_grid* g, int RY, int slots, const TileConfig& tc, Tb2P
         (meas ? key.cost_gen != g->tb2_ref_gen : (key.w_shell != tc.w_shell || key.w_ant != tc.w_ant))) {
         if (meas) {
             g->tb2_start = g->tb2_refined;
+            g->tb2_whole = 0;
         } else {
             const int nx = d.nx, ny = d.ny, nz = d.nz, npml = d.npml;
             const int nw = P.T * P.U;
@@ -174,10 +182,18 @@ static void tb2_plan(fdtd_grid* g, int RY, int slots, const TileConfig& tc, Tb2P
             // the whole windows, then ranges of the others (from first on) that
             // bring every CTA to the same cost: CTA c's share of them is what its
             // whole windows leave below the level
-            const int first = P.whole * slots;
-            std::vector<double> own(size_t(slots), 0.0), reach(size_t(slots) + 1, 0.0);
-            for (int w = 0; w < first; ++w) own[size_t(w % slots)] += cost[size_t(w)] * (zsum + kRestart);
             double rest = 0.0;
+            for (int w = 0; w < nw; ++w) rest += cost[size_t(w)] * (zsum + kRestart);
+            const double most = kWholeMost * rest / slots;
+            std::vector<double> own(size_t(slots), 0.0), reach(size_t(slots) + 1, 0.0);
+            int first = order == 0 ? nw / slots * slots : 0;
+            for (;; first -= slots) {
+                std::fill(own.begin(), own.end(), 0.0);
+                for (int w = 0; w < first; ++w) own[size_t(w % slots)] += cost[size_t(w)] * (zsum + kRestart);
+                if (first == 0 || *std::max_element(own.begin(), own.end()) <= most) break;
+            }
+            g->tb2_whole = first;
+            rest = 0.0;
             for (int w = first; w < nw; ++w) rest += cost[size_t(w)] * (zsum + kRestart);
             std::vector<double> level(own);
             std::sort(level.begin(), level.end());
@@ -210,6 +226,7 @@ static void tb2_plan(fdtd_grid* g, int RY, int slots, const TileConfig& tc, Tb2P
         key.w_shell = tc.w_shell; key.w_ant = tc.w_ant;
         key.measured = meas; key.cost_gen = g->tb2_ref_gen; key.order = order;
     }
+    P.whole = g->tb2_whole;
     for (int c = 0; c <= slots; ++c) P.start[c] = g->tb2_start[size_t(c)];
 }
 

@@ -111,8 +111,8 @@ constexpr int kTb2MaxCtas = 512;
 // positions apart.  The host picks D so that D windows of planes are close to
 // a whole number of CTA shares: x-neighbours then start at nearly the same
 // plane and march side by side.  D = 1: row by row.
-// whole > 0: CTA c first takes the windows c, c + CTAs, ... (whole of them) from
-// plane 0 to nz; the items then are those of the windows after these.
+// whole > 0: CTA c first takes the windows c, c + CTAs, ... below whole, from
+// plane 0 to nz; the items then are those of the windows from whole on.
 struct Tb2Plan {
     int T, U, D, whole;
     unsigned long long* prof;
@@ -958,20 +958,34 @@ __device__ __forceinline__ void tb2_run(const StepArgs<float>& a, const TmaMaps&
     uint32_t gq = 0;
     bool dead = false;   // a wait expired: run on without waiting, the error word is raised
     const long long t0 = tw.prof ? clock64() : 0;
-    const long long items = tw.start[blockIdx.x + 1] - tw.start[blockIdx.x];
-    // this CTA's work: its whole windows, then its range of items
-    for (long long w = -(long long)tw.whole * a.nz; w < items;) {
-        int window, kb, ke;
-        if (w < 0) {
-            window = int((w + (long long)tw.whole * a.nz) / a.nz) * int(gridDim.x) + int(blockIdx.x);
-            kb = 0;
-            ke = a.nz;
-        } else {
-            const long long at = tw.start[blockIdx.x] + w, left = items - w;
-            window = tw.whole * int(gridDim.x) + tb2_window_at(tw, int(at / a.nz));
-            kb = int(at % a.nz);
-            ke = left < (long long)(a.nz - kb) ? kb + int(left) : a.nz;
+    // this CTA's work: its whole windows, then its range of items.  The first
+    // thread keeps the place in shared memory: held in registers over the z
+    // march it spills there (FL: 145 us per step at 256 x 256 x 128, 104 so).
+    __shared__ long long at;     // the next item
+    __shared__ int pos, work[3]; // the next whole window; window, kb, ke of this turn
+    if (threadIdx.x == 0) {
+        pos = blockIdx.x;
+        at = tw.start[blockIdx.x];
+    }
+    for (;;) {
+        if (threadIdx.x == 0) {
+            if (pos < tw.whole) {
+                work[0] = tb2_window_at(tw, pos);
+                work[1] = 0;
+                work[2] = a.nz;
+                pos += gridDim.x;
+            } else {
+                const long long left = tw.start[blockIdx.x + 1] - at;
+                const int kb = int(at % a.nz), n = left < (long long)(a.nz - kb) ? int(left) : a.nz - kb;
+                work[0] = n > 0 ? tb2_window_at(tw, tw.whole + int(at / a.nz)) : -1;
+                work[1] = kb;
+                work[2] = kb + n;
+                at += n;
+            }
         }
+        __syncthreads();
+        const int window = work[0], kb = work[1], ke = work[2];
+        if (window < 0) break;
         // a window off the x (y) faces and shells runs without the checks of
         // the x (y) walls, psi and columns past the box
         const int wx = window % tw.T, wy = window / tw.T;
@@ -982,7 +996,6 @@ __device__ __forceinline__ void tb2_run(const StepArgs<float>& a, const TmaMaps&
         else if (!gy) tb2_window<RY, 1, W, CR, FL>(a, m, tt, tw, window, kb, ke, b, gq, dead);
         else if (!gx) tb2_window<RY, 2, W, CR, FL>(a, m, tt, tw, window, kb, ke, b, gq, dead);
         else tb2_window<RY, 3, W, CR, FL>(a, m, tt, tw, window, kb, ke, b, gq, dead);
-        w += ke - kb;
         __syncthreads();   // the ring and the exchange buffers are reused by the next window
     }
     if (dead) {   // copies may still be in flight: give each slot's last phase one more bounded wait
