@@ -109,10 +109,12 @@ bool compute_layout(const fdtd_grid_desc& d, Layout& L)
     L.psz_elems = w2z * ny * p;
     for (int buf = 0; buf < 2; ++buf)
         for (int c = 0; c < 2; ++c) L.phz[buf][c] = take(L.psz_elems * b);
-    for (int buf = 0; buf < 2; ++buf)
-        for (int c = 0; c < 2; ++c) L.pez[buf][c] = take(L.psz_elems * b);
+    for (int c = 0; c < 2; ++c) L.pez[0][c] = take(L.psz_elems * b);
     L.fluence = d.fluence ? take(nz * ny * p * 8) : 0;
     L.dynamic_bytes = off;
+    // the second copy of the z shells' E psi (two-step kernel only) is not part
+    // of a saved state: a state holds the current copy in the first one's place
+    for (int c = 0; c < 2; ++c) L.pez[1][c] = d.precision == FDTD_F32 ? take(L.psz_elems * b) : L.pez[0][c];
     L.chx = take(nx * b); L.cex = take(nx * b);
     L.chy = take(ny * b); L.cey = take(ny * b);
     L.chz = take(nz * b); L.cez = take(nz * b);
@@ -1009,6 +1011,20 @@ fdtd_status fdtd_set_field(fdtd_grid* g, int component, const void* src, int on_
     return fdtd_sync(g);
 }
 
+// The current z-shell E psi between the arena's second copy and its place in a
+// saved state (nothing to do where the first copy is current).
+static cudaError_t copy_pez(fdtd_grid* g, char* state, bool save)
+{
+    cudaError_t e = cudaSuccess;
+    for (int c = 0; c < 2 && g->pe == 1 && g->L.pez[1][c] != g->L.pez[0][c] && e == cudaSuccess; ++c) {
+        char* mine = static_cast<char*>(g->arena) + g->L.pez[1][c];
+        char* theirs = state + g->L.pez[0][c];
+        e = cudaMemcpyAsync(save ? theirs : mine, save ? mine : theirs, g->L.psz_elems * g->L.elem,
+                            cudaMemcpyDeviceToDevice, g->stream);
+    }
+    return e;
+}
+
 size_t fdtd_state_bytes(const fdtd_grid* g)
 {
     if (!g) return 0;
@@ -1020,10 +1036,11 @@ fdtd_status fdtd_save_state(fdtd_grid* g, void* dev_dst)
     if (!g || !dev_dst) return fail(FDTD_EINVAL, "null argument");
     const fdtd_status dev_st = check_device(g, "fdtd_save_state");
     if (dev_st != FDTD_OK) return dev_st;
-    int64_t hdr[5] = {g->step, g->cur, 0x46445444, g->pe, g->flip};
+    int64_t hdr[4] = {g->step, g->cur, 0x46445444, g->pe | g->flip << 1};
     char* D = static_cast<char*>(dev_dst);
     fdtd_status st = cuda_check(cudaMemcpyAsync(D, g->arena, g->L.dynamic_bytes, cudaMemcpyDeviceToDevice,
                                                 g->stream), "save state");
+    if (st == FDTD_OK) st = cuda_check(copy_pez(g, D, true), "save state");
     if (st == FDTD_OK)
         st = cuda_check(cudaMemcpyAsync(D + g->L.dynamic_bytes, hdr, sizeof(hdr), cudaMemcpyHostToDevice,
                                         g->stream), "save state");
@@ -1036,22 +1053,23 @@ fdtd_status fdtd_load_state(fdtd_grid* g, const void* dev_src)
     if (!g || !dev_src) return fail(FDTD_EINVAL, "null argument");
     const fdtd_status dev_st = check_device(g, "fdtd_load_state");
     if (dev_st != FDTD_OK) return dev_st;
-    int64_t hdr[5];
+    int64_t hdr[4];
     const char* S = static_cast<const char*>(dev_src);
     fdtd_status st = cuda_check(cudaMemcpyAsync(hdr, S + g->L.dynamic_bytes, sizeof(hdr), cudaMemcpyDeviceToHost,
                                                 g->stream), "load state");
     if (st == FDTD_OK) st = fdtd_sync(g);
     if (st != FDTD_OK) return st;
-    if (hdr[2] != 0x46445444 || (hdr[1] != 0 && hdr[1] != 1) || (hdr[3] != 0 && hdr[3] != 1) ||
-        (hdr[4] != 0 && hdr[4] != 1))
+    if (hdr[2] != 0x46445444 || (hdr[1] != 0 && hdr[1] != 1) || hdr[3] < 0 || hdr[3] > 3)
         return fail(FDTD_EINVAL, "state blob does not come from fdtd_save_state");
     st = cuda_check(cudaMemcpyAsync(g->arena, S, g->L.dynamic_bytes, cudaMemcpyDeviceToDevice, g->stream),
                     "load state");
     if (st != FDTD_OK) return st;
     g->step = hdr[0];
     g->cur = int(hdr[1]);
-    g->pe = int(hdr[3]);
-    g->flip = int(hdr[4]);
+    g->pe = int(hdr[3] & 1);
+    g->flip = int(hdr[3] >> 1);
+    st = cuda_check(copy_pez(g, const_cast<char*>(S), false), "load state");
+    if (st != FDTD_OK) return st;
     return fdtd_sync(g);
 }
 

@@ -97,6 +97,28 @@ def test_checkpoint_between_the_routes():
     assert torch.equal(a.fluence(), b.fluence())
 
 
+@pytest.mark.parametrize("npml_z,before", [(3, 2), (5, 4), (3, 3)])
+def test_z_walled_state_holds_the_current_psi(npml_z, before):
+    """A pair of steps leaves the z shells' E psi in the other copy; a state saved
+    there goes on alike in a grid that stands on the first copy, and back."""
+    shape = (26, 23, 40 * npml_z + 3)
+    a, _ = _pair(shape, 4, (before,), walls=True, npml_z=npml_z)
+    b, _ = _pair(shape, 4, (4,), walls=True, npml_z=npml_z, seed=5)
+    state, other = a.save_state(), b.save_state()
+    a.step(5)
+    b.load_state(state)
+    b.step(5)
+    for c in range(6):
+        assert torch.equal(a.field(c), b.field(c)), c
+    assert torch.equal(a.fluence(), b.fluence())
+    a.load_state(other)
+    b.load_state(other)
+    a.step(3)
+    b.step(3)
+    for c in range(6):
+        assert torch.equal(a.field(c), b.field(c)), c
+
+
 def test_batch_after_steps_and_a_state_loaded_into_a_batched_grid():
     """A batch reads the E-side psi copy its grids are at, also after a state
     of the other copy is loaded into a batched grid."""
