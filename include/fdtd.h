@@ -101,8 +101,8 @@ typedef struct {
 
 /* z boundary.  FDTD_Z_WALLS puts PEC walls at z = 0 and z = nz dz (tangential
  * E_x, E_y zero on the plane k = 0; fields past the last plane read as the
- * wall) with npml_z CPML cells inside each.  A z-walled grid runs on tile
- * variant 5 and the cell batch engines only
+ * wall) with npml_z CPML cells inside each.  A z-walled grid runs on its
+ * default tile, on tile variant 5 and in the cell batch engines only
  * (EINVAL elsewhere), takes no antenna (the antenna boxes are z-periodic,
  * Section 4) and has no adjoint (EINVAL). */
 enum { FDTD_Z_PERIODIC = 0, FDTD_Z_WALLS = 1 };
@@ -254,18 +254,18 @@ int64_t fdtd_antenna_points(const fdtd_grid* g, int component);
  *      that x-neighbouring windows march side by side, any other lz takes
  *      the windows row by row): windows of 32 x 24 columns (ty 16; 32 x 12
  *      with ty 8) march along z, recomputing their halo columns, so that
- *      fields, psi and the fluence cross HBM once per two steps.  An odd step count ends with
- *      one step of variant 5.  The CTAs' shares of the work are balanced on
+ *      fields, psi and the fluence cross HBM once per two steps.  An odd
+ *      step count ends with one step of variant 5.  The CTAs' shares of the work are balanced on
  *      per-window costs (fdtd_set_balance).
  * The TMA variants (1, 2, 4) have no FP64 32x16 tile (EINVAL).  A z-walled
  * grid or one with a wall source takes variant 5 only (EINVAL otherwise;
  * fdtd_autotune then times the ty of variant 5 only).
  * fdtd_create_grid picks a default (variant 5, ty 4).  As long as no tile is
  * chosen, an FP32 grid (z-walled ones from 40 planes per cell of a z face's
- * CPML on) takes its pairs of steps with the two-step kernel instead, which
+ * CPML on, from 6 for boxes of some 330 x 330 cells or more) takes its pairs of steps with the two-step kernel instead, which
  * then rounds every operation as variant 5 does: the results are variant 5's,
- * bit for bit.  fdtd_autotune times
- * the candidates on this grid (running `steps` steps for each, then
+ * bit for bit.  Its CTAs then take whole windows first and split the rest by
+ * estimated cost (fdtd_set_balance).  fdtd_autotune times the candidates on this grid (running `steps` steps for each, then
  * restoring the state) and keeps the fastest.  Results agree to rounding
  * for every configuration. */
 fdtd_status fdtd_set_tile(fdtd_grid* g, int variant, int ty, int lz);
@@ -276,8 +276,8 @@ fdtd_status fdtd_set_tile(fdtd_grid* g, int variant, int ty, int lz);
  * for both), plus w_antenna if it holds antenna columns, and each CTA takes a
  * contiguous range of (window, plane) work of equal estimated cost; a window
  * also costs some planes at its start (the two-step wavefront refills
- * there).  Weights in [0, 16] (else EINVAL); defaults 0.4 and 0.2.  fdtd_autotune times a few pairs, then refines the fastest pair's
- * ranges on measured times (fdtd_measure_balance), with the windows row by
+ * there).  Weights in [0, 16] (else EINVAL); defaults 0.4 and 0.2.
+ * fdtd_autotune times a few pairs, then refines the fastest pair's ranges on measured times (fdtd_measure_balance), with the windows row by
  * row and interleaved (lz 1 and 2), and times those; it keeps the fastest.
  * While refined ranges are in use, fdtd_get_balance returns -1 for both
  * weights; fdtd_set_balance returns to the weights.  The results do not
@@ -400,7 +400,8 @@ int fdtd_batch_get_engine(const fdtd_batch* b);
  * an unknown mode or the two-step mode on a grid that cannot take it.  The
  * default is FDTD_BATCH_MODE_CELL4; as long as no mode is chosen (and the batch
  * is not tuned), grids that would take the two-step kernel on their default
- * tile (fdtd_set_tile) take it in the graph too, with the same results.  -1 from the getter for a bad index. */
+ * tile (fdtd_set_tile) take it in the graph too, with the same results (the
+ * getter keeps naming the cell mode).  -1 from the getter for a bad index. */
 fdtd_status fdtd_batch_set_grid_mode(fdtd_batch* b, int q, int mode);
 int fdtd_batch_get_grid_mode(const fdtd_batch* b, int q);
 /* CTAs of grid q's two-step launches in the graph engine (-1 for a bad index). */

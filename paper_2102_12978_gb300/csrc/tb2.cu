@@ -119,10 +119,16 @@ constexpr double kCorner = 0.4;
 constexpr double kZPlane = 1.6;
 // A z-walled grid takes the two-step kernel from this many planes per CPML
 // cell of a z face on: a z-shell plane costs it about four inner ones, so
-// that short boxes run faster on the cell passes (411 x 411 cells, 16-cell z
-// CPML, us per step on both: 200 planes 743 / 712, 400 planes 1283 / 1376, 738
-// planes 2184 / 2486; without a z CPML, 200 planes, 480 / 686).
-constexpr int kShellPlanes = 40;
+// that short boxes run faster on the cell passes.  The line lies lower for
+// boxes of at least kManyWindows windows per SM, whose windows march together.
+// us per step, two-step / cell passes, 16-cell z CPML, at 4, 6, 12 and 24 planes
+// per cell: 411 x 411 234 / 263, 315 / 367, 526 / 685, 938 / 1320; 340 x 335 (255
+// windows) 171 / 183, 226 / 256, 392 / 472, 697 / 907; 300 x 300 (195 windows) 187 /
+// 156, 250 / 216, 444 / 403, 739 / 772; 205 x 211 104 / 83, 142 / 115, 229 / 210, 405 / 402;
+// 100 x 91 30 / 25, 43 / 33, 75 / 63, 130 / 117.  6-cell z CPML, 340 x 335: 82 / 73 at
+// 4, 99 / 101 at 6.
+constexpr int kShellPlanes = 40, kShellPlanesMany = 6;
+constexpr double kManyWindows = 1.5;
 // Whole windows first only as far as no CTA's whole windows cost more than this
 // times a CTA's mean share: few windows per CTA and the dear ones on the shell
 // would leave the others waiting (288 x 252 x 128, 156 windows on 152 SMs: 151 us
@@ -264,14 +270,18 @@ static cudaError_t tb2_blocks_per_sm(int* out)
 
 // Every FP32 box but short z-walled ones: the two-step kernel is the faster
 // one, or as fast, at every size measured (us per step, two-step / cell passes:
-// 16 x 16 x 8 7.2 / 8.2; 48 x 40 x 16 8.2 / 9.1; 64 x 64 x 32 10.3 / 10.3;
-// 96 x 96 x 64 15 / 18; 160 x 160 x 64 27 / 41; 332 x 332 x 46 66 / 111;
-// 640 x 640 x 64 352 / 514; 560 x 560 x 5 36 / 36).
+// 16 x 16 x 8 7.3 / 8.3; 48 x 40 x 16 8.3 / 8.3; 64 x 64 x 32 10.3 / 10.3;
+// 96 x 96 x 64 15 / 18; 160 x 160 x 64 27 / 40; 332 x 332 x 46 62 / 112;
+// 640 x 640 x 64 261 / 525; 560 x 560 x 5 36 / 36).
 bool default_two_step(const fdtd_grid* g)
 {
     const fdtd_grid_desc& d = g->desc;
     if (d.precision != FDTD_F32) return false;
-    return d.z_boundary != FDTD_Z_WALLS || d.nz >= kShellPlanes * d.npml_z;
+    if (d.z_boundary != FDTD_Z_WALLS) return true;
+    int T, U;
+    tb2_windows(d, kTb2Rows, &T, &U);
+    const bool many = double(T) * U >= kManyWindows * (g->sm_count > 0 ? g->sm_count : 152);
+    return d.nz >= (many ? kShellPlanesMany : kShellPlanes) * d.npml_z;
 }
 
 int tb2_slots(const fdtd_grid* g, int ty)

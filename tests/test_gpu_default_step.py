@@ -59,7 +59,7 @@ def test_periodic_boxes(shape, npml):
     _pair(shape, npml, (6, 5))
 
 
-@pytest.mark.parametrize("shape,npml,npml_z", [((24, 20, 2), 3, 0), ((25, 41, 12), 5, 5), ((49, 39, 13), 6, 3),
+@pytest.mark.parametrize("shape,npml,npml_z", [((24, 20, 2), 3, 0), ((25, 41, 12), 5, 5), ((49, 39, 13), 6, 3), ((345, 330, 14), 5, 2),
                                                ((48, 61, 40), 4, 8), ((96, 22, 9), 0, 2), ((33, 33, 200), 6, 16)])
 def test_z_walled_boxes(shape, npml, npml_z):
     sheet = dict(theta=0.4, w0=0.7, envelope="cw", ramp=0.2, plane=max(1, npml_z))
