@@ -11,7 +11,8 @@
 //     cell-parallel H and E passes of tile variant 5 on 32 x 4, 8 or 16
 //     blocks, or (FP32 z-periodic grids without a wall sheet) the two-step
 //     kernel of tile variant 7 on a share of the SMs proportional to its
-//     cells.  The per-step source time factors of every grid are evaluated on
+//     cells.  Until a mode is chosen, the grids whose default tile takes the
+//     two-step kernel do so here too, with the same bits.  The per-step source time factors of every grid are evaluated on
 //     the host in FP64, as for a single grid, and copied into a device table
 //     ahead of each replay; the kernels read their steps' entries.
 //   * persistent cell passes (FDTD_BATCH_PERSISTENT_CELL): one cooperative
@@ -549,6 +550,31 @@ void two_step_ctas(fdtd_batch* b, bool shared)
     }
 }
 
+// The same while no mode has been chosen: a grid of at least as many windows
+// as SMs takes every SM (its windows then march together, see tb2_plan), the
+// smaller ones take shares among themselves.  us per step, shares of all
+// cells / every grid on all SMs / this rule: 2 x (640^2, 320^2, 160^2, 96^2) x 64
+// 886 / 720 / 709, 3 x 320^2 x 64 251 / 220 / 220, 12 x 96^2 x 16 37 / 76 / 37,
+// 3 x (96^2, 160^2) x 64 102 / 109 / 102.
+void automatic_ctas(fdtd_batch* b)
+{
+    two_step_ctas(b, true);
+    const int sms = b->grids[0]->sm_count > 0 ? b->grids[0]->sm_count : 152;
+    double small = 0.0;
+    auto windows = [](const fdtd_grid* g) {
+        int t, u;
+        tb2_windows(g->desc, kTb2Rows, &t, &u);
+        return t * u;
+    };
+    auto cells = [](const fdtd_grid* g) { return double(g->desc.nx) * g->desc.ny * g->desc.nz; };
+    for (const fdtd_grid* g : b->grids)
+        if (windows(g) < sms) small += cells(g);
+    for (size_t q = 0; q < b->grids.size(); ++q) {
+        const fdtd_grid* g = b->grids[q];
+        b->ctas[q] = windows(g) >= sms ? sms : std::max(8, std::min(sms, int(cells(g) / small * sms + 0.5)));
+    }
+}
+
 bool two_step_eligible(const fdtd_batch* b, int q)
 {
     return b->precision == FDTD_F32 && !has_walls(b->grids[size_t(q)]);
@@ -597,7 +623,7 @@ fdtd_status fdtd_batch_create(fdtd_grid* const* grids, int n, void* dev_table, s
     b->fault = 0;
     b->mode.assign(size_t(n), kModeCell4);
     b->automatic = true;
-    two_step_ctas(b, true);
+    automatic_ctas(b);
     b->built[0] = b->built[1] = false;
     fdtd_status st = cuda_check(cudaStreamCreateWithFlags(&b->capture, cudaStreamNonBlocking), "capture stream");
     if (st != FDTD_OK) { delete b; return st; }
@@ -654,6 +680,7 @@ fdtd_status fdtd_batch_set_grid_mode(fdtd_batch* b, int q, int mode)
         return fail(FDTD_EINVAL, "the two-step mode takes FP32 z-periodic grids without a wall source");
     if (b->mode[size_t(q)] != mode || b->automatic) {
         b->mode[size_t(q)] = mode;
+        if (b->automatic) two_step_ctas(b, true);
         b->automatic = false;
         drop_graphs(b);
     }
