@@ -64,7 +64,10 @@
 //     the x (y) walls, psi and columns past the box (template flags GX, GY).
 //     A plane of an inner window takes 2400 cycles, of an x- or y-shell window
 //     3400, of a corner 4700.
-//   * A CTA takes a contiguous range of the flattened (window, plane) work:
+//   * On the default tile a CTA takes whole windows first, so that
+//     neighbouring windows march together and share halo planes in L2, then a
+//     range of what is left (tb2_plan).  On explicit tiles it takes
+//     a contiguous range of the flattened (window, plane) work:
 //     ranges of equal estimated cost (windows with CPML shell or antenna
 //     columns weigh more, with weights the autotuner picks by timing), or
 //     ranges the host refined until the CTAs' measured times were equal
@@ -79,8 +82,8 @@
 //     (W), whose planes off the z shells run the loop above with the walls'
 //     few extra tests; z-shell planes run apart.
 // FP32 fields with the Kahan FP32 fluence.  256 x 256 x 128 cells with a
-// 16-cell CPML, antenna and fluence: 101-105 us per step (one column per
-// thread, windows of 32 x 16 with 28 x 12 own columns: 122-130 us).
+// 16-cell CPML, antenna and fluence: 104 us per step (one column per thread,
+// windows of 32 x 16 with 28 x 12 own columns: 122-130 us); 512 x 512 x 64: 182 us.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>

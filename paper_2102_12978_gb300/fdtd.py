@@ -478,7 +478,8 @@ class Batch:
     """Several Grid objects advanced together (fdtd_batch_*): engine
     BATCH_CELL (a 64-step CUDA graph with one branch per grid, each grid in
     its own mode: cell passes on 32 x 4 / 8 / 16 blocks or the two-step
-    kernel; the default) or BATCH_PERSISTENT_CELL (one cooperative launch
+    kernel; until a mode is chosen, whichever the grid's default tile takes;
+    the default) or BATCH_PERSISTENT_CELL (one cooperative launch
     per 64 steps)."""
 
     def __init__(self, grids, engine: int | None = None):
