@@ -262,12 +262,13 @@ int64_t fdtd_antenna_points(const fdtd_grid* g, int component);
  * fdtd_autotune then times the ty of variant 5 only).
  * fdtd_create_grid picks a default (variant 5, ty 4).  As long as no tile is
  * chosen, an FP32 grid (z-walled ones from 40 planes per cell of a z face's
- * CPML on, from 6 for boxes of some 330 x 330 cells or more) takes its pairs of steps with the two-step kernel instead, which
- * then rounds every operation as variant 5 does: the results are variant 5's,
- * bit for bit.  Its CTAs then take whole windows first and split the rest by
- * estimated cost (fdtd_set_balance).  fdtd_autotune times the candidates on this grid (running `steps` steps for each, then
- * restoring the state) and keeps the fastest.  Results agree to rounding
- * for every configuration. */
+ * CPML on, from 6 for boxes of some 330 x 330 cells or more) takes its pairs
+ * of steps with the two-step kernel instead, which then rounds every
+ * operation as variant 5 does: the results are variant 5's, bit for bit.  Its
+ * CTAs then take whole windows first and split the rest by estimated cost
+ * (fdtd_set_balance).  fdtd_autotune times the candidates on this grid
+ * (running `steps` steps for each, then restoring the state) and keeps the
+ * fastest.  Results agree to rounding for every configuration. */
 fdtd_status fdtd_set_tile(fdtd_grid* g, int variant, int ty, int lz);
 
 /* Work-split weights of tile variant 7 (the paper has no counterpart): a
@@ -277,11 +278,12 @@ fdtd_status fdtd_set_tile(fdtd_grid* g, int variant, int ty, int lz);
  * contiguous range of (window, plane) work of equal estimated cost; a window
  * also costs some planes at its start (the two-step wavefront refills
  * there).  Weights in [0, 16] (else EINVAL); defaults 0.4 and 0.2.
- * fdtd_autotune times a few pairs, then refines the fastest pair's ranges on measured times (fdtd_measure_balance), with the windows row by
- * row and interleaved (lz 1 and 2), and times those; it keeps the fastest.
- * While refined ranges are in use, fdtd_get_balance returns -1 for both
- * weights; fdtd_set_balance returns to the weights.  The results do not
- * depend on the balance, only the time does. */
+ * fdtd_autotune times a few pairs, then refines the fastest pair's ranges on
+ * measured times (fdtd_measure_balance), with the windows row by row and
+ * interleaved (lz 1 and 2), and times those; it keeps the fastest. While
+ * refined ranges are in use, fdtd_get_balance returns -1 for both weights;
+ * fdtd_set_balance returns to the weights.  The results do not depend on the
+ * balance, only the time does. */
 fdtd_status fdtd_set_balance(fdtd_grid* g, float w_shell, float w_antenna);
 fdtd_status fdtd_get_balance(const fdtd_grid* g, float* w_shell, float* w_antenna);
 /* Refine the CTAs' work ranges of the grid's variant-7 tile on measured

@@ -12,9 +12,10 @@
 //     blocks, or (FP32 z-periodic grids without a wall sheet) the two-step
 //     kernel of tile variant 7 on a share of the SMs proportional to its
 //     cells.  Until a mode is chosen, the grids whose default tile takes the
-//     two-step kernel do so here too, with the same bits.  The per-step source time factors of every grid are evaluated on
-//     the host in FP64, as for a single grid, and copied into a device table
-//     ahead of each replay; the kernels read their steps' entries.
+//     two-step kernel do so here too, with the same bits.  The per-step
+//     source time factors of every grid are evaluated on the host in FP64, as
+//     for a single grid, and copied into a device table ahead of each replay;
+//     the kernels read their steps' entries.
 //   * persistent cell passes (FDTD_BATCH_PERSISTENT_CELL): one cooperative
 //     kernel launch runs up to K steps of every grid.  The 32 x 4 cell
 //     blocks of all grids form one list; the CTAs (one per resident slot)
