@@ -316,6 +316,11 @@ fdtd_status fdtd_measure_balance(fdtd_grid* g, void* scratch_state);
 int fdtd_debug_tb2_order(int t, int u, int nz, int slots, int order, int* out);
 fdtd_status fdtd_debug_tb2_refine(int slots, const long long* starts, const unsigned long long* cycles, double step,
                                   long long* out);
+/* Test hook (no device work; the paper has no counterpart): the bookkeeping of
+ * what the two-step kernel sets up once per device of the process.  Call q
+ * comes from device devices[q]; a set-up, if one runs, gives results[q] (0:
+ * it fails).  values[q] is what the call then works with (-1: the failure). */
+fdtd_status fdtd_debug_per_device(const int* devices, const int* results, int n, int* values);
 
 /* Measurement (the paper has no counterpart): advance `nsteps` steps like
  * fdtd_step and time every kernel launch of a step with CUDA events recorded

@@ -2,6 +2,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstddef>
 #include <cstdint>
 #include <vector>
@@ -58,6 +59,34 @@ struct TileConfig {
     // the default tile, chosen by nobody: runs of steps take the two-step
     // kernel where it is the faster one (default_two_step)
     bool automatic = false;
+};
+
+// A positive number that is made once per device of the process.  A kernel's
+// attributes (the opt-in to more than 48 KB of dynamic shared memory, and the
+// residency that follows) belong to one device's copy of it: a second device
+// needs its own.
+class PerDevice {
+public:
+    // make(&n) sets the device up; run on the device's first call and again
+    // until it succeeds (by each thread that comes before the first is done:
+    // make may be repeated).
+    template <typename F>
+    cudaError_t get(int device, int* out, F&& make)
+    {
+        const bool kept = device >= 0 && device < kDevices;
+        int n = kept ? value_[device].load() : 0;
+        if (n == 0) {
+            const cudaError_t e = make(&n);
+            if (e != cudaSuccess) return e;
+            if (kept) value_[device].store(n);
+        }
+        *out = n;
+        return cudaSuccess;
+    }
+
+private:
+    static constexpr int kDevices = 64;
+    std::atomic<int> value_[kDevices] = {};
 };
 
 fdtd_status fail(fdtd_status st, const char* fmt, ...);

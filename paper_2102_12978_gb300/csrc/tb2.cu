@@ -5,7 +5,6 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 
 #include "grid_impl.h"
@@ -236,15 +235,15 @@ static void tb2_plan(fdtd_grid* g, int RY, int slots, const TileConfig& tc, Tb2P
     for (int c = 0; c <= slots; ++c) P.start[c] = g->tb2_start[size_t(c)];
 }
 
-// Resident CTAs per SM of the kernels of one RY (dynamic shared memory set
-// on first use).
+// Resident CTAs per SM of the kernels of one RY on the device `device`, the
+// current one (dynamic shared memory set on the device's first use).
 template <int RY>
-static cudaError_t tb2_blocks_per_sm(int* out)
+static cudaError_t tb2_blocks_per_sm(int device, int* out)
 {
     using S = Tb2Smem<RY>;
     static_assert(S::bytes() <= 232448, "the window's shared memory exceeds the 227 KB a CTA can hold");
-    static std::atomic<int> blocks_per_sm{0};
-    if (blocks_per_sm.load() == 0) {
+    static PerDevice blocks_per_sm;
+    return blocks_per_sm.get(device, out, [](int* n) {
         const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
         const int bytes = int(S::bytes());
         cudaError_t e = cudaFuncSetAttribute(yee_tb2<RY, false, false, true>, at, bytes);
@@ -258,14 +257,9 @@ static cudaError_t tb2_blocks_per_sm(int* out)
             if (e == cudaSuccess) e = cudaFuncSetAttribute(yee_tb2_t<RY, true, true, true>, at, bytes);
         }
         if (e != cudaSuccess) return e;
-        int n = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, yee_tb2<RY, false, false, true>, S::NT, S::bytes());
-        if (e != cudaSuccess) return e;
-        if (n < 1) return cudaErrorInvalidConfiguration;
-        blocks_per_sm.store(n);
-    }
-    *out = blocks_per_sm.load();
-    return cudaSuccess;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, yee_tb2<RY, false, false, true>, S::NT, S::bytes());
+        return e == cudaSuccess && *n < 1 ? cudaErrorInvalidConfiguration : e;
+    });
 }
 
 // Every FP32 box but short z-walled ones: the two-step kernel is the faster
@@ -287,7 +281,8 @@ bool default_two_step(const fdtd_grid* g)
 int tb2_slots(const fdtd_grid* g, int ty)
 {
     int per_sm = 0;
-    const cudaError_t e = ty == 8 ? tb2_blocks_per_sm<kTb2RowsSmall>(&per_sm) : tb2_blocks_per_sm<kTb2Rows>(&per_sm);
+    const cudaError_t e = ty == 8 ? tb2_blocks_per_sm<kTb2RowsSmall>(g->device, &per_sm)
+                                   : tb2_blocks_per_sm<kTb2Rows>(g->device, &per_sm);
     if (e != cudaSuccess) return -1;
     return std::min(kTb2MaxCtas, (g->sm_count > 0 ? g->sm_count : 152) * per_sm);
 }
@@ -322,7 +317,7 @@ static cudaError_t launch_tb2_t(const fdtd_grid* cg, int cur, long long n, const
     fdtd_grid* g = const_cast<fdtd_grid*>(cg);
     using S = Tb2Smem<RY>;
     int per_sm = 0;
-    cudaError_t e = tb2_blocks_per_sm<RY>(&per_sm);
+    cudaError_t e = tb2_blocks_per_sm<RY>(g->device, &per_sm);
     if (e != cudaSuccess) return e;
     const int slots = std::min(kTb2MaxCtas, (g->sm_count > 0 ? g->sm_count : 152) * per_sm);
     Tb2Plan plan;
@@ -372,7 +367,7 @@ cudaError_t launch_tb2_table(const fdtd_grid* cg, int cur, const StepTime<float>
     constexpr int RY = kTb2Rows;
     using S = Tb2Smem<RY>;
     int per_sm = 0;
-    cudaError_t e = tb2_blocks_per_sm<RY>(&per_sm);
+    cudaError_t e = tb2_blocks_per_sm<RY>(g->device, &per_sm);
     if (e != cudaSuccess) return e;
     const int all = std::min(kTb2MaxCtas, (g->sm_count > 0 ? g->sm_count : 152) * per_sm);
     const int slots = std::max(1, std::min(all, max_ctas));
@@ -402,6 +397,21 @@ int fdtd_debug_tb2_order(int t, int u, int nz, int slots, int order, int* out)
     const int D = tb2_order_d(t, u, nz, slots, order == 2 ? 2 : 1);
     for (int m = 0; m < t * u; ++m) out[m] = tb2_window_host(t, u, D, m);
     return D;
+}
+
+fdtd_status fdtd_debug_per_device(const int* devices, const int* results, int n, int* values)
+{
+    if (!devices || !results || !values || n < 1) return fail(FDTD_EINVAL, "invalid argument");
+    PerDevice p;
+    for (int q = 0; q < n; ++q) {
+        values[q] = 0;
+        const cudaError_t e = p.get(devices[q], &values[q], [&](int* v) {
+            *v = results[q];
+            return results[q] > 0 ? cudaSuccess : cudaErrorInvalidValue;
+        });
+        if (e != cudaSuccess) values[q] = -1;
+    }
+    return FDTD_OK;
 }
 
 fdtd_status fdtd_debug_tb2_refine(int slots, const long long* starts, const unsigned long long* cycles, double step,

@@ -101,6 +101,7 @@ _SIGS = {
     "fdtd_measure_balance": (C.c_int, [C.c_void_p, C.c_void_p]),
     "fdtd_debug_tb2_order": (C.c_int, [C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_void_p]),
     "fdtd_debug_tb2_refine": (C.c_int, [C.c_int, C.c_void_p, C.c_void_p, C.c_double, C.c_void_p]),
+    "fdtd_debug_per_device": (C.c_int, [C.c_void_p, C.c_void_p, C.c_int, C.c_void_p]),
     "fdtd_destroy_grid": (None, [C.c_void_p]),
     "fdtd_batch_required_bytes": (C.c_size_t, [C.c_int, C.c_int]),
     "fdtd_batch_create": (C.c_int, [C.POINTER(C.c_void_p), C.c_int, C.c_void_p, C.c_size_t, C.c_void_p,
@@ -306,6 +307,18 @@ def tb2_refine(starts, cycles, step: float = 1.0):
     out = np.zeros_like(st)
     check(lib().fdtd_debug_tb2_refine(int(cy.size), st.ctypes.data, cy.ctypes.data, float(step), out.ctypes.data),
           "fdtd_debug_tb2_refine")
+    return out
+
+
+def per_device(devices, results):
+    """Calls from `devices` to a set-up that is made once per device
+    (fdtd_debug_per_device): what each call works with."""
+    d, r = np.ascontiguousarray(devices, np.int32), np.ascontiguousarray(results, np.int32)
+    if d.size != r.size:
+        raise ValueError("results needs one entry per call")
+    out = np.zeros_like(d)
+    check(lib().fdtd_debug_per_device(d.ctypes.data, r.ctypes.data, int(d.size), out.ctypes.data),
+          "fdtd_debug_per_device")
     return out
 
 
