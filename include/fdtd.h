@@ -392,8 +392,9 @@ void fdtd_destroy_grid(fdtd_grid* g);
  * another parity) makes fdtd_batch_step return ESTATE.
  * fdtd_batch_set_engine switches engines between steps (EINVAL for an
  * unknown engine).  fdtd_batch_sync waits for the stream and reports CUDA
- * errors or an expired device wait (ETIMEOUT).  fdtd_batch_work_items: cell
- * blocks per step and pass. */
+ * errors or an expired device wait, the batch's own or one of its grids'
+ * (ETIMEOUT; reported once, here or by the grid's next synchronising call).
+ * fdtd_batch_work_items: cell blocks per step and pass. */
 enum { FDTD_BATCH_PERSISTENT = 0, FDTD_BATCH_CELL = 1, FDTD_BATCH_PERSISTENT_CELL = 2 };
 /* Grid modes of the graph engine. */
 enum { FDTD_BATCH_MODE_CELL4 = 0, FDTD_BATCH_MODE_CELL8 = 1, FDTD_BATCH_MODE_CELL16 = 2,

@@ -251,6 +251,22 @@ yee_batch_cell(const __grid_constant__ PCellParams<real> P)
     }
 }
 
+// The grids' own error words, which the two-step kernel's expired waits raise:
+// a word that is raised is moved into the batch's header.
+constexpr int kErrWords = 64;
+struct ErrWords {
+    int* word[kErrWords];
+    int n;
+};
+__global__ void collect_errors(const ErrWords w, BatchHeader* hdr)
+{
+    if (int(threadIdx.x) >= w.n) return;
+    const int e = *w.word[threadIdx.x];
+    if (e == 0) return;
+    atomicOr(&hdr->err, e);
+    *w.word[threadIdx.x] = 0;
+}
+
 }  // namespace fdtd
 
 using namespace fdtd;
@@ -744,7 +760,8 @@ static fdtd_status batch_step_ranges(fdtd_batch* b, int nsteps)
         const fdtd_status pst = b->precision == FDTD_F64 ? pcell_fill<double>(b) : pcell_fill<float>(b);
         if (pst != FDTD_OK) return pst;
     }
-    for (fdtd_grid* g : b->grids) g->err_dirty = true;   // replays of two-step launches
+    for (fdtd_grid* g : b->grids)
+        if (b->precision == FDTD_F32) g->err_dirty = true;   // replays of two-step launches
     int done = 0;
     while (done < nsteps) {
         const int count = nsteps - done < kBatchGraphSteps ? nsteps - done : kBatchGraphSteps;
@@ -790,7 +807,19 @@ fdtd_status fdtd_batch_sync(fdtd_batch* b)
     if (!b) return fail(FDTD_EINVAL, "null batch");
     const fdtd_status dev_st = check_device(b->grids[0], "fdtd_batch_sync");
     if (dev_st != FDTD_OK) return dev_st;
-    fdtd_status st = cuda_check(cudaStreamSynchronize(b->stream), "batch synchronize");
+    ErrWords w;
+    w.n = 0;
+    fdtd_status st = FDTD_OK;
+    for (size_t q = 0; q < b->grids.size() && st == FDTD_OK; ++q) {
+        const fdtd_grid* g = b->grids[q];
+        if (g->err_dirty) w.word[w.n++] = reinterpret_cast<int*>(static_cast<char*>(g->arena) + g->L.err);
+        if (w.n == kErrWords || (w.n > 0 && q + 1 == b->grids.size())) {
+            collect_errors<<<1, kErrWords, 0, b->stream>>>(w, static_cast<BatchHeader*>(b->table));
+            st = cuda_check(cudaGetLastError(), "collect errors");
+            w.n = 0;
+        }
+    }
+    if (st == FDTD_OK) st = cuda_check(cudaStreamSynchronize(b->stream), "batch synchronize");
     if (st != FDTD_OK) return st;
     BatchHeader h;
     st = cuda_check(cudaMemcpy(&h, b->table, sizeof(h), cudaMemcpyDeviceToHost), "read batch header");
