@@ -761,7 +761,7 @@ static fdtd_status batch_step_ranges(fdtd_batch* b, int nsteps)
         if (pst != FDTD_OK) return pst;
     }
     for (fdtd_grid* g : b->grids)
-        if (b->precision == FDTD_F32) g->err_dirty = true;   // replays of two-step launches
+        if (b->precision == FDTD_F32) mark_waits(g, b->stream);   // two-step launches
     int done = 0;
     while (done < nsteps) {
         const int count = nsteps - done < kBatchGraphSteps ? nsteps - done : kBatchGraphSteps;
@@ -812,7 +812,7 @@ fdtd_status fdtd_batch_sync(fdtd_batch* b)
     fdtd_status st = FDTD_OK;
     for (size_t q = 0; q < b->grids.size() && st == FDTD_OK; ++q) {
         const fdtd_grid* g = b->grids[q];
-        if (g->err_dirty) w.word[w.n++] = reinterpret_cast<int*>(static_cast<char*>(g->arena) + g->L.err);
+        if (g->err_dirty || g->err_always) w.word[w.n++] = reinterpret_cast<int*>(static_cast<char*>(g->arena) + g->L.err);
         if (w.n == kErrWords || (w.n > 0 && q + 1 == b->grids.size())) {
             collect_errors<<<1, kErrWords, 0, b->stream>>>(w, static_cast<BatchHeader*>(b->table));
             st = cuda_check(cudaGetLastError(), "collect errors");

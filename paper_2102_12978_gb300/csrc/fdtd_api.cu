@@ -52,6 +52,22 @@ fdtd_status check_device(const fdtd_grid* g, const char* what)
     return FDTD_OK;
 }
 
+bool stream_captured(cudaStream_t s)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
+void mark_waits(fdtd_grid* g, cudaStream_t s)
+{
+    g->err_dirty = true;
+    if (s != g->stream || stream_captured(s)) g->err_always = true;
+}
+
 // True if p is device memory of the grid's device, aligned to `align` bytes: a
 // kernel of the grid may write it.
 static bool plain_device_array(const fdtd_grid* g, const void* p, size_t align)
@@ -360,7 +376,7 @@ static cudaError_t launch_tma(const fdtd_grid* cg, int cur, long long n, int lz,
     dim3 block(32, TR / R);
     dim3 grid((g->desc.nx + 31) / 32, (g->desc.ny + TR - 1) / TR, (g->desc.nz + lz - 1) / lz);
     int* err = reinterpret_cast<int*>(static_cast<char*>(g->arena) + g->L.err);
-    g->err_dirty = true;
+    mark_waits(g, s);
     yee_step_tma<real, TR, R, S><<<grid, block, smem, s>>>(make_args<real>(g, cur), *m, n, lz, err);
     return cudaGetLastError();
 }
@@ -477,7 +493,7 @@ fdtd_status fdtd_create_grid(const fdtd_grid_desc* d, void* arena, size_t arena_
     g->step = 0;
     g->cur = 0;
     g->pe = 0;
-    g->err_dirty = false;
+    g->err_dirty = g->err_always = false;
     g->flip = 0;
     g->has_source = false;
     g->src_gen = 0;
@@ -931,18 +947,17 @@ fdtd_status fdtd_sync(fdtd_grid* g)
     const fdtd_status dev_st = check_device(g, "fdtd_sync");
     if (dev_st != FDTD_OK) return dev_st;
     // the error word is read in stream order, so that one wait serves both, and
-    // only if a kernel with bounded waits was queued since it last read zero
+    // only if a kernel with bounded waits may have run since it last read zero
     // (a read costs 6 us; a look at seven arrays waits seven times)
     int err = 0;
     fdtd_status st = FDTD_OK;
-    if (g->err_dirty)
+    if (g->err_dirty || g->err_always)
         st = cuda_check(cudaMemcpyAsync(&err, static_cast<char*>(g->arena) + g->L.err, sizeof(int),
                                         cudaMemcpyDeviceToHost, g->stream), "read error word");
     if (st == FDTD_OK) st = cuda_check(cudaStreamSynchronize(g->stream), "stream synchronize");
     if (st == FDTD_OK) st = cuda_check(cudaGetLastError(), "pending CUDA error");
     if (st != FDTD_OK) return st;
-    // a batch may run the grid on another stream: keep reading while one holds it
-    if (err == 0 && g->batch_refs == 0) g->err_dirty = false;
+    if (err == 0) g->err_dirty = false;
     if (err != 0) {
         cudaMemsetAsync(static_cast<char*>(g->arena) + g->L.err, 0, sizeof(int), g->stream);
         cudaStreamSynchronize(g->stream);

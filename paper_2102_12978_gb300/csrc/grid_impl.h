@@ -129,6 +129,8 @@ struct fdtd_grid {
     fdtd::SrcTime srct;
     int64_t counts[6];
     bool err_dirty;          // kernels that may raise the error word were queued since it was last read as zero
+    bool err_always;         // such kernels may also run where the grid's own waits do not see them, on
+                             // another stream or in replays of a caller's graph: the word is always read
     int sm_count;
     int device;                 // CUDA device current at fdtd_create_grid
     fdtd::TileConfig tile;
@@ -164,6 +166,10 @@ struct fdtd_grid {
 };
 
 namespace fdtd {
+// True while a caller captures stream s into a graph.
+bool stream_captured(cudaStream_t s);
+// Notes that kernels that may raise the grid's error word are queued on s.
+void mark_waits(fdtd_grid* g, cudaStream_t s);
 template <typename real>
 StepArgs<real> make_args(const fdtd_grid* g, int cur);
 // One step on stream s.  `mid`, if not null, is recorded between the two

@@ -90,7 +90,7 @@ static cudaError_t launch_hflu(const fdtd_grid* cg, int cur, long long n, int lz
     dim3 grid((g->desc.nx + 31) / 32, (g->desc.ny + TY - 1) / TY, (g->desc.nz + lz - 1) / lz);
     int* err = reinterpret_cast<int*>(static_cast<char*>(g->arena) + g->L.err);
     const StepArgs<real> a = make_args<real>(g, cur);
-    g->err_dirty = true;
+    mark_waits(g, s);
     yee_hflu_tma<real, TY, S><<<grid, block, smem, s>>>(a, *m, n, lz, err);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;

@@ -332,7 +332,7 @@ static cudaError_t launch_tb2_t(const fdtd_grid* cg, int cur, long long n, const
     tt.th1 = t1.th; tt.te1 = t1.te; tt.tw1 = t1.tw;
     TmaMaps* m = nullptr;
     if (!tb2_maps<RY>(g, cur, &m)) return cudaErrorInvalidValue;
-    g->err_dirty = true;
+    mark_waits(g, s);
     const StepArgs<float> a = make_args<float>(g, cur);
     const unsigned ctas = unsigned(slots);
     if constexpr (RY == kTb2Rows) {
@@ -376,7 +376,6 @@ cudaError_t launch_tb2_table(const fdtd_grid* cg, int cur, const StepTime<float>
     tb2_plan(g, RY, slots, tc, plan);
     TmaMaps* m = nullptr;
     if (!tb2_maps<RY>(g, cur, &m)) return cudaErrorInvalidValue;
-    g->err_dirty = true;
     const StepArgs<float> a = make_args<float>(g, cur);
     const unsigned ctas = unsigned(slots);
     if (!automatic) yee_tb2_t<RY, false, false, true><<<ctas, S::NT, S::bytes(), s>>>(a, times, i0, i1, *m, plan);

@@ -37,3 +37,44 @@ def test_batch_sync_reports_a_grids_expired_wait(grids, bad):
     b.sync()              # reported once
     gs[bad].sync()
     b.close()
+
+
+def test_word_raised_by_a_batch_on_another_stream():
+    """A batch runs its grids on the first one's stream.  A grid with a stream
+    of its own cannot wait for them, so a look at its word that comes before
+    the batch's kernels raise it is not the last one."""
+    w = W.small(nx=32, ny=30, nz=4, npml=4, r_center=7.0, ramp=1.0)
+    d = fdtd.make_grid_desc(w.nx, w.ny, w.nz, w.npml, w.dx, w.dx, w.dz, courant=w.courant, precision="f32")
+    other = torch.cuda.Stream()
+    a, g = gpu_grid(w, "f32"), fdtd.Grid(d, stream=other)
+    b = fdtd.Batch([a, g])
+    b.step(4)
+    b.close()
+    g.sync()              # reads zero: nothing has expired yet
+    _raise_word(g)
+    _times_out(g.sync)
+    g.sync()
+
+
+@pytest.mark.parametrize("tile", [None, (7, 16, 1), (1, 8, 4)])
+def test_word_raised_by_a_replayed_graph(tile):
+    """Steps captured into the caller's graph run when it is replayed, which
+    the grid does not see."""
+    w = W.small(nx=32, ny=30, nz=4, npml=4, r_center=7.0, ramp=1.0)
+    d = fdtd.make_grid_desc(w.nx, w.ny, w.nz, w.npml, w.dx, w.dx, w.dz, courant=w.courant, precision="f32")
+    stream = torch.cuda.Stream()
+    g = fdtd.Grid(d, stream=stream)
+    if tile:
+        g.set_tile(*tile)
+    g.step(4)
+    g.sync()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        g.step(4)
+    g.sync()
+    graph.replay()
+    _raise_word(g)
+    _times_out(g.sync)
+    g.sync()
+    _raise_word(g)        # and after the next replay
+    _times_out(g.sync)
