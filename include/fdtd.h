@@ -204,7 +204,9 @@ fdtd_status fdtd_wall_coefficients(const fdtd_grid_desc* d, const fdtd_wall_desc
  * E^{n+1} (with CPML psi) -> E soft source at (n+1) dt (Eq. 13) -> wall
  * source at (n+1) dt.  One or two kernel launches per step (tile variant);
  * an FP32 grid on its default tile takes pairs of steps in one launch (see
- * fdtd_set_tile).
+ * fdtd_set_tile).  Captured into a graph on the default tile, an even nsteps
+ * can be replayed: every replay advances the state by nsteps (the source
+ * keeps the time of the captured steps).
  * Small grids, whose passes take a few microseconds, are bound by the cost
  * of those launches; a batch of one grid (fdtd_batch_create with n = 1)
  * replays 64 steps from one CUDA graph instead, with the same results
