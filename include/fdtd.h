@@ -349,6 +349,11 @@ fdtd_status fdtd_debug_inject_fault(fdtd_grid* g, int kind);
  * queued) a grid whose device is not the current one.  The grid is unusable
  * until its own device is recorded again.  EINVAL for device < 0. */
 fdtd_status fdtd_debug_set_device(fdtd_grid* g, int device);
+/* Test hook: 1 if a read-out of `bytes` bytes to dst is written by a kernel of
+ * the grid (dst on its device, aligned to `align` bytes, all the bytes inside
+ * dst's allocation), 0 if it goes through the runtime's copy, which refuses an
+ * array that is too small. */
+int fdtd_debug_direct_output(const fdtd_grid* g, const void* dst, size_t bytes, size_t align);
 fdtd_status fdtd_get_tile(const fdtd_grid* g, int* variant, int* ty, int* lz);
 fdtd_status fdtd_autotune(fdtd_grid* g, int steps, void* scratch_state);
 

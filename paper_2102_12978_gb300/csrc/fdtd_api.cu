@@ -68,16 +68,32 @@ void mark_waits(fdtd_grid* g, cudaStream_t s)
     if (s != g->stream || stream_captured(s)) g->err_always = true;
 }
 
-// True if p is device memory of the grid's device, aligned to `align` bytes: a
-// kernel of the grid may write it.
-static bool plain_device_array(const fdtd_grid* g, const void* p, size_t align)
+// True if the `bytes` bytes from p on lie in one allocation of the grid's
+// device, aligned to `align` bytes: a kernel of the grid may write them.  (The
+// runtime's copies check the range of a device array and refuse one that is
+// too small; a kernel would write past it.)
+static bool plain_device_array(const fdtd_grid* g, const void* p, size_t bytes, size_t align)
 {
-    cudaPointerAttributes at;
-    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return at.type == cudaMemoryTypeDevice && at.device == g->device && reinterpret_cast<uintptr_t>(p) % align == 0;
+    static const PFN_cuPointerGetAttributes_v7000 attributes = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        const bool ok = cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 7000, cudaEnableDefault, &q) ==
+                            cudaSuccess &&
+                        q == cudaDriverEntryPointSuccess;
+        return reinterpret_cast<PFN_cuPointerGetAttributes_v7000>(ok ? f : nullptr);
+    }();
+    if (!attributes || reinterpret_cast<uintptr_t>(p) % align != 0) return false;
+    unsigned type = 0, managed = 1;
+    int device = -1;
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                                  CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                  CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void* out[] = {&type, &managed, &device, &base, &size};
+    const CUdeviceptr at = reinterpret_cast<CUdeviceptr>(p);
+    return attributes(5, what, out, at) == CUDA_SUCCESS && type == CU_MEMORYTYPE_DEVICE && managed == 0 &&
+           device == g->device && at >= base && at - base <= size && bytes <= size - (at - base);
 }
 
 fdtd_status copy_field_out(const fdtd_grid* g, const void* src, void* dst, bool on_device)
@@ -85,7 +101,7 @@ fdtd_status copy_field_out(const fdtd_grid* g, const void* src, void* dst, bool 
     const fdtd_grid_desc& d = g->desc;
     const size_t b = g->L.elem;
     const long long rows = (long long)d.ny * d.nz;
-    if (on_device && plain_device_array(g, dst, b))
+    if (on_device && plain_device_array(g, dst, size_t(rows) * d.nx * b, b))
         return cuda_check(b == 8 ? launch_field_export<double>(src, dst, d.nx, rows, g->L.pitch, g->sm_count, g->stream)
                                  : launch_field_export<float>(src, dst, d.nx, rows, g->L.pitch, g->sm_count, g->stream),
                           "copy field");
@@ -877,6 +893,11 @@ fdtd_status fdtd_debug_inject_fault(fdtd_grid* g, int kind)
     return FDTD_OK;
 }
 
+int fdtd_debug_direct_output(const fdtd_grid* g, const void* dst, size_t bytes, size_t align)
+{
+    return g && align > 0 && plain_device_array(g, dst, bytes, align) ? 1 : 0;
+}
+
 fdtd_status fdtd_debug_set_device(fdtd_grid* g, int device)
 {
     if (!g || device < 0) return fail(FDTD_EINVAL, "invalid argument");
@@ -983,9 +1004,9 @@ fdtd_status fdtd_fluence(fdtd_grid* g, void* dst, int on_device, int reset)
     // straight to the caller's array if it is plain memory of the grid's device,
     // else through the staging array (256 x 256 x 128 cells: 115 us for the whole
     // read-out through it, 50 us straight)
-    const bool direct = on_device && plain_device_array(g, dst, 8);
-    double* out = direct ? static_cast<double*>(dst) : reinterpret_cast<double*>(A + g->L.flu_out);
     const long long rows = (long long)d.ny * d.nz;
+    const bool direct = on_device && plain_device_array(g, dst, size_t(rows) * d.nx * 8, 8);
+    double* out = direct ? static_cast<double*>(dst) : reinterpret_cast<double*>(A + g->L.flu_out);
     const void* F = A + g->L.fluence;
     fdtd_status st = cuda_check(
         d.precision == FDTD_F64

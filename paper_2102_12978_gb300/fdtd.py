@@ -84,6 +84,7 @@ _SIGS = {
     "fdtd_set_tile": (C.c_int, [C.c_void_p, C.c_int, C.c_int, C.c_int]),
     "fdtd_step_timed": (C.c_int, [C.c_void_p, C.c_int, C.POINTER(C.c_float), C.c_int, C.POINTER(C.c_int)]),
     "fdtd_debug_inject_fault": (C.c_int, [C.c_void_p, C.c_int]),
+    "fdtd_debug_direct_output": (C.c_int, [C.c_void_p, C.c_void_p, C.c_size_t, C.c_size_t]),
     "fdtd_debug_set_device": (C.c_int, [C.c_void_p, C.c_int]),
     "fdtd_set_balance": (C.c_int, [C.c_void_p, C.c_float, C.c_float]),
     "fdtd_batch_set_grid_mode": (C.c_int, [C.c_void_p, C.c_int, C.c_int]),
@@ -393,6 +394,10 @@ class Grid:
     def debug_set_device(self, device: int):
         """Test hook: record `device` as the grid's device (fdtd_debug_set_device)."""
         check(lib().fdtd_debug_set_device(C.c_void_p(self.handle), int(device)), "fdtd_debug_set_device")
+
+    def debug_direct_output(self, ptr: int, nbytes: int, align: int) -> bool:
+        """Test hook: a kernel writes a read-out of nbytes to ptr (fdtd_debug_direct_output)."""
+        return bool(lib().fdtd_debug_direct_output(C.c_void_p(self.handle), C.c_void_p(ptr), nbytes, align))
 
     def set_tile(self, variant: int, ty: int, lz: int):
         check(lib().fdtd_set_tile(C.c_void_p(self.handle), int(variant), int(ty), int(lz)), "fdtd_set_tile")
