@@ -263,9 +263,10 @@ int64_t fdtd_antenna_points(const fdtd_grid* g, int component);
  * grid or one with a wall source takes variant 5 only (EINVAL otherwise;
  * fdtd_autotune then times the ty of variant 5 only).
  * fdtd_create_grid picks a default (variant 5, ty 4).  As long as no tile is
- * chosen, an FP32 grid (z-walled ones from 40 planes per cell of a z face's
- * CPML on, from 6 for boxes of some 330 x 330 cells or more) takes its pairs
- * of steps with the two-step kernel instead, which then rounds every
+ * chosen, an FP32 grid takes its pairs of steps with the two-step kernel
+ * instead where that is estimated to be faster (the time depends on the box:
+ * it is slower on boxes of a few planes, on tall ones of one or two windows,
+ * and on small or fluence-less ones with z walls).  It then rounds every
  * operation as variant 5 does: the results are variant 5's, bit for bit.  Its
  * CTAs then take whole windows first and split the rest by estimated cost
  * (fdtd_set_balance).  fdtd_autotune times the candidates on this grid
@@ -318,6 +319,16 @@ fdtd_status fdtd_measure_balance(fdtd_grid* g, void* scratch_state);
 int fdtd_debug_tb2_order(int t, int u, int nz, int slots, int order, int* out);
 fdtd_status fdtd_debug_tb2_refine(int slots, const long long* starts, const unsigned long long* cycles, double step,
                                   long long* out);
+/* Test hooks of the default tile's route (no device work; the paper has no
+ * counterpart).  fdtd_debug_route_us: the estimated us per step of a grid's
+ * pairs of steps on the two-step kernel with `ctas` CTAs (sheet: with a wall
+ * source) and of its steps on the cell passes.  fdtd_debug_set_route: 0 takes
+ * the faster by estimate, 1 the two-step kernel (FP32 only), 2 the cell
+ * passes; refused while the grid belongs to a batch (ESTATE).
+ * fdtd_debug_get_route: 1 or 2, what a pair of steps takes (-1 for null). */
+fdtd_status fdtd_debug_route_us(const fdtd_grid_desc* d, int sheet, int ctas, double* two_step, double* cells);
+fdtd_status fdtd_debug_set_route(fdtd_grid* g, int route);
+int fdtd_debug_get_route(const fdtd_grid* g);
 /* Test hook (no device work; the paper has no counterpart): the bookkeeping of
  * what the two-step kernel sets up once per device of the process.  Call q
  * comes from device devices[q]; a set-up, if one runs, gives results[q] (0:

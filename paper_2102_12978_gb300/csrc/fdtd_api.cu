@@ -529,6 +529,7 @@ fdtd_status fdtd_create_grid(const fdtd_grid_desc* d, void* arena, size_t arena_
     std::memset(&g->wall, 0, sizeof(g->wall));
     std::memset(&g->wallt, 0, sizeof(g->wallt));
     g->fault = 0;
+    g->route = 0;
     for (int c = 0; c < 6; ++c) g->counts[c] = 0;
     int dev = 0, sms = 152;
     st = cuda_check(cudaGetDevice(&dev), "current device");

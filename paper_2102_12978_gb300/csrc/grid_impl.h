@@ -61,6 +61,11 @@ struct TileConfig {
     bool automatic = false;
 };
 
+// Estimated us per step of a grid's pairs of steps on the two-step kernel with
+// `ctas` CTAs (sheet: with a wall source), and of its steps on the cell passes.
+double two_step_us(const fdtd_grid_desc& d, bool sheet, int ctas);
+double cell_step_us(const fdtd_grid_desc& d);
+
 // A positive number that is made once per device of the process.  A kernel's
 // attributes (the opt-in to more than 48 KB of dynamic shared memory, and the
 // residency that follows) belong to one device's copy of it: a second device
@@ -140,6 +145,7 @@ struct fdtd_grid {
     bool hmaps_ok[2][3];
     fdtd::TmaMaps tb2maps[2][2];   // [read copy][window height] of the two-step kernel
     bool tb2maps_ok[2][2];
+    int route;                  // fdtd_debug_set_route: 0 as estimated, 1 two-step kernel, 2 cell passes
     int fault;                  // fdtd_debug_inject_fault: applies to the next step only
     int batch_refs;             // batches holding this grid (their kernels hold copies of its arguments)
     bool has_wall;              // fdtd_set_wall_source

@@ -22,6 +22,19 @@ void tb2_windows(const fdtd_grid_desc& d, int ry, int* t, int* u)
     *u = (d.ny + ry - 5) / (ry - 4);
 }
 
+// True if the windows of column wx of T (of row wy of U) run the x (y) shell
+// and wall code.
+static bool shell_x(const fdtd_grid_desc& d, int wx, int T)
+{
+    const int L0 = kTb2Sx * wx - kTb2Ox;
+    return wx == 0 || wx == T - 1 || (d.npml > 0 && (L0 < d.npml || L0 + kTb2Wx > d.nx - d.npml));
+}
+static bool shell_y(const fdtd_grid_desc& d, int ry, int wy, int U)
+{
+    const int M0 = (ry - 4) * wy - kTb2Oy;
+    return wy == 0 || wy == U - 1 || (d.npml > 0 && (M0 < d.npml || M0 + ry > d.ny - d.npml));
+}
+
 std::vector<long long> tb2_refined_ranges(const std::vector<long long>& s, const unsigned long long* cycles,
                                           double step)
 {
@@ -116,18 +129,6 @@ static int tb2_window_host(int T, int U, int D, int pos)
 constexpr double kRestart = 5.3;
 constexpr double kCorner = 0.4;
 constexpr double kZPlane = 1.6;
-// A z-walled grid takes the two-step kernel from this many planes per CPML
-// cell of a z face on: a z-shell plane costs it about four inner ones, so
-// that short boxes run faster on the cell passes.  The line lies lower for
-// boxes of at least kManyWindows windows per SM, whose windows march together.
-// us per step, two-step / cell passes, 16-cell z CPML, at 4, 6, 12 and 24 planes
-// per cell: 411 x 411 234 / 263, 315 / 367, 526 / 685, 938 / 1320; 340 x 335 (255
-// windows) 171 / 183, 226 / 256, 392 / 472, 697 / 907; 300 x 300 (195 windows) 187 /
-// 156, 250 / 216, 444 / 403, 739 / 772; 205 x 211 104 / 83, 142 / 115, 229 / 210, 405 / 402;
-// 100 x 91 30 / 25, 43 / 33, 75 / 63, 130 / 117.  6-cell z CPML, 340 x 335: 82 / 73 at
-// 4, 99 / 101 at 6.
-constexpr int kShellPlanes = 40, kShellPlanesMany = 6;
-constexpr double kManyWindows = 1.5;
 // Whole windows first only as far as no CTA's whole windows cost more than this
 // times a CTA's mean share: few windows per CTA and the dear ones on the shell
 // would leave the others waiting (288 x 252 x 128, 156 windows on 152 SMs: 151 us
@@ -156,7 +157,7 @@ static void tb2_plan(fdtd_grid* g, int RY, int slots, const TileConfig& tc, Tb2P
             g->tb2_start = g->tb2_refined;
             g->tb2_whole = 0;
         } else {
-            const int nx = d.nx, ny = d.ny, nz = d.nz, npml = d.npml;
+            const int nx = d.nx, ny = d.ny, nz = d.nz;
             const int nw = P.T * P.U;
             std::vector<double> cost(size_t(nw), 1.0);
             for (int wy = 0; wy < P.U; ++wy)
@@ -164,9 +165,7 @@ static void tb2_plan(fdtd_grid* g, int RY, int slots, const TileConfig& tc, Tb2P
                     const int L0 = kTb2Sx * wx - kTb2Ox, M0 = (RY - 4) * wy - kTb2Oy;
                     const int i0 = std::max(L0, 0), i1 = std::min(L0 + kTb2Wx, nx);
                     const int j0 = std::max(M0, 0), j1 = std::min(M0 + RY, ny);
-                    // windows that run the x (y) shell and wall code
-                    const int sx = wx == 0 || wx == P.T - 1 || (npml > 0 && (L0 < npml || L0 + kTb2Wx > nx - npml));
-                    const int sy = wy == 0 || wy == P.U - 1 || (npml > 0 && (M0 < npml || M0 + RY > ny - npml));
+                    const int sx = shell_x(d, wx, P.T), sy = shell_y(d, RY, wy, P.U);
                     bool ant = false;
                     if (!g->hmask.empty())
                         for (int j = j0; j < j1 && !ant; ++j)
@@ -262,20 +261,71 @@ static cudaError_t tb2_blocks_per_sm(int device, int* out)
     });
 }
 
-// Every FP32 box but short z-walled ones: the two-step kernel is the faster
-// one, or as fast, at every size measured (us per step, two-step / cell passes:
-// 16 x 16 x 8 7.3 / 8.3; 48 x 40 x 16 8.3 / 8.3; 64 x 64 x 32 10.3 / 10.3;
-// 96 x 96 x 64 15 / 18; 160 x 160 x 64 27 / 40; 332 x 332 x 46 62 / 112;
-// 640 x 640 x 64 261 / 525; 560 x 560 x 5 36 / 36).
-bool default_two_step(const fdtd_grid* g)
+// ---- the route of the default tile
+// Estimated us per step of the two kernels that a pair of steps can take.  The
+// bits are the same, so the default tile takes the one estimated to be faster.
+// The constants were fitted to 703 boxes measured both ways on one GB300 (2 x 2 x 1
+// to 2048 x 2048 x 12 and 8 x 8 x 16384 cells, with and without fluence, CPML, z
+// walls, z CPML and sheet): the faster kernel is taken, or one within 3 % of it,
+// for 656 of them, and the others cost 11 % on average.  us per step, two-step /
+// cell passes: 2048 x 2048 x 1 224 / 79, x 3 295 / 273, x 12 603 / 1075; 560 x 560 x
+// 2 24.6 / 16.5, x 12 56 / 75; 32 x 32 x 1024 36 / 25, 20 x 20 x 4096 38 / 69; 332 x
+// 332 x 46 62 / 109; 16 x 16 x 64 7.2 / 8.2; z walls, 360 x 360 x 6 34 / 21, 411 x 411
+// x 192 with 16 z-CPML cells 508 / 684, 205 x 205 x 400 with 8 417 / 402.
+//
+// Two-step kernel on `ctas` CTAs: the planes of a CTA's share, and kRefill for
+// each window it starts and for the range in which it goes on inside one,
+// times the time of a plane.
+constexpr double kRefill = 5.6;                       // planes
+constexpr double kPlane = 1.24, kPlaneNoFlu = 1.0;    // us, an inner window's, with and without the fluence terms
+constexpr double kPlaneWall = 1.4;                    // the wall kernel, which has the fluence terms always
+constexpr double kShellWall = 0.3;                    // as w_shell, for the wall kernel
+constexpr double kOddShell = 0.32;                    // more for an x shell off even columns (4-byte psi accesses)
+constexpr double kZShell = 2.1;                       // a z-shell plane, in planes
+constexpr double kZCode = 1.27, kZCodeFew = 1.6;      // all of it with a z CPML: many and few windows per CTA
+constexpr double kManyWindows = 1.5;
+constexpr double kWallFloor = 8.5;
+double two_step_us(const fdtd_grid_desc& d, bool sheet, int ctas)
 {
-    const fdtd_grid_desc& d = g->desc;
-    if (d.precision != FDTD_F32) return false;
-    if (d.z_boundary != FDTD_Z_WALLS) return true;
     int T, U;
     tb2_windows(d, kTb2Rows, &T, &U);
-    const bool many = double(T) * U >= kManyWindows * (g->sm_count > 0 ? g->sm_count : 152);
-    return d.nz >= (many ? kShellPlanesMany : kShellPlanes) * d.npml_z;
+    const bool zw = d.z_boundary == FDTD_Z_WALLS, wall = zw || sheet;
+    double fx = 0.0, fy = 0.0;   // shares of the windows with x and with y shell code
+    for (int wx = 0; wx < T; ++wx) fx += shell_x(d, wx, T) ? 1.0 / T : 0.0;
+    for (int wy = 0; wy < U; ++wy) fy += shell_y(d, kTb2Rows, wy, U) ? 1.0 / U : 0.0;
+    const double odd = d.npml > 0 && ((d.nx | d.npml) & 1) ? kOddShell : 0.0;
+    const double cost = 1.0 + (wall ? kShellWall : TileConfig().w_shell) * (fx * (1.0 + odd) + fy + kCorner * fx * fy);
+    const double windows = double(T) * U / ctas;   // per CTA
+    const int npz = zw ? d.npml_z : 0;
+    const double nz = d.nz, z = nz + 2.0 * npz * (kZShell - 1.0);
+    const double planes = std::max(windows * z, z / nz) + (kRefill + (zw ? 1.0 : 0.0)) * (windows + 1.0);
+    const double plane = wall ? kPlaneWall : (d.fluence ? kPlane : kPlaneNoFlu);
+    const double us = 0.5 * cost * planes * plane * (npz == 0 ? 1.0 : (windows < kManyWindows ? kZCodeFew : kZCode));
+    return wall ? std::max(us, kWallFloor) : us;
+}
+
+// Cell passes: two launches, and from some 10^5 cells on the cells (in whole
+// 32 x 4 blocks) at the rate of the passes, the shells' with half a cell's
+// work more.
+constexpr double kCellRate = 52.0e3, kCellRateNoFlu = 70.0e3;   // cells per us
+constexpr double kCellShell = 0.55;
+double cell_step_us(const fdtd_grid_desc& d)
+{
+    const double cells = double((d.nx + 31) / 32 * 32) * ((d.ny + 3) / 4 * 4) * d.nz;
+    const double inner = std::max(0.0, 1.0 - 2.0 * d.npml / d.nx) * std::max(0.0, 1.0 - 2.0 * d.npml / d.ny);
+    const int npz = d.z_boundary == FDTD_Z_WALLS ? d.npml_z : 0;
+    const double shell = 1.0 - (d.npml > 0 ? inner : 1.0) * (1.0 - 2.0 * npz / d.nz);
+    const double work = 2.9 + cells * (1.0 + kCellShell * shell) / (d.fluence ? kCellRate : kCellRateNoFlu);
+    const double launches = d.fluence ? std::max(8.9, 8.2 + std::min(cells / 65e3, 4.1))
+                                      : 8.2 + std::min(std::max(0.0, cells - 190e3) / 20e3, 4.1);
+    return std::max(launches, work);
+}
+
+bool default_two_step(const fdtd_grid* g)
+{
+    if (g->desc.precision != FDTD_F32) return false;
+    if (g->route != 0) return g->route == 1;
+    return two_step_us(g->desc, g->has_wall, g->sm_count > 0 ? g->sm_count : 152) < cell_step_us(g->desc);
 }
 
 int tb2_slots(const fdtd_grid* g, int ty)
@@ -397,6 +447,27 @@ int fdtd_debug_tb2_order(int t, int u, int nz, int slots, int order, int* out)
     for (int m = 0; m < t * u; ++m) out[m] = tb2_window_host(t, u, D, m);
     return D;
 }
+
+fdtd_status fdtd_debug_route_us(const fdtd_grid_desc* d, int sheet, int ctas, double* two_step, double* cells)
+{
+    const fdtd_status st = validate(d);
+    if (st != FDTD_OK) return st;
+    if (ctas < 1 || !two_step || !cells) return fail(FDTD_EINVAL, "invalid argument");
+    *two_step = two_step_us(*d, sheet != 0, ctas);
+    *cells = cell_step_us(*d);
+    return FDTD_OK;
+}
+
+fdtd_status fdtd_debug_set_route(fdtd_grid* g, int route)
+{
+    if (!g || route < 0 || route > 2 || (route == 1 && g->desc.precision != FDTD_F32))
+        return fail(FDTD_EINVAL, "invalid argument");
+    if (g->batch_refs > 0) return fail(FDTD_ESTATE, "fdtd_debug_set_route: the grid belongs to a batch");
+    g->route = route;
+    return FDTD_OK;
+}
+
+int fdtd_debug_get_route(const fdtd_grid* g) { return !g ? -1 : (default_two_step(g) ? 1 : 2); }
 
 fdtd_status fdtd_debug_per_device(const int* devices, const int* results, int n, int* values)
 {

@@ -102,6 +102,10 @@ _SIGS = {
     "fdtd_measure_balance": (C.c_int, [C.c_void_p, C.c_void_p]),
     "fdtd_debug_tb2_order": (C.c_int, [C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_void_p]),
     "fdtd_debug_tb2_refine": (C.c_int, [C.c_int, C.c_void_p, C.c_void_p, C.c_double, C.c_void_p]),
+    "fdtd_debug_route_us": (C.c_int, [C.POINTER(fdtd_grid_desc), C.c_int, C.c_int, C.POINTER(C.c_double),
+                                      C.POINTER(C.c_double)]),
+    "fdtd_debug_set_route": (C.c_int, [C.c_void_p, C.c_int]),
+    "fdtd_debug_get_route": (C.c_int, [C.c_void_p]),
     "fdtd_debug_per_device": (C.c_int, [C.c_void_p, C.c_void_p, C.c_int, C.c_void_p]),
     "fdtd_destroy_grid": (None, [C.c_void_p]),
     "fdtd_batch_required_bytes": (C.c_size_t, [C.c_int, C.c_int]),
@@ -311,6 +315,15 @@ def tb2_refine(starts, cycles, step: float = 1.0):
     return out
 
 
+def route_us(d: fdtd_grid_desc, sheet: bool = False, ctas: int = 152):
+    """Estimated us per step on the two-step kernel and on the cell passes
+    (fdtd_debug_route_us)."""
+    two, cells = C.c_double(), C.c_double()
+    check(lib().fdtd_debug_route_us(C.byref(d), int(sheet), int(ctas), C.byref(two), C.byref(cells)),
+          "fdtd_debug_route_us")
+    return two.value, cells.value
+
+
 def per_device(devices, results):
     """Calls from `devices` to a set-up that is made once per device
     (fdtd_debug_per_device): what each call works with."""
@@ -394,6 +407,14 @@ class Grid:
     def debug_set_device(self, device: int):
         """Test hook: record `device` as the grid's device (fdtd_debug_set_device)."""
         check(lib().fdtd_debug_set_device(C.c_void_p(self.handle), int(device)), "fdtd_debug_set_device")
+
+    def debug_set_route(self, route: int):
+        """Test hook: the kernels of the default tile (fdtd_debug_set_route)."""
+        check(lib().fdtd_debug_set_route(C.c_void_p(self.handle), int(route)), "fdtd_debug_set_route")
+
+    def debug_route(self) -> int:
+        """Test hook: 1 if a pair of steps on the default tile takes the two-step kernel, 2 for the cell passes."""
+        return int(lib().fdtd_debug_get_route(C.c_void_p(self.handle)))
 
     def debug_direct_output(self, ptr: int, nbytes: int, align: int) -> bool:
         """Test hook: a kernel writes a read-out of nbytes to ptr (fdtd_debug_direct_output)."""
