@@ -418,6 +418,10 @@ enum { FDTD_BATCH_PERSISTENT = 0, FDTD_BATCH_CELL = 1, FDTD_BATCH_PERSISTENT_CEL
 enum { FDTD_BATCH_MODE_CELL4 = 0, FDTD_BATCH_MODE_CELL8 = 1, FDTD_BATCH_MODE_CELL16 = 2,
        FDTD_BATCH_MODE_TWO_STEP = 3 };
 size_t fdtd_batch_required_bytes(int n_grids, int precision);
+/* Test hook (no device work): the CTAs and the route (1 two-step kernel, 2 cell
+ * passes) of n FP32 grids in a batch's graph while no mode is chosen; sheets[q]
+ * tells whether grid q has a wall source. */
+fdtd_status fdtd_debug_batch_routes(const fdtd_grid_desc* d, const int* sheets, int n, int sms, int* ctas, int* routes);
 fdtd_status fdtd_batch_create(fdtd_grid* const* grids, int n, void* dev_table, size_t table_bytes, void* stream,
                               fdtd_batch** out);
 fdtd_status fdtd_batch_set_engine(fdtd_batch* b, int engine);
@@ -425,9 +429,9 @@ int fdtd_batch_get_engine(const fdtd_batch* b);
 /* Mode of grid q (0-based, creation order) in the graph engine; EINVAL for
  * an unknown mode or the two-step mode on a grid that cannot take it.  The
  * default is FDTD_BATCH_MODE_CELL4; as long as no mode is chosen (and the batch
- * is not tuned), grids that would take the two-step kernel on their default
- * tile (fdtd_set_tile) take it in the graph too, with the same results (the
- * getter keeps naming the cell mode).  -1 from the getter for a bad index. */
+ * is not tuned), FP32 grids take the two-step kernel in the graph where it is
+ * estimated to be faster there, with the same results, bit for bit (the getter
+ * keeps naming the cell mode).  -1 from the getter for a bad index. */
 fdtd_status fdtd_batch_set_grid_mode(fdtd_batch* b, int q, int mode);
 int fdtd_batch_get_grid_mode(const fdtd_batch* b, int q);
 /* CTAs of grid q's two-step launches in the graph engine (-1 for a bad index). */

@@ -11,11 +11,11 @@
 //     cell-parallel H and E passes of tile variant 5 on 32 x 4, 8 or 16
 //     blocks, or (FP32 z-periodic grids without a wall sheet) the two-step
 //     kernel of tile variant 7 on a share of the SMs proportional to its
-//     cells.  Until a mode is chosen, the grids whose default tile takes the
-//     two-step kernel do so here too, with the same bits.  The per-step
-//     source time factors of every grid are evaluated on the host in FP64, as
-//     for a single grid, and copied into a device table ahead of each replay;
-//     the kernels read their steps' entries.
+//     cells.  Until a mode is chosen, FP32 grids take the two-step kernel where
+//     it is estimated to be the faster, with the bits of the cell passes.  The
+//     per-step source time factors of every grid are evaluated on the host in
+//     FP64, as for a single grid, and copied into a device table ahead of each
+//     replay; the kernels read their steps' entries.
 //   * persistent cell passes (FDTD_BATCH_PERSISTENT_CELL): one cooperative
 //     kernel launch runs up to K steps of every grid.  The 32 x 4 cell
 //     blocks of all grids form one list; the CTAs (one per resident slot)
@@ -289,8 +289,9 @@ struct fdtd_batch {
     int nbranch;
     std::vector<unsigned char> host_times;
     std::vector<int> mode;           // graph engine: each grid's mode (kModeCell4 ... kModeTwoStep)
-    bool automatic;                  // nobody chose modes: grids take the two-step kernel where the default
-                                     // tile would (default_two_step), the results being the same
+    bool automatic;                  // nobody chose modes: grids take the kernel estimated to be the faster
+                                     // (automatic_routes), the results being the same
+    std::vector<char> two;           // automatic: grids that take the two-step kernel in the graph
     std::vector<int> ctas;           // two-step mode: CTAs of the grid's launches
     bool shared_sms;                 // two-step launches on proportional shares of the SMs (else all)
     int cur;                         // copy parity of the grids (fdtd_grid::flip applied)
@@ -369,10 +370,10 @@ cudaError_t cell_launch_grid_any(fdtd_batch* b, int q, int parity, int step, cud
     return cell_launch_grid<float, 4>(b, q, parity, step, s);
 }
 
-// Grid q's pairs of steps run on the two-step kernel.
+// Grid q's pairs of steps in the graph run on the two-step kernel.
 bool takes_two_step(const fdtd_batch* b, int q)
 {
-    if (b->automatic) return b->precision == FDTD_F32 && default_two_step(b->grids[size_t(q)]);
+    if (b->automatic) return b->two[size_t(q)] != 0;
     return b->mode[size_t(q)] == kModeTwoStep;
 }
 
@@ -396,12 +397,13 @@ cudaError_t two_step_launches(fdtd_batch* b, int q, int parity, int launches, in
 }
 
 // `count` steps of every grid on one stream (steps that do not fill a graph
-// replay): where nobody chose modes, the two-step kernel in pairs of launches
-// on all SMs as far as they go, and the cell passes.
+// replay): where nobody chose modes and a grid alone would take it, the
+// two-step kernel in pairs of launches on all SMs as far as they go, and the
+// cell passes.
 cudaError_t remainder_steps(fdtd_batch* b, int parity, int count, cudaStream_t s)
 {
     for (int q = 0; q < int(b->grids.size()); ++q) {
-        const int paired = b->automatic && takes_two_step(b, q) ? count / 4 * 4 : 0;
+        const int paired = b->automatic && default_two_step(b->grids[size_t(q)]) ? count / 4 * 4 : 0;
         cudaError_t e = two_step_launches(b, q, parity, paired / 2, kTb2MaxCtas, s);
         for (int st = paired; st < count && e == cudaSuccess; ++st)
             e = cell_launch_grid_any(b, q, parity ^ (st & 1), st, s);
@@ -567,28 +569,65 @@ void two_step_ctas(fdtd_batch* b, bool shared)
     }
 }
 
-// The same while no mode has been chosen: a grid of at least as many windows
-// as SMs takes every SM (its windows then march together, see tb2_plan), the
-// smaller ones take shares among themselves.  us per step, shares of all
-// cells / every grid on all SMs / this rule: 2 x (640^2, 320^2, 160^2, 96^2) x 64
-// 886 / 720 / 709, 3 x 320^2 x 64 251 / 220 / 220, 12 x 96^2 x 16 37 / 76 / 37,
-// 3 x (96^2, 160^2) x 64 102 / 109 / 102.
+// CTAs and route of the FP32 grids for which no mode has been chosen.
+//
+// CTAs: a grid of at least as many windows as SMs takes every SM (its windows
+// then march together, see tb2_plan), the smaller ones take shares among
+// themselves.  us per step, shares of all cells / every grid on all SMs / this
+// rule: 2 x (640^2, 320^2, 160^2, 96^2) x 64 886 / 720 / 709, 3 x 320^2 x 64 251 / 220 /
+// 220, 12 x 96^2 x 16 37 / 76 / 37, 3 x (96^2, 160^2) x 64 102 / 109 / 102.
+//
+// Route: the two-step kernel where it is estimated to be the faster on that
+// share.  The two kernels' launches come out of a graph here, so that the cell
+// passes of a small grid cost 5.4 us per step and not 8 to 12, and of many grids
+// their launches count: two cell passes of a grid 0.54 us, half a two-step
+// launch 0.65.  us per step, two-step / cell passes: 16 x (48, 40, 16) 14.3 / 13.0, 1 x
+// (64, 64, 32) 8.4 / 5.4, 8 x (64, 64, 3) 9.1 / 7.0, 2 x (560, 560, 2) 42 / 18, 4 x (32, 32, 1024)
+// 114 / 97, 40 x (24, 24, 8) 26 / 22, 12 x (96, 96, 16) 34 / 42, 4 x (160, 160, 40) 53 / 81, 2 x
+// (332, 332, 46) 109 / 200, without fluence (the graph's kernel has its terms) 108 / 143.
+constexpr double kGraphStep = 5.4, kCellLaunches = 0.54, kTwoStepLaunch = 0.65;   // us
+void automatic_routes(const std::vector<const fdtd_grid_desc*>& d, const std::vector<char>& sheet, int sms,
+                      std::vector<int>& ctas, std::vector<char>& two)
+{
+    const size_t n = d.size();
+    ctas.assign(n, sms);
+    two.assign(n, 0);
+    std::vector<char> small(n, 0);
+    double cells_small = 0.0, taken = 0.0;
+    auto cells = [](const fdtd_grid_desc& g) { return double(g.nx) * g.ny * g.nz; };
+    for (size_t q = 0; q < n; ++q) {
+        int t, u;
+        tb2_windows(*d[q], kTb2Rows, &t, &u);
+        small[q] = (long long)t * u < sms;
+        if (small[q]) cells_small += cells(*d[q]);
+    }
+    for (size_t q = 0; q < n; ++q)
+        if (small[q]) {
+            ctas[q] = std::max(8, std::min(sms, int(cells(*d[q]) / cells_small * sms + 0.5)));
+            taken += ctas[q];
+        }
+    const double over = std::max(1.0, taken / sms);   // shares of 8 CTAs at least may be more than the SMs
+    for (size_t q = 0; q < n; ++q) {
+        const double turns = small[q] ? over : 1.0;
+        const double ts = two_step_us(*d[q], sheet[q] != 0, ctas[q], true) * turns;
+        const double cs = cell_work_us(*d[q]) * turns * sms / ctas[q];
+        two[q] = std::max(ts, kTwoStepLaunch * n) < std::max(std::max(cs, kGraphStep), kCellLaunches * n);
+    }
+}
+
 void automatic_ctas(fdtd_batch* b)
 {
-    two_step_ctas(b, true);
-    const int sms = b->grids[0]->sm_count > 0 ? b->grids[0]->sm_count : 152;
-    double small = 0.0;
-    auto windows = [](const fdtd_grid* g) {
-        int t, u;
-        tb2_windows(g->desc, kTb2Rows, &t, &u);
-        return t * u;
-    };
-    auto cells = [](const fdtd_grid* g) { return double(g->desc.nx) * g->desc.ny * g->desc.nz; };
-    for (const fdtd_grid* g : b->grids)
-        if (windows(g) < sms) small += cells(g);
+    b->shared_sms = true;
+    std::vector<const fdtd_grid_desc*> d;
+    std::vector<char> sheet;
+    for (const fdtd_grid* g : b->grids) {
+        d.push_back(&g->desc);
+        sheet.push_back(g->has_wall ? 1 : 0);
+    }
+    automatic_routes(d, sheet, b->grids[0]->sm_count > 0 ? b->grids[0]->sm_count : 152, b->ctas, b->two);
     for (size_t q = 0; q < b->grids.size(); ++q) {
-        const fdtd_grid* g = b->grids[q];
-        b->ctas[q] = windows(g) >= sms ? sms : std::max(8, std::min(sms, int(cells(g) / small * sms + 0.5)));
+        if (b->grids[q]->route != 0) b->two[q] = b->grids[q]->route == 1;
+        if (b->precision != FDTD_F32) b->two[q] = 0;
     }
 }
 
@@ -605,6 +644,25 @@ size_t fdtd_batch_required_bytes(int n_grids, int precision)
 {
     if (n_grids < 1 || (precision != FDTD_F32 && precision != FDTD_F64)) return 0;
     return times_offset() + size_t(kBatchGraphSteps) * n_grids * time_entry_bytes(precision);
+}
+
+fdtd_status fdtd_debug_batch_routes(const fdtd_grid_desc* d, const int* sheets, int n, int sms, int* ctas, int* routes)
+{
+    if (!d || !sheets || n < 1 || sms < 1 || !ctas || !routes) return fail(FDTD_EINVAL, "invalid argument");
+    std::vector<const fdtd_grid_desc*> v;
+    for (int q = 0; q < n; ++q) {
+        const fdtd_status st = validate(&d[q]);
+        if (st != FDTD_OK) return st;
+        v.push_back(&d[q]);
+    }
+    std::vector<int> c;
+    std::vector<char> two;
+    automatic_routes(v, std::vector<char>(sheets, sheets + n), sms, c, two);
+    for (int q = 0; q < n; ++q) {
+        ctas[q] = c[size_t(q)];
+        routes[q] = two[size_t(q)] ? 1 : 2;
+    }
+    return FDTD_OK;
 }
 
 fdtd_status fdtd_batch_create(fdtd_grid* const* grids, int n, void* dev_table, size_t table_bytes, void* stream,

@@ -62,9 +62,12 @@ struct TileConfig {
 };
 
 // Estimated us per step of a grid's pairs of steps on the two-step kernel with
-// `ctas` CTAs (sheet: with a wall source), and of its steps on the cell passes.
-double two_step_us(const fdtd_grid_desc& d, bool sheet, int ctas);
+// `ctas` CTAs (sheet: with a wall source; terms: with the fluence terms
+// compiled in), and of its steps on the cell passes: alone, launches
+// included, and the work of the passes.
+double two_step_us(const fdtd_grid_desc& d, bool sheet, int ctas, bool terms);
 double cell_step_us(const fdtd_grid_desc& d);
+double cell_work_us(const fdtd_grid_desc& d);
 
 // A positive number that is made once per device of the process.  A kernel's
 // attributes (the opt-in to more than 48 KB of dynamic shared memory, and the

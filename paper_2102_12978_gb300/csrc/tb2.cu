@@ -285,7 +285,7 @@ constexpr double kZShell = 2.1;                       // a z-shell plane, in pla
 constexpr double kZCode = 1.27, kZCodeFew = 1.6;      // all of it with a z CPML: many and few windows per CTA
 constexpr double kManyWindows = 1.5;
 constexpr double kWallFloor = 8.5;
-double two_step_us(const fdtd_grid_desc& d, bool sheet, int ctas)
+double two_step_us(const fdtd_grid_desc& d, bool sheet, int ctas, bool terms)
 {
     int T, U;
     tb2_windows(d, kTb2Rows, &T, &U);
@@ -299,7 +299,7 @@ double two_step_us(const fdtd_grid_desc& d, bool sheet, int ctas)
     const int npz = zw ? d.npml_z : 0;
     const double nz = d.nz, z = nz + 2.0 * npz * (kZShell - 1.0);
     const double planes = std::max(windows * z, z / nz) + (kRefill + (zw ? 1.0 : 0.0)) * (windows + 1.0);
-    const double plane = wall ? kPlaneWall : (d.fluence ? kPlane : kPlaneNoFlu);
+    const double plane = wall ? kPlaneWall : (terms ? kPlane : kPlaneNoFlu);
     const double us = 0.5 * cost * planes * plane * (npz == 0 ? 1.0 : (windows < kManyWindows ? kZCodeFew : kZCode));
     return wall ? std::max(us, kWallFloor) : us;
 }
@@ -309,23 +309,33 @@ double two_step_us(const fdtd_grid_desc& d, bool sheet, int ctas)
 // work more.
 constexpr double kCellRate = 52.0e3, kCellRateNoFlu = 70.0e3;   // cells per us
 constexpr double kCellShell = 0.55;
-double cell_step_us(const fdtd_grid_desc& d)
+static double cell_blocks(const fdtd_grid_desc& d)   // cells in whole blocks
 {
-    const double cells = double((d.nx + 31) / 32 * 32) * ((d.ny + 3) / 4 * 4) * d.nz;
+    return double((d.nx + 31) / 32 * 32) * ((d.ny + 3) / 4 * 4) * d.nz;
+}
+
+double cell_work_us(const fdtd_grid_desc& d)
+{
     const double inner = std::max(0.0, 1.0 - 2.0 * d.npml / d.nx) * std::max(0.0, 1.0 - 2.0 * d.npml / d.ny);
     const int npz = d.z_boundary == FDTD_Z_WALLS ? d.npml_z : 0;
     const double shell = 1.0 - (d.npml > 0 ? inner : 1.0) * (1.0 - 2.0 * npz / d.nz);
-    const double work = 2.9 + cells * (1.0 + kCellShell * shell) / (d.fluence ? kCellRate : kCellRateNoFlu);
+    return cell_blocks(d) * (1.0 + kCellShell * shell) / (d.fluence ? kCellRate : kCellRateNoFlu);
+}
+
+double cell_step_us(const fdtd_grid_desc& d)
+{
+    const double cells = cell_blocks(d);
     const double launches = d.fluence ? std::max(8.9, 8.2 + std::min(cells / 65e3, 4.1))
                                       : 8.2 + std::min(std::max(0.0, cells - 190e3) / 20e3, 4.1);
-    return std::max(launches, work);
+    return std::max(launches, 2.9 + cell_work_us(d));
 }
 
 bool default_two_step(const fdtd_grid* g)
 {
     if (g->desc.precision != FDTD_F32) return false;
     if (g->route != 0) return g->route == 1;
-    return two_step_us(g->desc, g->has_wall, g->sm_count > 0 ? g->sm_count : 152) < cell_step_us(g->desc);
+    return two_step_us(g->desc, g->has_wall, g->sm_count > 0 ? g->sm_count : 152, g->desc.fluence != 0) <
+           cell_step_us(g->desc);
 }
 
 int tb2_slots(const fdtd_grid* g, int ty)
@@ -453,7 +463,7 @@ fdtd_status fdtd_debug_route_us(const fdtd_grid_desc* d, int sheet, int ctas, do
     const fdtd_status st = validate(d);
     if (st != FDTD_OK) return st;
     if (ctas < 1 || !two_step || !cells) return fail(FDTD_EINVAL, "invalid argument");
-    *two_step = two_step_us(*d, sheet != 0, ctas);
+    *two_step = two_step_us(*d, sheet != 0, ctas, d->fluence != 0);
     *cells = cell_step_us(*d);
     return FDTD_OK;
 }

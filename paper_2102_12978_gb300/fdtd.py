@@ -104,6 +104,8 @@ _SIGS = {
     "fdtd_debug_tb2_refine": (C.c_int, [C.c_int, C.c_void_p, C.c_void_p, C.c_double, C.c_void_p]),
     "fdtd_debug_route_us": (C.c_int, [C.POINTER(fdtd_grid_desc), C.c_int, C.c_int, C.POINTER(C.c_double),
                                       C.POINTER(C.c_double)]),
+    "fdtd_debug_batch_routes": (C.c_int, [C.POINTER(fdtd_grid_desc), C.c_void_p, C.c_int, C.c_int, C.c_void_p,
+                                          C.c_void_p]),
     "fdtd_debug_set_route": (C.c_int, [C.c_void_p, C.c_int]),
     "fdtd_debug_get_route": (C.c_int, [C.c_void_p]),
     "fdtd_debug_per_device": (C.c_int, [C.c_void_p, C.c_void_p, C.c_int, C.c_void_p]),
@@ -322,6 +324,18 @@ def route_us(d: fdtd_grid_desc, sheet: bool = False, ctas: int = 152):
     check(lib().fdtd_debug_route_us(C.byref(d), int(sheet), int(ctas), C.byref(two), C.byref(cells)),
           "fdtd_debug_route_us")
     return two.value, cells.value
+
+
+def batch_routes(descs, sheets=None, sms: int = 152):
+    """CTAs and route (1 two-step kernel, 2 cell passes) of FP32 grids in a
+    batch's graph while no mode is chosen (fdtd_debug_batch_routes)."""
+    n = len(descs)
+    d = (fdtd_grid_desc * n)(*descs)
+    s = np.ascontiguousarray(sheets if sheets is not None else [0] * n, np.int32)
+    ctas, routes = np.zeros(n, np.int32), np.zeros(n, np.int32)
+    check(lib().fdtd_debug_batch_routes(d, s.ctypes.data, n, int(sms), ctas.ctypes.data, routes.ctypes.data),
+          "fdtd_debug_batch_routes")
+    return ctas, routes
 
 
 def per_device(devices, results):

@@ -52,3 +52,26 @@ def test_estimates_grow_with_the_box_and_shrink_with_the_ctas():
             assert fdtd.route_us(d, ctas=8)[0] > t
     with pytest.raises(fdtd.FDTDError):
         fdtd.route_us(d, ctas=0)
+
+
+# grids of a batch, fluence, which of them take the two-step kernel in the graph (None: either, the times are close)
+BATCHES = [
+    ([(64, 64, 32, 8)], True, [2]), ([(64, 64, 3, 6)] * 8, True, [2] * 8), ([(332, 332, 3, 6)] * 2, True, [2] * 2),
+    ([(32, 32, 1024, 6)] * 4, True, [2] * 4), ([(48, 40, 16, 6)] * 16, True, [2] * 16),
+    ([(24, 24, 8, 4)] * 40, True, [2] * 40), ([(96, 96, 16, 16)] * 12, True, [1] * 12),
+    ([(160, 160, 40, 8)] * 4, False, [1] * 4), ([(332, 332, 46, 6)] * 2, False, [1] * 2),
+    ([(n, n, 64, 16) for n in (640, 320, 160, 96) for _ in range(2)], True, [1] * 8),
+    ([(560, 560, 2, 6), (320, 320, 64, 16)], True, [2, 1]),
+]
+
+
+@pytest.mark.parametrize("boxes,fluence,routes", BATCHES)
+def test_grids_of_a_batch(boxes, fluence, routes):
+    """Both ways of each batch were measured (us per step; csrc/batch.cu)."""
+    descs = [fdtd.make_grid_desc(*b, 0.05, 0.05, 0.05, fluence=fluence) for b in boxes]
+    ctas, got = fdtd.batch_routes(descs)
+    assert got.tolist() == routes
+    assert all(8 <= c <= 152 for c in ctas)
+    for b, c in zip(boxes, ctas):
+        windows = -(-b[0] // 24) * -(-b[1] // 20)
+        assert c == 152 or windows < 152      # grids of many windows have every SM
