@@ -253,15 +253,16 @@ int64_t fdtd_antenna_points(const fdtd_grid* g, int component);
  *      (needs nz <= 65535, else EINVAL);
  *   7  two steps per launch (temporal blocking; FP32 grids, ty 8 or 16,
  *      else EINVAL; lz 2 interleaves the window rows in the CTAs' work so
- *      that x-neighbouring windows march side by side, any other lz takes
- *      the windows row by row): windows of 32 x 24 columns (ty 16; 32 x 12
+ *      that x-neighbouring windows march side by side, lz 3 gives every CTA
+ *      whole windows first, any other lz takes the windows row by row):
+ *      windows of 32 x 24 columns (ty 16; 32 x 12
  *      with ty 8) march along z, recomputing their halo columns, so that
  *      fields, psi and the fluence cross HBM once per two steps.  An odd
  *      step count ends with one step of variant 5.  The CTAs' shares of the work are balanced on
  *      per-window costs (fdtd_set_balance).
  * The TMA variants (1, 2, 4) have no FP64 32x16 tile (EINVAL).  A z-walled
  * grid or one with a wall source takes variant 5 only (EINVAL otherwise;
- * fdtd_autotune then times the ty of variant 5 only).
+ * fdtd_autotune then times the ty of variant 5 and the default tile).
  * fdtd_create_grid picks a default (variant 5, ty 4).  As long as no tile is
  * chosen, an FP32 grid takes its pairs of steps with the two-step kernel
  * instead where that is estimated to be faster (the time depends on the box:
@@ -271,7 +272,9 @@ int64_t fdtd_antenna_points(const fdtd_grid* g, int component);
  * CTAs then take whole windows first and split the rest by estimated cost
  * (fdtd_set_balance).  fdtd_autotune times the candidates on this grid
  * (running `steps` steps for each, then restoring the state) and keeps the
- * fastest.  Results agree to rounding for every configuration. */
+ * fastest; the two-step kernel with the default tile's work split is one
+ * (variant 7, lz 3; with z walls or a wall source the default tile itself,
+ * which fdtd_get_tile names as variant 5, ty 4).  Results agree to rounding for every configuration. */
 fdtd_status fdtd_set_tile(fdtd_grid* g, int variant, int ty, int lz);
 
 /* Work-split weights of tile variant 7 (the paper has no counterpart): a
@@ -325,7 +328,8 @@ fdtd_status fdtd_debug_tb2_refine(int slots, const long long* starts, const unsi
  * source) and of its steps on the cell passes.  fdtd_debug_set_route: 0 takes
  * the faster by estimate, 1 the two-step kernel (FP32 only), 2 the cell
  * passes; refused while the grid belongs to a batch (ESTATE).
- * fdtd_debug_get_route: 1 or 2, what a pair of steps takes (-1 for null). */
+ * fdtd_debug_get_route: 1 or 2, what a pair of steps takes on the grid's tile,
+ * default or not (-1 for null). */
 fdtd_status fdtd_debug_route_us(const fdtd_grid_desc* d, int sheet, int ctas, double* two_step, double* cells);
 fdtd_status fdtd_debug_set_route(fdtd_grid* g, int route);
 int fdtd_debug_get_route(const fdtd_grid* g);

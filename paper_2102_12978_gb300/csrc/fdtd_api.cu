@@ -1196,18 +1196,22 @@ fdtd_status fdtd_autotune(fdtd_grid* g, int steps, void* scratch_state)
     g->fault = 0;
     fdtd_status st = fdtd_save_state(g, scratch_state);
     if (st != FDTD_OK) return st;
-    struct Cand { int variant, ty; float w_shell = 0.0f, w_ant = 0.0f; };
+    struct Cand { int variant, ty; float w_shell = 0.0f, w_ant = 0.0f; int lz = 1; };
     std::vector<Cand> cands = {{6, 4}, {6, 8}, {6, 16}, {5, 4}, {5, 8}, {5, 16}, {4, 4}, {4, 8}, {4, 16}, {3, 4},
                                {3, 8}, {3, 16}, {2, 8}, {2, 16}, {1, 4}, {1, 8}, {1, 16}, {0, 4}, {0, 8}, {0, 16}};
     if (g->desc.precision == FDTD_F64)
         cands = {{6, 4}, {6, 8}, {6, 16}, {5, 4}, {5, 8}, {5, 16}, {4, 4}, {4, 8}, {3, 4}, {3, 8}, {2, 8}, {2, 4},
                  {1, 4}, {1, 8}, {0, 4}, {0, 8}};
     if (g->desc.nz > 65535) cands.erase(cands.begin(), cands.begin() + 3);   // variant 6 takes nz <= 65535
-    if (g->desc.precision == FDTD_F32)   // variant 7 with its work-split weights (shell, antenna)
-        cands.insert(cands.begin(), {{7, 16, 0.0f, 0.0f}, {7, 16, 0.15f, 0.1f}, {7, 16, 0.3f, 0.2f},
+    const TileConfig none;
+    if (g->desc.precision == FDTD_F32)   // variant 7 with its work-split weights (shell, antenna); as on the default tile first
+        cands.insert(cands.begin(), {{7, 16, none.w_shell, none.w_ant, 3}, {7, 16, 0.0f, 0.0f}, {7, 16, 0.15f, 0.1f}, {7, 16, 0.3f, 0.2f},
                                      {7, 16, 0.45f, 0.3f}, {7, 16, 0.3f, 0.4f}, {7, 16, 0.6f, 0.4f},
                                      {7, 8, 0.3f, 0.2f}});
-    if (has_walls(g)) cands = {{5, 4}, {5, 8}, {5, 16}};
+    if (has_walls(g)) {
+        cands = {{5, 4}, {5, 8}, {5, 16}};
+        if (default_two_step(g)) cands.insert(cands.begin(), {-1, 4});   // the default tile, whose pairs of steps no explicit tile takes
+    }
     const int nz = g->desc.nz;
     std::vector<int> lzs;
     for (int segs : {1, 2, 3, 4, 6, 8, 12, 16}) {
@@ -1228,9 +1232,10 @@ fdtd_status fdtd_autotune(fdtd_grid* g, int steps, void* scratch_state)
     cudaError_t err = cudaSuccess;
     for (const Cand& cd : cands)
         for (int lz : lzs) {
-            if (cd.variant >= 5 && lz != lzs[0]) continue;   // one cell per thread: no z segments
+            if ((cd.variant >= 5 || cd.variant < 0) && lz != lzs[0]) continue;   // one cell per thread: no z segments
             TileConfig tc; tc.variant = cd.variant; tc.tx = 32; tc.ty = cd.ty; tc.lz = lz;
-            if (cd.variant == 7) { tc.w_shell = cd.w_shell; tc.w_ant = cd.w_ant; tc.lz = 1; }
+            if (cd.variant == 7) { tc.w_shell = cd.w_shell; tc.w_ant = cd.w_ant; tc.lz = cd.lz; }
+            if (cd.variant < 0) tc = default_tile(g->desc, g->sm_count);
             err = run_steps(g, 2, tc);   // warm-up
             if (err != cudaSuccess) break;
             cudaEventRecord(e0, g->stream);

@@ -108,8 +108,8 @@ static int tb2_window_host(int T, int U, int D, int pos)
 
 // CTA work ranges of variant 7 on grid g: windows of 32 x RY columns, `slots`
 // resident CTAs.  Each CTA gets a contiguous range of (window, plane) items,
-// on the default tile after as many whole windows as every CTA can have
-// (kWholeMost): CTA c takes the windows c, c + slots, ..., so that `slots` consecutive windows
+// on the default tile and with lz 3 after as many whole windows as every CTA can
+// have (kWholeMost): CTA c takes the windows c, c + slots, ..., so that `slots` consecutive windows
 // march up z together and find each other's halo planes in L2 (a range starts
 // at any plane, and its neighbours' halos come from HBM: 105 bytes read per
 // cell and launch, 32 needed).  us per step, ranges only / whole windows
@@ -144,7 +144,10 @@ static void tb2_plan(fdtd_grid* g, int RY, int slots, const TileConfig& tc, Tb2P
     P.prof = nullptr;
     P.dt16 = float(g->dt * 0.0625);
     P.err = reinterpret_cast<int*>(static_cast<char*>(g->arena) + g->L.err);
-    const int order = tc.automatic ? 0 : (tc.lz == 2 ? 2 : 1);
+    // whole windows first (0), rows interleaved (2) or row by row (1); measured
+    // ranges, and the launches that measure them, hold every window
+    const bool measure = tc.measured || g->tb2_profile;
+    const int order = tc.automatic || (tc.lz == 3 && !measure) ? 0 : (tc.lz == 2 ? 2 : 1);
     P.D = tb2_order_d(P.T, P.U, d.nz, slots, order);
     const bool meas = tc.measured && g->tb2_ref_ry == RY && g->tb2_ref_slots == slots &&
                       g->tb2_ref_src == g->src_gen && g->tb2_refined.size() == size_t(slots) + 1 &&
@@ -477,7 +480,11 @@ fdtd_status fdtd_debug_set_route(fdtd_grid* g, int route)
     return FDTD_OK;
 }
 
-int fdtd_debug_get_route(const fdtd_grid* g) { return !g ? -1 : (default_two_step(g) ? 1 : 2); }
+int fdtd_debug_get_route(const fdtd_grid* g)
+{
+    if (!g) return -1;
+    return g->tile.variant == 7 || (g->tile.automatic && default_two_step(g)) ? 1 : 2;
+}
 
 fdtd_status fdtd_debug_per_device(const int* devices, const int* results, int n, int* values)
 {
