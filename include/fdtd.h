@@ -432,10 +432,10 @@ fdtd_status fdtd_batch_set_engine(fdtd_batch* b, int engine);
 int fdtd_batch_get_engine(const fdtd_batch* b);
 /* Mode of grid q (0-based, creation order) in the graph engine; EINVAL for
  * an unknown mode or the two-step mode on a grid that cannot take it.  The
- * default is FDTD_BATCH_MODE_CELL4; as long as no mode is chosen (and the batch
- * is not tuned), FP32 grids take the two-step kernel in the graph where it is
- * estimated to be faster there, with the same results, bit for bit (the getter
- * keeps naming the cell mode).  -1 from the getter for a bad index. */
+ * default is FDTD_BATCH_MODE_CELL4; as long as no mode is chosen for it (and the
+ * batch is not tuned), an FP32 grid takes the two-step kernel in the graph
+ * where it is estimated to be faster there, with the same results, bit for bit
+ * (the getter keeps naming the cell mode).  -1 from the getter for a bad index. */
 fdtd_status fdtd_batch_set_grid_mode(fdtd_batch* b, int q, int mode);
 int fdtd_batch_get_grid_mode(const fdtd_batch* b, int q);
 /* CTAs of grid q's two-step launches in the graph engine (-1 for a bad index). */
@@ -446,7 +446,9 @@ int fdtd_batch_get_grid_ctas(const fdtd_batch* b, int q);
  * Times each grid alone on the cell passes of each block height (32 x 4, 8,
  * 16) over `steps` steps (rounded up to even) and keeps the fastest as its
  * cell mode.  Then times, over 64 steps of the whole batch (the better of two
- * replays): the graph engine with every grid of at least N cells on the
+ * replays): the graph engine as it runs while no mode is chosen (if that is
+ * kept, the getter names FDTD_BATCH_MODE_TWO_STEP for the grids on the two-step
+ * kernel that can be set to it); the graph engine with every grid of at least N cells on the
  * two-step kernel, for N over the sizes of the grids that can take it (and
  * with none), each with the two-step launches on shares of the SMs
  * proportional to the grids' cells or on every SM; and the persistent cell

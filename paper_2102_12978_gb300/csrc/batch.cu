@@ -27,10 +27,10 @@
 //     grid, grid barrier, E pass, barrier, and so on.  The cell arithmetic is
 //     that of tile variant 5, bit for bit; the barriers are bounded waits.
 // fdtd_batch_autotune picks each grid's cell-pass block height alone, then
-// times the whole batch with the grids above each size threshold on the
-// two-step kernel (on proportional shares of the SMs or on all of them) and
-// on the persistent cell engine, keeps the fastest, and restores every
-// grid's state.
+// times the whole batch as it runs untuned, with the grids above each size
+// threshold on the two-step kernel (on proportional shares of the SMs or on
+// all of them) and on the persistent cell engine, keeps the fastest, and
+// restores every grid's state.
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
@@ -57,8 +57,10 @@ constexpr int kBatchGraphSteps = 64;   // even, so a replay leaves the read copy
 // ---- graph engine
 constexpr int kCellTY = 4;          // 32 x 4 x 1 cell blocks (tile variant 5) of the persistent cell engine
 constexpr int kCellBranches = 16;   // concurrent graph branches (grids share them round-robin)
-// Per-grid modes of the graph engine.
-enum { kModeCell4 = 0, kModeCell8 = 1, kModeCell16 = 2, kModeTwoStep = 3 };
+// Per-grid modes of the graph engine; kModeAuto: nobody chose one, and the grid
+// takes the kernel estimated to be the faster (automatic_routes), the results
+// being the same.
+enum { kModeAuto = -1, kModeCell4 = 0, kModeCell8 = 1, kModeCell16 = 2, kModeTwoStep = 3 };
 
 // ---- persistent cell engine
 // Kernel parameter of one persistent cell launch: a group of at most
@@ -288,10 +290,9 @@ struct fdtd_batch {
     cudaStream_t branch[kCellBranches];
     int nbranch;
     std::vector<unsigned char> host_times;
-    std::vector<int> mode;           // graph engine: each grid's mode (kModeCell4 ... kModeTwoStep)
-    bool automatic;                  // nobody chose modes: grids take the kernel estimated to be the faster
-                                     // (automatic_routes), the results being the same
-    std::vector<char> two;           // automatic: grids that take the two-step kernel in the graph
+    std::vector<int> mode;           // graph engine: each grid's mode (kModeAuto ... kModeTwoStep)
+    std::vector<char> two;           // kModeAuto: grids that take the two-step kernel in the graph
+    bool tuned;                      // fdtd_batch_autotune chose the modes
     std::vector<int> ctas;           // two-step mode: CTAs of the grid's launches
     bool shared_sms;                 // two-step launches on proportional shares of the SMs (else all)
     int cur;                         // copy parity of the grids (fdtd_grid::flip applied)
@@ -373,7 +374,7 @@ cudaError_t cell_launch_grid_any(fdtd_batch* b, int q, int parity, int step, cud
 // Grid q's pairs of steps in the graph run on the two-step kernel.
 bool takes_two_step(const fdtd_batch* b, int q)
 {
-    if (b->automatic) return b->two[size_t(q)] != 0;
+    if (b->mode[size_t(q)] == kModeAuto) return b->two[size_t(q)] != 0;
     return b->mode[size_t(q)] == kModeTwoStep;
 }
 
@@ -390,20 +391,20 @@ cudaError_t two_step_launches(fdtd_batch* b, int q, int parity, int launches, in
     for (int l = 0; l < launches && e == cudaSuccess; ++l) {
         g->pe = pe0 ^ (l & 1);   // make_args picks the E-side psi copy of this launch
         e = launch_tb2_table(g, parity ^ g->flip ^ (l & 1), times, 2 * l * n + q, (2 * l + 1) * n + q, ctas,
-                             b->automatic, s);
+                             b->mode[size_t(q)] == kModeAuto, s);
     }
     g->pe = pe0;
     return e;
 }
 
 // `count` steps of every grid on one stream (steps that do not fill a graph
-// replay): where nobody chose modes and a grid alone would take it, the
+// replay): where nobody chose its mode and a grid alone would take it, the
 // two-step kernel in pairs of launches on all SMs as far as they go, and the
 // cell passes.
 cudaError_t remainder_steps(fdtd_batch* b, int parity, int count, cudaStream_t s)
 {
     for (int q = 0; q < int(b->grids.size()); ++q) {
-        const int paired = b->automatic && default_two_step(b->grids[size_t(q)]) ? count / 4 * 4 : 0;
+        const int paired = b->mode[size_t(q)] == kModeAuto && default_two_step(b->grids[size_t(q)]) ? count / 4 * 4 : 0;
         cudaError_t e = two_step_launches(b, q, parity, paired / 2, kTb2MaxCtas, s);
         for (int st = paired; st < count && e == cudaSuccess; ++st)
             e = cell_launch_grid_any(b, q, parity ^ (st & 1), st, s);
@@ -696,8 +697,8 @@ fdtd_status fdtd_batch_create(fdtd_grid* const* grids, int n, void* dev_table, s
     b->times_off = times_offset();
     b->bar_off = bar_offset();
     b->fault = 0;
-    b->mode.assign(size_t(n), kModeCell4);
-    b->automatic = true;
+    b->mode.assign(size_t(n), kModeAuto);
+    b->tuned = false;
     automatic_ctas(b);
     b->built[0] = b->built[1] = false;
     fdtd_status st = cuda_check(cudaStreamCreateWithFlags(&b->capture, cudaStreamNonBlocking), "capture stream");
@@ -753,10 +754,8 @@ fdtd_status fdtd_batch_set_grid_mode(fdtd_batch* b, int q, int mode)
         return fail(FDTD_EINVAL, "mode %d is not a batch grid mode", mode);
     if (mode == FDTD_BATCH_MODE_TWO_STEP && !two_step_eligible(b, q))
         return fail(FDTD_EINVAL, "the two-step mode takes FP32 z-periodic grids without a wall source");
-    if (b->mode[size_t(q)] != mode || b->automatic) {
+    if (b->mode[size_t(q)] != mode) {   // the others' modes and all shares of the SMs stay
         b->mode[size_t(q)] = mode;
-        if (b->automatic) two_step_ctas(b, true);
-        b->automatic = false;
         drop_graphs(b);
     }
     return FDTD_OK;
@@ -765,7 +764,9 @@ fdtd_status fdtd_batch_set_grid_mode(fdtd_batch* b, int q, int mode)
 int fdtd_batch_get_grid_mode(const fdtd_batch* b, int q)
 {
     if (!b || q < 0 || q >= int(b->grids.size())) return -1;
-    return b->mode[size_t(q)];
+    if (b->mode[size_t(q)] != kModeAuto) return b->mode[size_t(q)];
+    // a tuner that kept the automatic mode names the one that can be chosen for it
+    return b->tuned && b->two[size_t(q)] && two_step_eligible(b, q) ? kModeTwoStep : kModeCell4;
 }
 
 int fdtd_batch_get_grid_ctas(const fdtd_batch* b, int q)
@@ -987,10 +988,12 @@ fdtd_status fdtd_batch_autotune(fdtd_batch* b, int steps, void* scratch, size_t 
         if (fdtd_load_state(g, S + offs[size_t(q)]) != FDTD_OK && err == cudaSuccess) err = cudaErrorUnknown;
     }
     // 2. the whole batch, kBatchGraphSteps steps after a warm-up replay, best
-    //    of two: the graph with the grids of at least `thr` cells on the
-    //    two-step kernel (thr over every eligible grid's size, and none), on
-    //    shares of the SMs or on all of them; the persistent cell engine
-    std::vector<long long> thresholds = {-1};   // -1: no grid on the two-step kernel
+    //    of two: the graph as on an untuned batch; the graph with the grids of
+    //    at least `thr` cells on the two-step kernel (thr over every eligible
+    //    grid's size, and none), on shares of the SMs or on all of them; the
+    //    persistent cell engine
+    constexpr long long kUntuned = -2;
+    std::vector<long long> thresholds = {kUntuned, -1};   // -1: no grid on the two-step kernel
     for (int q = 0; q < n; ++q)
         if (two_step_eligible(b, q)) {
             const fdtd_grid* g = b->grids[size_t(q)];
@@ -998,6 +1001,12 @@ fdtd_status fdtd_batch_autotune(fdtd_batch* b, int steps, void* scratch, size_t 
             if (std::find(thresholds.begin(), thresholds.end(), c) == thresholds.end()) thresholds.push_back(c);
         }
     auto apply = [&](long long thr) {
+        if (thr == kUntuned) {   // as on an untuned batch, the cell passes on the best block height
+            automatic_ctas(b);
+            for (int q = 0; q < n; ++q) b->mode[size_t(q)] = b->two[size_t(q)] ? kModeAuto : cell_mode[size_t(q)];
+            drop_graphs(b);
+            return;
+        }
         for (int q = 0; q < n; ++q) {
             const fdtd_grid* g = b->grids[size_t(q)];
             const long long c = (long long)g->desc.nx * g->desc.ny * g->desc.nz;
@@ -1021,17 +1030,17 @@ fdtd_status fdtd_batch_autotune(fdtd_batch* b, int steps, void* scratch, size_t 
         return st == FDTD_OK;
     };
     const int keep_engine = b->engine;
-    b->automatic = false;
+    const std::vector<int> keep_mode = b->mode;
     float best_t = 1e30f;
-    long long best_thr = -1;
+    long long best_thr = kUntuned;
     bool best_shared = true;
     int best_engine = FDTD_BATCH_CELL;
     b->engine = FDTD_BATCH_CELL;
     for (long long thr : thresholds) {
         for (int sh = 0; sh < 2 && err == cudaSuccess; ++sh) {
-            if (thr < 0 && sh == 1) break;   // no two-step grid: the shares do not matter
+            if (thr < 0 && sh == 1) break;   // one work split only
+            if (thr != kUntuned) two_step_ctas(b, sh == 0);
             apply(thr);
-            two_step_ctas(b, sh == 0);
             float t = 0.0f;
             if (!time_batch(&t)) { err = cudaErrorUnknown; break; }
             if (t < best_t) { best_t = t; best_thr = thr; best_shared = sh == 0; best_engine = FDTD_BATCH_CELL; }
@@ -1048,11 +1057,14 @@ fdtd_status fdtd_batch_autotune(fdtd_batch* b, int steps, void* scratch, size_t 
     cudaEventDestroy(e1);
     if (err == cudaSuccess) {
         b->engine = best_engine;
+        if (best_thr != kUntuned) two_step_ctas(b, best_shared);
         apply(best_thr);
-        two_step_ctas(b, best_shared);
+        b->tuned = true;
     } else {
         b->engine = keep_engine;
-        apply(-1);
+        automatic_ctas(b);
+        b->mode = keep_mode;
+        drop_graphs(b);
     }
     const fdtd_status rst = load_all();
     if (err != cudaSuccess) return st != FDTD_OK ? st : fail(FDTD_ECUDA, "batch autotune failed: %s", fdtd_last_error());

@@ -434,7 +434,9 @@ cudaError_t launch_tb2_table(const fdtd_grid* cg, int cur, const StepTime<float>
     if (e != cudaSuccess) return e;
     const int all = std::min(kTb2MaxCtas, (g->sm_count > 0 ? g->sm_count : 152) * per_sm);
     const int slots = std::max(1, std::min(all, max_ctas));
-    TileConfig tc = g->tile;
+    // an automatic launch has the default tile's work split, whatever tile the
+    // grid's own steps take
+    const TileConfig tc = automatic ? default_tile(g->desc, g->sm_count) : g->tile;
     Tb2Plan plan;
     tb2_plan(g, RY, slots, tc, plan);
     TmaMaps* m = nullptr;

@@ -57,3 +57,63 @@ def test_whole_windows_first_changes_no_result(shape, npml):
     for other in runs[1:]:
         for x, y in zip(runs[0], other):
             assert torch.isfinite(x).all() and torch.equal(x, y)
+
+
+def _batch(shapes, walls=False):
+    gs = []
+    for nx, ny, nz in shapes:
+        g = fdtd.Grid(fdtd.make_grid_desc(nx, ny, nz, 6, 0.05, 0.05, 0.05, z_walls=walls))
+        if walls:
+            g.set_wall_source(theta=0.4, w0=0.7, ramp=0.2, plane=1)
+        else:
+            g.set_source(theta=0.35, r_center=min(nx, ny) / 2 - 10, ramp=0.2)
+        gs.append(g)
+    return gs, fdtd.Batch(gs)
+
+
+@pytest.mark.parametrize("walls", [False, True])
+def test_tuned_batch_is_no_slower_than_an_untuned_one(walls):
+    """Uneven grids on which the untuned batch's split of the SMs or, with
+    walls, its two-step kernel beats the modes that can be chosen (1.1 to 1.5
+    times): within 8 % of the untuned time after tuning."""
+    shapes = [(420, 400, 40), (420, 400, 40), (160, 150, 40), (96, 90, 40)] if not walls else [(200, 200, 60)] * 3
+    times = []
+    for tune in (False, True):
+        gs, b = _batch(shapes, walls)
+        if tune:
+            b.autotune(steps=4)
+        b.step(64)
+        b.sync()
+        e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        best = 1e9
+        for _ in range(5):
+            e[0].record(gs[0].stream)
+            b.step(64)
+            e[1].record(gs[0].stream)
+            b.sync()
+            best = min(best, e[0].elapsed_time(e[1]))
+        times.append(best)
+        b.close()
+    assert times[1] <= 1.08 * times[0], times
+
+
+def test_a_mode_chosen_for_one_grid_leaves_the_others_alone():
+    """The others keep their route, their shares of the SMs and the bits of the cell passes."""
+    shapes = [(160, 150, 24), (140, 150, 24), (150, 140, 24)]
+    ref, alone = _batch(shapes)
+    alone.close()
+    gs, b = _batch(shapes)
+    ctas, routes = fdtd.batch_routes([g.desc for g in gs])
+    assert routes.tolist() == [1, 1, 1]
+    b.set_grid_mode(1, fdtd.BATCH_MODE_CELL8)
+    assert [b.grid_mode(q) for q in range(3)] == [0, 1, 0]
+    assert [b.grid_ctas(q) for q in range(3)] == ctas.tolist()
+    b.step(70)
+    b.sync()
+    for g, x in zip(ref, gs):
+        g.set_tile(5, 4, 1)
+        g.step(70)
+        for c in range(6):
+            assert torch.equal(g.field(c), x.field(c)), c
+        assert torch.equal(g.fluence(), x.fluence())
+    b.close()
