@@ -488,7 +488,7 @@ def full_length_error(torch, make, steps, tile32, balance32):
 def run_batched(torch, fdtd, W, dev, steps):
     """The 16-configuration sweep (l in 0..3 x theta in 5, 10, 20, 30 deg,
     N^2 x 64 grids with N = 96 .. 640), all grids advanced together: the
-    graph engine with every grid on the cell passes (its default), the
+    graph engine as it is untuned and with every grid on the cell passes, the
     persistent cell engine (one cooperative launch per 64 steps), and the
     batch as fdtd_batch_autotune leaves it (each grid's mode, then the
     engine).  Against the same grids stepped one grid at a time, with the
@@ -526,9 +526,12 @@ def run_batched(torch, fdtd, W, dev, steps):
             g.close()
         return ms
 
-    def batched(engine=None, tune=False):
+    def batched(engine=None, tune=False, mode=None):
         bat = [make(wl) for wl in ws_]
         b = fdtd.Batch(bat, engine=engine)
+        if mode is not None:
+            for q in range(len(bat)):
+                b.set_grid_mode(q, mode)
         tuned = b.autotune(steps=8) if tune else None
         if tune:
             tuned = (*tuned, [b.grid_ctas(q) for q in range(len(bat))])
@@ -546,17 +549,18 @@ def run_batched(torch, fdtd, W, dev, steps):
         return ms, tuned
 
     ms_seq = sequential([None] * len(ws_))
-    ms_cell, _ = batched(fdtd.BATCH_CELL)
+    ms_untuned, _ = batched(fdtd.BATCH_CELL)
+    ms_cell, _ = batched(fdtd.BATCH_CELL, mode=fdtd.BATCH_MODE_CELL4)
     ms_pc, _ = batched(fdtd.BATCH_PERSISTENT_CELL)
     ms_tuned, (engine, modes, ctas) = batched(tune=True)
-    mode_tile = {0: (5, 4, 1), 1: (5, 8, 1), 2: (5, 16, 1), 3: (7, 16, 1)}
+    mode_tile = {0: (5, 4, 1), 1: (5, 8, 1), 2: (5, 16, 1), 3: (7, 16, 3)}
     ms_seq_tuned = sequential([mode_tile[m] for m in modes])
     rate = lambda ms: round(cells * steps / (ms * 1e-3) / 1e9, 3)
     return {"value": rate(ms_tuned), "unit": UNIT, "engine": "graph" if engine == fdtd.BATCH_CELL else "persistent_cell",
             "grid_modes": {wl.name: ["cell4", "cell8", "cell16", "two_step"][m] for wl, m in zip(ws_, modes)},
             "two_step_ctas": {wl.name: c for wl, m, c in zip(ws_, modes, ctas) if m == 3},
             "tuned_by": "fdtd_batch_autotune (each grid's mode alone, then the engine over the batch)",
-            "cell_value": rate(ms_cell), "persistent_cell_value": rate(ms_pc),
+            "untuned_value": rate(ms_untuned), "cell_value": rate(ms_cell), "persistent_cell_value": rate(ms_pc),
             "sequential_value": rate(ms_seq), "sequential_tuned_tiles_value": rate(ms_seq_tuned),
             "speedup_vs_sequential": round(ms_seq / ms_tuned, 3),
             "speedup_vs_sequential_same_kernels": round(ms_seq_tuned / ms_tuned, 3),
@@ -566,7 +570,7 @@ def run_batched(torch, fdtd, W, dev, steps):
 
 def run_bessel_gauss(torch, fdtd, W, dev, steps, peak):
     """Section 2's Bessel-Gauss box (411 x 411 x 738 cells with the CPML, z
-    walls, the Gaussian-axicon E_x sheet), FP32 on the cell passes: `steps`
+    walls, the Gaussian-axicon E_x sheet), FP32 on the default tile: `steps`
     of its 3635 steps timed with CUDA events (the fields and fluence, 7.6 GB,
     exceed L2), then the same number with events around each kernel."""
     w = W.bessel_gauss()
@@ -583,10 +587,12 @@ def run_bessel_gauss(torch, fdtd, W, dev, steps, peak):
     e1.record(g.stream)
     torch.cuda.synchronize(dev)
     ms = e0.elapsed_time(e1)
-    pass_ms = g.step_timed(steps)
-    rows, dom = kernel_roofline(w, g.tile(), pass_ms, steps, 4, peak, w.cells)
-    for r in rows:   # z-walled grids run the *_w instantiations of the cell passes
-        r["kernel"] += "_w"
+    timed = max(2, steps // 2 * 2)
+    pass_ms = g.step_timed(timed)   # one kernel where pairs of steps take the two-step kernel, else two
+    tile = (7, 16, 1) if len(pass_ms) == 1 else g.tile()
+    rows, dom = kernel_roofline(w, tile, pass_ms, timed, 4, peak, w.cells)
+    for r in rows:   # z-walled grids run instantiations of their own
+        r["kernel"] += "_w" if len(pass_ms) > 1 else " (z walls)"
     out = {"workload": w.name, "cells": w.cells, "grid": [w.nx, w.ny, w.nz], "npml": w.npml,
            "npml_z": w.npml_z, "theta_deg": w.theta_deg, "w0_lambda": w.w0, "steps_timed": steps,
            "steps_full_run": w.steps, "value": round(job_rate(w.cells, steps, 1, ms), 3), "unit": UNIT,

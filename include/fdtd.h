@@ -343,10 +343,14 @@ fdtd_status fdtd_debug_per_device(const int* devices, const int* results, int n,
  * fdtd_step and time every kernel launch of a step with CUDA events recorded
  * on the grid's stream.  pass_ms[p] (host array of max_passes floats) gets
  * the total milliseconds of kernel p of a step summed over the steps;
- * *n_passes = kernels per step (1 for variants 0-2; 2 for variants 3-5:
+ * *n_passes = kernels per step (1 for variants 0-2 and 6; 2 for variants 3-5:
  * [0] H pass, [1] E pass with the fluence term, or for variant 4 [0] H pass
- * with the fluence term, [1] E pass).  Synchronizes the stream.  EINVAL if
- * max_passes is smaller than the kernels per step. */
+ * with the fluence term, [1] E pass; 1 for variant 7, whose launches take two
+ * steps: EINVAL for an odd nsteps).  On a default tile whose pairs of steps
+ * take the two-step kernel: [0] its launches, and for an odd nsteps [1] and [2]
+ * the H and E pass of the last step (with max_passes < 3 an odd nsteps runs and
+ * times the cell passes alone, to the same results).  Synchronizes the stream.
+ * EINVAL if max_passes is smaller than the kernels per step. */
 fdtd_status fdtd_step_timed(fdtd_grid* g, int nsteps, float* pass_ms, int max_passes, int* n_passes);
 
 /* Test hook (the paper has no counterpart): fault injection on the host side

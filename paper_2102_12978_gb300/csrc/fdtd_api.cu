@@ -788,6 +788,18 @@ fdtd_status fdtd_clear_source(fdtd_grid* g)
     return FDTD_OK;
 }
 
+// A pair of steps in one launch (tile variant 7 in configuration tc).
+static cudaError_t launch_pair(fdtd_grid* g, const TileConfig& tc)
+{
+    const cudaError_t e = launch_tb2(g, g->cur, g->step, tc, g->stream);
+    if (e != cudaSuccess) return e;
+    g->cur ^= 1;
+    g->pe ^= 1;
+    if (tc.automatic) g->flip ^= 1;
+    g->step += 2;
+    return cudaSuccess;
+}
+
 // Advance the grid by nsteps with tile configuration tc on its stream: pairs
 // of steps as one launch of variant 7, every other step as one launch_step.
 static cudaError_t run_steps(fdtd_grid* g, int nsteps, const TileConfig& tc)
@@ -806,12 +818,8 @@ static cudaError_t run_steps(fdtd_grid* g, int nsteps, const TileConfig& tc)
     if (tc.automatic && two.variant == 7 && stream_captured(g->stream)) paired = nsteps / 4 * 4;
     if (two.variant == 7)
         for (; s < paired; s += 2) {
-            cudaError_t e = launch_tb2(g, g->cur, g->step, two, g->stream);
+            cudaError_t e = launch_pair(g, two);
             if (e != cudaSuccess) return e;
-            g->cur ^= 1;
-            g->pe ^= 1;
-            if (tc.automatic) g->flip ^= 1;
-            g->step += 2;
         }
     const TileConfig one = single_step_tile(tc);
     for (; s < nsteps; ++s) {
@@ -912,59 +920,53 @@ fdtd_status fdtd_step_timed(fdtd_grid* g, int nsteps, float* pass_ms, int max_pa
     const fdtd_status dev_st = check_device(g, "fdtd_step_timed");
     if (dev_st != FDTD_OK) return dev_st;
     if (g->batch_refs > 0) return not_batched(g, "fdtd_step_timed");
-    if (g->tile.variant == 7) {
-        // one kernel per two steps: pass_ms[0] sums the launches
-        if (nsteps % 2) return fail(FDTD_EINVAL, "variant 7 times an even number of steps (%d)", nsteps);
-        const int nl = nsteps / 2;
-        std::vector<cudaEvent_t> ev(size_t(nl) + 1, nullptr);
-        fdtd_status st = FDTD_OK;
-        for (auto& e : ev)
-            if (st == FDTD_OK) st = cuda_check(cudaEventCreate(&e), "event create");
-        if (st == FDTD_OK) cudaEventRecord(ev[0], g->stream);
-        for (int l = 0; l < nl && st == FDTD_OK; ++l) {
-            st = cuda_check(launch_tb2(g, g->cur, g->step, g->tile, g->stream), "step launch");
-            cudaEventRecord(ev[size_t(l) + 1], g->stream);
-            if (st == FDTD_OK) { g->cur ^= 1; g->pe ^= 1; g->step += 2; }
-        }
-        if (st == FDTD_OK) st = cuda_check(cudaEventSynchronize(ev.back()), "event synchronize");
-        pass_ms[0] = 0.0f;
-        for (int l = 0; l < nl && st == FDTD_OK; ++l) {
-            float ms = 0.0f;
-            st = cuda_check(cudaEventElapsedTime(&ms, ev[size_t(l)], ev[size_t(l) + 1]), "event elapsed time");
-            pass_ms[0] += ms;
-        }
-        for (auto& e : ev)
-            if (e) cudaEventDestroy(e);
-        *n_passes = 1;
-        if (st != FDTD_OK) return st;
-        return fdtd_sync(g);
+    // the kernels fdtd_step takes: two-step launches for the pairs, then single
+    // steps.  On the default tile an odd count ends with a step of the cell
+    // passes, which takes two entries more; a caller without room for them gets
+    // the cell passes alone (the results are the same).
+    TileConfig two = g->tile;
+    bool pairs = g->tile.variant == 7;
+    if (g->tile.automatic && nsteps >= 2 && (nsteps % 2 == 0 || max_passes >= 3) && default_two_step(g)) {
+        pairs = true;
+        two.variant = 7;
+        two.ty = 16;
     }
-    const int np = passes_per_step(g->tile);
-    if (max_passes < np) return fail(FDTD_EINVAL, "max_passes=%d < %d kernels per step", max_passes, np);
-    std::vector<cudaEvent_t> ev(size_t(nsteps) * (np + 1), nullptr);
+    if (g->tile.variant == 7 && nsteps % 2)
+        return fail(FDTD_EINVAL, "variant 7 times an even number of steps (%d)", nsteps);
+    const int nl = pairs ? nsteps / 2 : 0, ns = nsteps - 2 * nl;   // launches of pairs, single steps
+    const int np = ns > 0 ? passes_per_step(g->tile) : 0, first = nl > 0 ? 1 : 0;
+    if (max_passes < first + np) return fail(FDTD_EINVAL, "max_passes=%d < %d kernels per step", max_passes, first + np);
+    std::vector<cudaEvent_t> ev(size_t(nl) + 1 + size_t(ns) * (np + 1), nullptr);
     fdtd_status st = FDTD_OK;
     for (auto& e : ev)
         if (st == FDTD_OK) st = cuda_check(cudaEventCreate(&e), "event create");
-    for (int s = 0; s < nsteps && st == FDTD_OK; ++s) {
-        cudaEvent_t* e = &ev[size_t(s) * (np + 1)];
+    cudaEvent_t* const single = ev.data() + nl + 1;
+    if (st == FDTD_OK) cudaEventRecord(ev[0], g->stream);
+    for (int l = 0; l < nl && st == FDTD_OK; ++l) {
+        st = cuda_check(launch_pair(g, two), "step launch");
+        cudaEventRecord(ev[size_t(l) + 1], g->stream);
+    }
+    for (int s = 0; s < ns && st == FDTD_OK; ++s) {
+        cudaEvent_t* e = single + size_t(s) * (np + 1);
         cudaEventRecord(e[0], g->stream);
         st = cuda_check(launch_step(g, g->cur, g->step, g->tile, g->stream, np == 2 ? e[1] : nullptr), "step launch");
         g->fault = 0;
         cudaEventRecord(e[np], g->stream);
         if (st == FDTD_OK) { g->cur ^= 1; g->step += 1; }
     }
-    if (st == FDTD_OK) st = cuda_check(cudaEventSynchronize(ev.back()), "event synchronize");
-    for (int p = 0; p < np; ++p) pass_ms[p] = 0.0f;
-    for (int s = 0; s < nsteps && st == FDTD_OK; ++s)
-        for (int p = 0; p < np; ++p) {
-            float ms = 0.0f;
-            st = cuda_check(cudaEventElapsedTime(&ms, ev[size_t(s) * (np + 1) + p], ev[size_t(s) * (np + 1) + p + 1]),
-                            "event elapsed time");
-            pass_ms[p] += ms;
-        }
+    if (st == FDTD_OK) st = cuda_check(cudaEventSynchronize(ns > 0 ? ev.back() : ev[size_t(nl)]), "event synchronize");
+    for (int p = 0; p < first + np; ++p) pass_ms[p] = 0.0f;
+    auto add = [&](int p, cudaEvent_t from, cudaEvent_t to) {
+        float ms = 0.0f;
+        if (st == FDTD_OK) st = cuda_check(cudaEventElapsedTime(&ms, from, to), "event elapsed time");
+        pass_ms[p] += ms;
+    };
+    for (int l = 0; l < nl; ++l) add(0, ev[size_t(l)], ev[size_t(l) + 1]);
+    for (int s = 0; s < ns; ++s)
+        for (int p = 0; p < np; ++p) add(first + p, single[size_t(s) * (np + 1) + p], single[size_t(s) * (np + 1) + p + 1]);
     for (auto& e : ev)
         if (e) cudaEventDestroy(e);
-    *n_passes = np;
+    *n_passes = first + np;
     if (st != FDTD_OK) return st;
     return fdtd_sync(g);
 }
