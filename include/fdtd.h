@@ -256,7 +256,7 @@ int64_t fdtd_antenna_points(const fdtd_grid* g, int component);
  *      that x-neighbouring windows march side by side, lz 3 gives every CTA
  *      whole windows first, any other lz takes the windows row by row):
  *      windows of 32 x 24 columns (ty 16; 32 x 12
- *      with ty 8) march along z, recomputing their halo columns, so that
+ *      with ty 8, and with ty 16 on the smallest boxes) march along z, recomputing their halo columns, so that
  *      fields, psi and the fluence cross HBM once per two steps.  An odd
  *      step count ends with one step of variant 5.  The CTAs' shares of the work are balanced on
  *      per-window costs (fdtd_set_balance).

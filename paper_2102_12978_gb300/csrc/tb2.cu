@@ -13,8 +13,24 @@
 
 namespace fdtd {
 
-// Window rows of the kernel that serves tile height ty.
-static int tb2_rows(int ty) { return ty == 8 ? kTb2RowsSmall : kTb2Rows; }
+// Window rows of the kernel that serves tile height ty on a box: ty 16 takes
+// the small windows too where the large ones hold so few planes per SM that a
+// launch is the latency of a handful of planes, which a plane of six warps has
+// less of than one of twelve.  The small windows' kernel has the fluence terms
+// always, so that without a fluence the line lies lower.  us per step, 24 rows /
+// 12 rows, and (window, plane) items per SM: 48 x 40 x 16 8.2 / 6.3 (0.4), 64 x 48 x
+// 12 8.2 / 7.2 (0.7), 40 x 40 x 32 8.2 / 7.2 (0.8), 64 x 64 x 32 9.8 / 9.3 (2.5), 80 x 80 x
+// 40 11.3 / 13.3 (4.2), 40 x 40 x 160 11.9 / 13.1 (4.2); without a fluence 48 x 40 x 16 7.2 /
+// 6.4, 64 x 48 x 12 7.2 / 7.2, 80 x 80 x 16 8.2 / 9.3 (1.7), 64 x 64 x 32 8.2 / 9.3.
+constexpr double kFewItems = 2.6, kFewItemsNoFlu = 0.7;
+static int tb2_rows(const fdtd_grid* g, int ty)
+{
+    if (ty == 8) return kTb2RowsSmall;
+    int t, u;
+    tb2_windows(g->desc, kTb2Rows, &t, &u);
+    const double items = double(t) * u * g->desc.nz / (g->sm_count > 0 ? g->sm_count : 152);
+    return items <= (g->desc.fluence ? kFewItems : kFewItemsNoFlu) ? kTb2RowsSmall : kTb2Rows;
+}
 
 void tb2_windows(const fdtd_grid_desc& d, int ry, int* t, int* u)
 {
@@ -68,7 +84,7 @@ std::vector<long long> tb2_refined_ranges(const std::vector<long long>& s, const
 
 void tb2_refine(fdtd_grid* g, int ty, int slots, const unsigned long long* cycles, double step)
 {
-    const int ry = tb2_rows(ty);
+    const int ry = tb2_rows(g, ty);
     // the ranges the measured launches ran: the cached plan of this shape
     if (g->tb2_key.ry != ry || g->tb2_key.slots != slots || g->tb2_start.size() != size_t(slots) + 1) return;
     g->tb2_refined = tb2_refined_ranges(g->tb2_start, cycles, step);
@@ -344,8 +360,9 @@ bool default_two_step(const fdtd_grid* g)
 int tb2_slots(const fdtd_grid* g, int ty)
 {
     int per_sm = 0;
-    const cudaError_t e = ty == 8 ? tb2_blocks_per_sm<kTb2RowsSmall>(g->device, &per_sm)
-                                   : tb2_blocks_per_sm<kTb2Rows>(g->device, &per_sm);
+    const cudaError_t e = tb2_rows(g, ty) == kTb2RowsSmall
+                              ? tb2_blocks_per_sm<kTb2RowsSmall>(g->device, &per_sm)
+                              : tb2_blocks_per_sm<kTb2Rows>(g->device, &per_sm);
     if (e != cudaSuccess) return -1;
     return std::min(kTb2MaxCtas, (g->sm_count > 0 ? g->sm_count : 152) * per_sm);
 }
@@ -418,7 +435,7 @@ static cudaError_t launch_tb2_t(const fdtd_grid* cg, int cur, long long n, const
 cudaError_t launch_tb2(const fdtd_grid* g, int cur, long long n, const TileConfig& tc, cudaStream_t s)
 {
     if (g->desc.precision != FDTD_F32 || (has_walls(g) && !tc.automatic)) return cudaErrorInvalidValue;
-    if (tc.ty == 8) return launch_tb2_t<kTb2RowsSmall>(g, cur, n, tc, s);
+    if (!tc.automatic && tb2_rows(g, tc.ty) == kTb2RowsSmall) return launch_tb2_t<kTb2RowsSmall>(g, cur, n, tc, s);
     return launch_tb2_t<kTb2Rows>(g, cur, n, tc, s);
 }
 

@@ -1,0 +1,30 @@
+"""The explicit two-step tile on small boxes: the window height the box is given
+and the ranges kept after measuring change no result."""
+import pytest
+import torch
+
+from paper_2102_12978_gb300 import workloads as W
+from tests.gpu_cases import gpu_grid
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("fluence", [True, False])
+@pytest.mark.parametrize("shape,npml", [((48, 40, 16), 6), ((64, 64, 32), 8), ((64, 64, 33), 8), ((40, 40, 5), 4),
+                                        ((25, 21, 1), 3), ((80, 80, 16), 8), ((60, 47, 19), 6)])
+def test_tile_heights_agree(shape, npml, fluence):
+    """ty 16 against ty 8 on both sides of the line between the window heights."""
+    nx, ny, nz = shape
+    w = W.small(nx=nx, ny=ny, nz=nz, npml=npml, r_center=min(nx, ny) / 2 - npml - 3, ramp=0.3)
+    out = []
+    for tile, measure in (((7, 8, 1), False), ((7, 16, 1), False), ((7, 16, 2), True), ((7, 8, 2), True), ((7, 16, 3), False)):
+        g = gpu_grid(w, "f32", fluence=fluence, tile=tile)
+        g.step(6)
+        if measure:
+            g.measure_balance()
+            assert g.balance() == (-1.0, -1.0)
+        g.step(7)
+        out.append([g.field(c) for c in range(6)] + ([g.fluence()] if fluence else []))
+    for other in out[1:]:
+        for x, y in zip(out[0], other):
+            assert torch.isfinite(x).all() and torch.equal(x, y)
