@@ -296,7 +296,8 @@ fdtd_status fdtd_get_balance(const fdtd_grid* g, float* w_shell, float* w_antenn
  * times (the paper has no counterpart): in four rounds, three launches record
  * the SM cycles every CTA takes, and the ranges' boundaries move toward equal
  * shares of the measured time (all the way in the first round, three
- * quarters of the way after it).  The 24 steps run from a copy of the state
+ * quarters of the way after it); where that made the slowest CTA slower, the
+ * best ranges measured are kept.  The 24 steps run from a copy of the state
  * and are undone (the state is saved to
  * `scratch_state`, fdtd_state_bytes bytes of device memory the caller owns,
  * and restored).  The refined ranges are used from then on (fdtd_autotune
