@@ -141,7 +141,13 @@ static int tb2_window_host(int T, int U, int D, int pos)
 // the weights or the launch shape change.
 // Measured on GB300 (cycles per plane, 256 x 256 x 128 cells): inner windows
 // 2400, with antenna columns 2750, x shell 3340, y shell 3380, both 4720; the
-// default weights 0.4 and 0.2 follow (0.15 is slower by up to 2 %).
+// default weights 0.4 and 0.2 follow (0.15 is slower by up to 2 %).  A z-shell
+// plane takes about 2.3 inner ones (411 x 411 x 192: 448 us per step with 4 cells of
+// z CPML, 508 with 16), and a launch 15 to 55 us more for having any, whatever
+// their number.  The split does best with less weight than that: us per step at
+// kZPlane 1.6 / 2.2 / 3 / 4, 411 x 411 x 192 with 16 cells 508 / 519 / 520 / 521, 340 x
+// 340 x 192 417 / 423 / 426 / 431, 205 x 205 x 400 with 8 417 / 429 / 438 / 456, 332 x 332 x 40
+// with 1 91 / 82 / 82 / 81.
 constexpr double kRestart = 5.3;
 constexpr double kCorner = 0.4;
 constexpr double kZPlane = 1.6;

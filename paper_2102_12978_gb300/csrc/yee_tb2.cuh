@@ -48,9 +48,10 @@
 //     memory when the window starts; the per-plane phase e^{i beta z_k} is
 //     loaded one plane ahead.
 //   * The fluence of cell (i, j, k) needs E and H at i+1, j+1, k+1; a
-//     window's fluence cells are its E^{n+2} cells shifted by -1 in x, y and
-//     z (plus the last cell before the far wall), so that the H^{n+3/2} they
-//     need lie inside the window.  Both terms of a cell (steps n and n+1) are
+//     window's fluence cells are its own columns, their rows and planes
+//     shifted by -1 (plus the last row before the far wall; on z-walled grids
+//     the last plane too), so that the H^{n+3/2} they need lie inside the
+//     window.  Both terms of a cell (steps n and n+1) are
 //     added, Kahan-compensated, in one read-modify-write.
 //   * Reading step n from one copy of the fields and psi and writing step
 //     n+2 into the other (ping-pong, E-side psi included) makes the halo
@@ -64,9 +65,9 @@
 //     the x (y) walls, psi and columns past the box (template flags GX, GY).
 //     A plane of an inner window takes 2400 cycles, of an x- or y-shell window
 //     3400, of a corner 4700.
-//   * On the default tile a CTA takes whole windows first, so that
-//     neighbouring windows march together and share halo planes in L2, then a
-//     range of what is left (tb2_plan).  On explicit tiles it takes
+//   * On the default tile (and with lz 3) a CTA takes whole windows first, so
+//     that neighbouring windows march together and share halo planes in L2,
+//     then a range of what is left (tb2_plan).  On other tiles it takes
 //     a contiguous range of the flattened (window, plane) work:
 //     ranges of equal estimated cost (windows with CPML shell or antenna
 //     columns weigh more, with weights the autotuner picks by timing), or
