@@ -210,7 +210,8 @@ fdtd_status fdtd_wall_coefficients(const fdtd_grid_desc* d, const fdtd_wall_desc
  * Small grids, whose passes take a few microseconds, are bound by the cost
  * of those launches; a batch of one grid (fdtd_batch_create with n = 1)
  * replays 64 steps from one CUDA graph instead, with the same results
- * (64 x 64 x 32 cells on GB300: 10.3 us per step alone, 6.0 in a batch). */
+ * (64 x 64 x 32 cells on GB300: 10.3 us per step alone, 5.4 to 5.9 in a
+ * batch). */
 fdtd_status fdtd_step(fdtd_grid* g, int nsteps);
 
 /* Copy the fluence (nz*ny*nx doubles, x fastest, dense) to dst (device if
@@ -258,11 +259,12 @@ int64_t fdtd_antenna_points(const fdtd_grid* g, int component);
  *      windows of 32 x 24 columns (ty 16; 32 x 12
  *      with ty 8, and with ty 16 on the smallest boxes) march along z, recomputing their halo columns, so that
  *      fields, psi and the fluence cross HBM once per two steps.  An odd
- *      step count ends with one step of variant 5.  The CTAs' shares of the work are balanced on
- *      per-window costs (fdtd_set_balance).
+ *      step count ends with one step of variant 5.  The CTAs' shares of the
+ *      work are balanced on per-window costs (fdtd_set_balance).
  * The TMA variants (1, 2, 4) have no FP64 32x16 tile (EINVAL).  A z-walled
  * grid or one with a wall source takes variant 5 only (EINVAL otherwise;
- * fdtd_autotune then times the ty of variant 5 and the default tile).
+ * fdtd_autotune then times the ty of variant 5 and the default tile, and
+ * may return the grid to that).
  * fdtd_create_grid picks a default (variant 5, ty 4).  As long as no tile is
  * chosen, an FP32 grid takes its pairs of steps with the two-step kernel
  * instead where that is estimated to be faster (the time depends on the box:
@@ -274,7 +276,8 @@ int64_t fdtd_antenna_points(const fdtd_grid* g, int component);
  * (running `steps` steps for each, then restoring the state) and keeps the
  * fastest; the two-step kernel with the default tile's work split is one
  * (variant 7, lz 3; with z walls or a wall source the default tile itself,
- * which fdtd_get_tile names as variant 5, ty 4).  Results agree to rounding for every configuration. */
+ * which fdtd_get_tile names as variant 5, ty 4).  Results agree to rounding
+ * for every configuration. */
 fdtd_status fdtd_set_tile(fdtd_grid* g, int variant, int ty, int lz);
 
 /* Work-split weights of tile variant 7 (the paper has no counterpart): a
@@ -394,9 +397,9 @@ void fdtd_destroy_grid(fdtd_grid* g);
  *     tile variant 5 on 32 x 4, 32 x 8 or 32 x 16 blocks (the arithmetic of
  *     variant 5, bit for bit), or, for FP32 z-periodic grids without a wall
  *     source, the two-step kernel of tile variant 7 on a share of the SMs
- *     proportional to the grid's cells (the arithmetic of variant 7, bit for
- *     bit).  Steps that do not fill a replay run one by one with the cell
- *     passes.
+ *     (the arithmetic of variant 7, bit for bit).  Steps that do not fill a
+ *     replay run with the cell passes; while no mode is chosen for a grid, as
+ *     on its default tile.
  *   FDTD_BATCH_PERSISTENT_CELL: one cooperative kernel launch per 64 steps
  *     and per group of up to 24 grids (no graph): every CTA stays resident
  *     and takes runs of cell blocks of all grids in order from a counter,

@@ -447,8 +447,8 @@ class Grid:
         return ws.value, wa.value
 
     def measure_balance(self):
-        """Balance the variant-7 ranges on per-window costs measured in one
-        launch (fdtd_measure_balance; the state is saved and restored)."""
+        """Balance the variant-7 ranges on the CTAs' measured times
+        (fdtd_measure_balance; the state is saved and restored)."""
         scratch = self.torch.empty(self.state_bytes(), dtype=self.torch.uint8, device=self.device)
         check(lib().fdtd_measure_balance(C.c_void_p(self.handle), C.c_void_p(scratch.data_ptr())),
               "fdtd_measure_balance")
@@ -531,9 +531,9 @@ class Batch:
     """Several Grid objects advanced together (fdtd_batch_*): engine
     BATCH_CELL (a 64-step CUDA graph with one branch per grid, each grid in
     its own mode: cell passes on 32 x 4 / 8 / 16 blocks or the two-step
-    kernel; until a mode is chosen, whichever the grid's default tile takes;
-    the default) or BATCH_PERSISTENT_CELL (one cooperative launch
-    per 64 steps)."""
+    kernel; until a mode is chosen for it, whichever is estimated to be the
+    faster; the default) or BATCH_PERSISTENT_CELL (one cooperative launch per
+    64 steps)."""
 
     def __init__(self, grids, engine: int | None = None):
         import torch
