@@ -157,6 +157,7 @@ struct fdtd_grid {
     std::vector<uint8_t> hmask; // antenna component mask per (i, j) column (host copy), empty without a source
     int src_gen;                // bumped whenever the antenna's columns (hmask) change
     int ant_cols[2];            // antenna columns with H points, with E points (lists at L.alist)
+    int ant_warps;              // warps of 32 columns of a row that hold antenna points
     bool ant_apart;             // the FP64 cell passes may add the source in antenna_add (no antenna
                                 // column on the i = 0 or j = 0 wall, where the E pass zeroes after it)
     std::vector<long long> tb2_start;   // variant 7: cached CTA work ranges

@@ -112,12 +112,16 @@ static cudaError_t launch_step_cell(const fdtd_grid* g, int cur, long long n, cu
 }
 
 // FP64 grids with an antenna (z-periodic, no wall sheet) add its source in
-// antenna_add after each pass instead of inside it, from kApartCells cells on.
-// Below, two launches more per step (6 us each with the gap) cost more than the
-// FP64 pipe saves (us per step, apart / inside: 48 x 40 x 16 28 / 16.5, 64 x 64 x
-// 32 37 / 29, 96 x 96 x 64 94.6 / 93.2, 128 x 128 x 64 147.5 / 150.1, 256 x 256
-// x 128 927 / 980).
-constexpr double kApartCells = 8e5;
+// antenna_add after each pass instead of inside it, from kApartWarps warps with
+// antenna columns (per plane, times planes) on: inside, each such warp costs the
+// FP64 pipe some 13 instructions per pass, apart, a step has two launches more
+// (6 us each with the gap).  100 boxes and rings measured both ways, 74000 to
+// 2.9 M cells: at most 1.6 % from the better side of this line, 11 % with a line at
+// 8e5 cells.  us per step, apart / inside, and warps x planes: 96 x 96 x 16 37 / 29
+// (1024), 600 x 600 x 3 145 / 139 (3609), 160 x 160 x 16 68.7 / 65.0 (4544), 96 x 96 x 64
+// 95.0 / 95.5 (7296), 128 x 96 x 64 114 / 118 (10112), 64 x 64 x 160 105 / 114 (14080), 50 x
+// 50 x 300 147 / 164 (19500), 128 x 128 x 96 205 / 224 (21216).
+constexpr long long kApartWarps = 8000;
 template <typename real>
 static cudaError_t antenna_pass(const fdtd_grid* g, const StepArgs<real>& a, int side, Cpx<real> t, cudaStream_t s)
 {
@@ -149,7 +153,7 @@ static cudaError_t launch_cell(const fdtd_grid* g, int cur, long long n, cudaStr
     dim3 block(32, TY);
     const bool wall = has_walls(g);   // z walls or a wall sheet: the *_w kernels
     const bool apart = sizeof(real) == 8 && g->has_source && g->ant_apart && !wall &&
-                       double(g->desc.nx) * g->desc.ny * nz >= kApartCells;
+                       (long long)g->ant_warps * nz >= kApartWarps;
     const StepArgs<real> full = make_args<real>(g, cur);
     StepArgs<real> a = full;
     if (apart) a.smask = nullptr;   // the passes run without the antenna
