@@ -680,13 +680,7 @@ fdtd_status fdtd_set_annulus_source(fdtd_grid* g, const fdtd_annulus_desc* s)
     g->ant_cols[0] = ncol_h;
     g->ant_cols[1] = int(alist.size()) - ncol_h;
     g->ant_apart = !on_wall;
-    g->ant_warps = 0;
-    for (int j = 0; j < d.ny; ++j)
-        for (int i = 0, last = -1; i < d.nx; ++i)
-            if ((mask[size_t(j) * d.nx + i] & 0x3f) && i / 32 != last) {
-                last = i / 32;
-                ++g->ant_warps;
-            }
+    g->ant_warps = antenna_warps(mask, d.nx, d.ny);
     g->has_source = true;
     if (mask != g->hmask) g->src_gen += 1;   // the antenna's columns changed
     g->hmask = mask;

@@ -231,6 +231,10 @@ inline TileConfig single_step_tile(const TileConfig& tc)
     one.variant = 5; one.tx = 32; one.ty = 4; one.lz = tc.lz;
     return one;
 }
+// Warps of 32 columns of a row that hold antenna points of any component.
+// (Apart from fdtd_set_annulus_source: inlined there, the loop changed how the
+// compiler fuses the products with the weights on Arm, and so the tables' last bits.)
+int antenna_warps(const std::vector<uint8_t>& mask, int nx, int ny);
 // The cell-parallel and two-pass steps on stream s: variant 3 yee_h_pass then
 // yee_e_pass (with the fluence term); variant 4 yee_hflu_tma (with the
 // fluence term) then yee_e_pass; variant 5 yee_h_cell then yee_e_cell;

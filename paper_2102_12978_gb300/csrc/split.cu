@@ -122,6 +122,17 @@ static cudaError_t launch_step_cell(const fdtd_grid* g, int cur, long long n, cu
 // 95.0 / 95.5 (7296), 128 x 96 x 64 114 / 118 (10112), 64 x 64 x 160 105 / 114 (14080), 50 x
 // 50 x 300 147 / 164 (19500), 128 x 128 x 96 205 / 224 (21216).
 constexpr long long kApartWarps = 8000;
+int antenna_warps(const std::vector<uint8_t>& mask, int nx, int ny)
+{
+    int n = 0;
+    for (int j = 0; j < ny; ++j)
+        for (int i = 0, last = -1; i < nx; ++i)
+            if ((mask[size_t(j) * nx + i] & 0x3f) && i / 32 != last) {
+                last = i / 32;
+                ++n;
+            }
+    return n;
+}
 template <typename real>
 static cudaError_t antenna_pass(const fdtd_grid* g, const StepArgs<real>& a, int side, Cpx<real> t, cudaStream_t s)
 {
