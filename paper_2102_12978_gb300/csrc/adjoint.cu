@@ -22,6 +22,7 @@
 // g_c(col) = sum over steps and planes of lambda f e^{i (beta z_k - Phi_n)},
 // with lambda = e' (E points) or h' (H points); dL/dw follows per column as
 // Re{e^{i phi} A g} and -w Im{e^{i phi} A g} summed over components.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
@@ -254,8 +255,15 @@ yee_adj_e_cell(const AdjArgs<real> A)
 // the planes, and warp c adds up component c.  384 x 384 x 96 cells, ring 3 cells
 // thick: 23 us per step (one warp per column, lanes over planes, u_c formed per
 // column: 36 us; this form with each load used before the next: 53 us).
+//
+// Tall boxes with few columns would leave most SMs idle and every warp a long
+// run of planes: there a cluster of K CTAs shares the planes of 32 columns,
+// each CTA adds up its own and the first CTA the K sums, from the others'
+// shared memory and in order (adj_grad_ctas).  us per reverse step, FP32, one
+// warp per column / one CTA / K CTAs: 60 x 60 x 300 63.0 / 72.7 / 42.9, 40 x 40 x 2000 321 /
+// 411 / 160, 80 x 87 x 96 37.0 / 39.1 / 33.9, 200 x 200 x 96 101 / 99.5 / 94.3.
 constexpr int kGradWarps = 8, kGradPlanes = 3;
-template <typename real>
+template <typename real, int K>
 __global__ void __launch_bounds__(32 * kGradWarps)
 adj_source_grad(const AdjArgs<real> A, const int* __restrict__ cols, int ncols, double2 te, double2 th)
 {
@@ -264,7 +272,9 @@ adj_source_grad(const AdjArgs<real> A, const int* __restrict__ cols, int ncols, 
     const StepArgs<real>& a = A.f;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nx = a.nx, ny = a.ny, nz = a.nz, plane = a.pitch * ny;
-    const int w = blockIdx.x * 32 + lane;
+    const int rank = K > 1 ? int(blockIdx.x) % K : 0;   // in the cluster
+    constexpr int kStride = kGradWarps * K;             // planes from one load of a warp to the next
+    const int w = int(blockIdx.x) / K * 32 + lane;
     const int col = w < ncols ? cols[w] : 0;
     const int j = col / nx, i = col - j * nx, at = j * a.pitch + i;
     unsigned mk = w < ncols ? a.smask[col] & 0x3fu : 0u;
@@ -274,11 +284,11 @@ adj_source_grad(const AdjArgs<real> A, const int* __restrict__ cols, int ncols, 
     double2 acc[6];
     #pragma unroll
     for (int c = 0; c < 6; ++c) acc[c] = make_double2(0.0, 0.0);
-    for (int k0 = warp; k0 < nz; k0 += kGradPlanes * kGradWarps) {
+    for (int k0 = rank * kGradWarps + warp; k0 < nz; k0 += kGradPlanes * kStride) {
         real r[kGradPlanes][6];   // every load of a few planes in flight at once
         #pragma unroll
         for (int q = 0; q < kGradPlanes; ++q) {
-            const int k = k0 + q * kGradWarps;
+            const int k = k0 + q * kStride;
             #pragma unroll
             for (int c = 0; c < 6; ++c) {
                 const real* f = c < 3 ? A.ein[c] : A.hout[c - 3];
@@ -287,7 +297,7 @@ adj_source_grad(const AdjArgs<real> A, const int* __restrict__ cols, int ncols, 
         }
         #pragma unroll
         for (int q = 0; q < kGradPlanes; ++q) {
-            const int k = k0 + q * kGradWarps;
+            const int k = k0 + q * kStride;
             const double2 z = a.zph[k < nz ? k : 0];
             #pragma unroll
             for (int c = 0; c < 6; ++c) {
@@ -303,17 +313,61 @@ adj_source_grad(const AdjArgs<real> A, const int* __restrict__ cols, int ncols, 
     #pragma unroll
     for (int c = 0; c < 6; ++c) part[c][warp][lane] = acc[c];
     __syncthreads();
-    if (warp < 6 && (mk & (1u << warp))) {
-        double2 s = part[warp][0][lane];
+    double2 s = make_double2(0.0, 0.0);
+    if (warp < 6) {
+        s = part[warp][0][lane];
         for (int q = 1; q < kGradWarps; ++q) {
             s.x += part[warp][q][lane].x;
             s.y += part[warp][q][lane].y;
         }
+    }
+    if constexpr (K > 1) {
+        cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+        if (warp < 6) part[warp][0][lane] = s;
+        cluster.sync();
+        if (rank == 0 && warp < 6)
+            #pragma unroll
+            for (int q = 1; q < K; ++q) {
+                const double2 o = *cluster.map_shared_rank(&part[warp][0][lane], q);
+                s.x += o.x;
+                s.y += o.y;
+            }
+        cluster.sync();   // the first CTA has read the others' sums
+        if (rank != 0) return;
+    }
+    if (warp < 6 && (mk & (1u << warp))) {
         const double2 t = warp < 3 ? te : th;
         double2& g = A.grad[warp * nx * ny + col];
         g.x += s.x * t.x - s.y * t.y;
         g.y += s.x * t.y + s.y * t.x;
     }
+}
+
+// CTAs that share the planes of 32 columns: more as long as they fit the SMs and
+// every warp keeps more than 8 planes.
+int adj_grad_ctas(int blocks, int nz, int sms)
+{
+    int k = 1;
+    while (k < 8 && 2 * k * blocks <= sms && nz > 64 * k) k *= 2;
+    return k;
+}
+
+template <typename real, int K>
+cudaError_t launch_source_grad(const AdjArgs<real>& A, const int* cols, int ncols, double2 te, double2 th,
+                               cudaStream_t s)
+{
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3(unsigned((ncols + 31) / 32 * K));
+    c.blockDim = dim3(32 * kGradWarps);
+    c.dynamicSmemBytes = 6 * kGradWarps * 32 * 16;
+    c.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = K;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    c.attrs = at;
+    c.numAttrs = K > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&c, adj_source_grad<real, K>, A, cols, ncols, te, th);
 }
 
 // dL/dw per column from the accumulated g: sum over components of
@@ -445,8 +499,13 @@ cudaError_t adj_cell_launch(fdtd_adjoint* ad, long long n)
     source_time(g->srct, (double(n) + 0.5) * g->dt, c, sn, f);
     const double2 th = make_double2(f * c, -f * sn);
     const int* cols = reinterpret_cast<const int*>(static_cast<char*>(ad->arena) + ad->acols);
-    adj_source_grad<real><<<(ad->nacols + 31) / 32, 32 * kGradWarps, 6 * kGradWarps * 32 * 16, g->stream>>>(A, cols, ad->nacols, te, th);
-    return cudaGetLastError();
+    const int blocks = (ad->nacols + 31) / 32;
+    switch (adj_grad_ctas(blocks, g->desc.nz, g->sm_count > 0 ? g->sm_count : 152)) {
+        case 8: return launch_source_grad<real, 8>(A, cols, ad->nacols, te, th, g->stream);
+        case 4: return launch_source_grad<real, 4>(A, cols, ad->nacols, te, th, g->stream);
+        case 2: return launch_source_grad<real, 2>(A, cols, ad->nacols, te, th, g->stream);
+        default: return launch_source_grad<real, 1>(A, cols, ad->nacols, te, th, g->stream);
+    }
 }
 
 template <typename real>
