@@ -289,10 +289,10 @@ static cudaError_t tb2_blocks_per_sm(int device, int* out)
 // ---- the route of the default tile
 // Estimated us per step of the two kernels that a pair of steps can take.  The
 // bits are the same, so the default tile takes the one estimated to be faster.
-// The constants were fitted to 703 boxes measured both ways on one GB300 (2 x 2 x 1
+// The constants were fitted to 1123 boxes measured both ways on GB300 (2 x 2 x 1
 // to 2048 x 2048 x 12 and 8 x 8 x 16384 cells, with and without fluence, CPML, z
 // walls, z CPML and sheet): the faster kernel is taken, or one within 3 % of it,
-// for 656 of them, and the others cost 11 % on average.  us per step, two-step /
+// for 1044 of them, and the others cost 11 % on average.  us per step, two-step /
 // cell passes: 2048 x 2048 x 1 224 / 79, x 3 295 / 273, x 12 603 / 1075; 560 x 560 x
 // 2 24.6 / 16.5, x 12 56 / 75; 32 x 32 x 1024 36 / 25, 20 x 20 x 4096 38 / 69; 332 x
 // 332 x 46 62 / 109; 16 x 16 x 64 7.2 / 8.2; z walls, 360 x 360 x 6 34 / 21, 411 x 411
@@ -303,7 +303,7 @@ static cudaError_t tb2_blocks_per_sm(int device, int* out)
 // times the time of a plane.
 constexpr double kRefill = 5.6;                       // planes
 constexpr double kPlane = 1.24, kPlaneNoFlu = 1.0;    // us, an inner window's, with and without the fluence terms
-constexpr double kPlaneWall = 1.4;                    // the wall kernel, which has the fluence terms always
+constexpr double kPlaneWall = 1.43, kPlaneWallNoFlu = 1.6;   // the wall kernel's, which has the terms always
 constexpr double kShellWall = 0.3;                    // as w_shell, for the wall kernel
 constexpr double kOddShell = 0.32;                    // more for an x shell off even columns (4-byte psi accesses)
 constexpr double kZShell = 2.1;                       // a z-shell plane, in planes
@@ -324,7 +324,7 @@ double two_step_us(const fdtd_grid_desc& d, bool sheet, int ctas, bool terms)
     const int npz = zw ? d.npml_z : 0;
     const double nz = d.nz, z = nz + 2.0 * npz * (kZShell - 1.0);
     const double planes = std::max(windows * z, z / nz) + (kRefill + (zw ? 1.0 : 0.0)) * (windows + 1.0);
-    const double plane = wall ? kPlaneWall : (terms ? kPlane : kPlaneNoFlu);
+    const double plane = wall ? (d.fluence ? kPlaneWall : kPlaneWallNoFlu) : (terms ? kPlane : kPlaneNoFlu);
     const double us = 0.5 * cost * planes * plane * (npz == 0 ? 1.0 : (windows < kManyWindows ? kZCodeFew : kZCode));
     return wall ? std::max(us, kWallFloor) : us;
 }
