@@ -313,33 +313,38 @@ adj_source_grad(const AdjArgs<real> A, const int* __restrict__ cols, int ncols, 
     #pragma unroll
     for (int c = 0; c < 6; ++c) part[c][warp][lane] = acc[c];
     __syncthreads();
-    double2 s = make_double2(0.0, 0.0);
-    if (warp < 6) {
-        s = part[warp][0][lane];
+    auto add_up = [&]() {   // component `warp` over the CTA's warps
+        double2 s = part[warp][0][lane];
         for (int q = 1; q < kGradWarps; ++q) {
             s.x += part[warp][q][lane].x;
             s.y += part[warp][q][lane].y;
         }
-    }
-    if constexpr (K > 1) {
+        return s;
+    };
+    auto store = [&](double2 s) {
+        const double2 t = warp < 3 ? te : th;
+        double2& g = A.grad[warp * nx * ny + col];
+        g.x += s.x * t.x - s.y * t.y;
+        g.y += s.x * t.y + s.y * t.x;
+    };
+    const bool mine = warp < 6 && (mk & (1u << warp));
+    if constexpr (K == 1) {
+        if (mine) store(add_up());
+    } else {
         cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
-        if (warp < 6) part[warp][0][lane] = s;
+        if (mine) part[warp][0][lane] = add_up();
         cluster.sync();
-        if (rank == 0 && warp < 6)
+        if (rank == 0 && mine) {
+            double2 s = part[warp][0][lane];
             #pragma unroll
             for (int q = 1; q < K; ++q) {
                 const double2 o = *cluster.map_shared_rank(&part[warp][0][lane], q);
                 s.x += o.x;
                 s.y += o.y;
             }
+            store(s);
+        }
         cluster.sync();   // the first CTA has read the others' sums
-        if (rank != 0) return;
-    }
-    if (warp < 6 && (mk & (1u << warp))) {
-        const double2 t = warp < 3 ? te : th;
-        double2& g = A.grad[warp * nx * ny + col];
-        g.x += s.x * t.x - s.y * t.y;
-        g.y += s.x * t.y + s.y * t.x;
     }
 }
 
@@ -356,17 +361,23 @@ template <typename real, int K>
 cudaError_t launch_source_grad(const AdjArgs<real>& A, const int* cols, int ncols, double2 te, double2 th,
                                cudaStream_t s)
 {
+    const dim3 grid(unsigned((ncols + 31) / 32 * K)), block(32 * kGradWarps);
+    constexpr size_t smem = 6 * kGradWarps * 32 * 16;
+    if constexpr (K == 1) {
+        adj_source_grad<real, 1><<<grid, block, smem, s>>>(A, cols, ncols, te, th);
+        return cudaGetLastError();
+    }
     cudaLaunchConfig_t c = {};
-    c.gridDim = dim3(unsigned((ncols + 31) / 32 * K));
-    c.blockDim = dim3(32 * kGradWarps);
-    c.dynamicSmemBytes = 6 * kGradWarps * 32 * 16;
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
     c.stream = s;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = K;
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     c.attrs = at;
-    c.numAttrs = K > 1 ? 1 : 0;
+    c.numAttrs = 1;
     return cudaLaunchKernelEx(&c, adj_source_grad<real, K>, A, cols, ncols, te, th);
 }
 
