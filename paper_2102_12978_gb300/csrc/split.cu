@@ -3,6 +3,8 @@
 // (TMA-staged H pass with the fluence term, plain-load E pass).
 #include <cuda_runtime.h>
 
+#include <cstring>
+
 #include "grid_impl.h"
 #include "tma_host.h"
 #include "yee_cell.cuh"
@@ -126,11 +128,12 @@ int antenna_warps(const std::vector<uint8_t>& mask, int nx, int ny)
 {
     int n = 0;
     for (int j = 0; j < ny; ++j)
-        for (int i = 0, last = -1; i < nx; ++i)
-            if ((mask[size_t(j) * nx + i] & 0x3f) && i / 32 != last) {
-                last = i / 32;
-                ++n;
-            }
+        for (int i = 0; i < nx; i += 32) {
+            const uint8_t* m = mask.data() + size_t(j) * nx + i;
+            uint64_t w[4] = {};   // the warp's columns, eight at a time
+            std::memcpy(w, m, size_t(nx - i < 32 ? nx - i : 32));
+            n += ((w[0] | w[1] | w[2] | w[3]) & 0x3f3f3f3f3f3f3f3fULL) != 0;
+        }
     return n;
 }
 template <typename real>
