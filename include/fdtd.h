@@ -256,11 +256,11 @@ int64_t fdtd_antenna_points(const fdtd_grid* g, int component);
  *      else EINVAL; lz 2 interleaves the window rows in the CTAs' work so
  *      that x-neighbouring windows march side by side, lz 3 gives every CTA
  *      whole windows first, any other lz takes the windows row by row):
- *      windows of 32 x 24 columns (ty 16; 32 x 12
- *      with ty 8, and with ty 16 on the smallest boxes) march along z, recomputing their halo columns, so that
- *      fields, psi and the fluence cross HBM once per two steps.  An odd
- *      step count ends with one step of variant 5.  The CTAs' shares of the
- *      work are balanced on per-window costs (fdtd_set_balance).
+ *      windows of 32 x 24 columns (ty 16; 32 x 12 with ty 8, and with ty 16
+ *      on the smallest boxes) march along z, recomputing their halo columns,
+ *      so that fields, psi and the fluence cross HBM once per two steps.  An
+ *      odd step count ends with one step of variant 5.  The CTAs' shares of
+ *      the work are balanced on per-window costs (fdtd_set_balance).
  * The TMA variants (1, 2, 4) have no FP64 32x16 tile (EINVAL).  A z-walled
  * grid or one with a wall source takes variant 5 only (EINVAL otherwise;
  * fdtd_autotune then times the ty of variant 5 and the default tile, and
